@@ -20,6 +20,7 @@
 // stride-2 max-pool (read while staging, source stride 2) and the remaining stages on the half
 // grid with dilations 1, 2, 4: conv2 out H2+21, conv3 out H2+14, head out H2 = ceil(rows/2).
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -158,9 +159,188 @@ mb_status simt_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_
     return MB_OK;
 }
 
-// Tensor-core paths (BF16 or FP16): layer 1 on CUDA cores (FP32 arithmetic, 16-bit out); the two
-// 32->64 dilated convs and the head on the tensor cores (fastmemb_tc.cu); activations between
-// layers are 16-bit [slice][y][x][32] of the net's type.
+// Layer 1 of the tensor-core paths: conv 4x4 1 -> 64 from the uint8 slice in FP32, max-out over
+// pairs, rounding to the net's 16-bit type, the 2x2 max-filter, and (ST = 2) its stride: features in
+// the layout that the next conv's bulk copies read, [slice][row][chunk of 8][column][16 B].
+//
+// FP32 FMA issue bounds it (2,048 FLOP per conv pixel). A warp walks down a 64-column strip on its
+// own; a lane holds all 64 conv channels of columns l and l + 32, packed by channel pairs, so a
+// max-out group is one accumulator pair and a pixel's 16-byte chunks are stored whole. The weights
+// are kernel parameters: constant-bank operands, no shared-memory broadcasts beside the FMAs (those
+// took 62 % of the shared-memory pipe and left the FMA pipe at 50 %: 528 us). The inputs sit in shared
+// memory duplicated, ready for packed FMAs. Tap order and rounding are those of fm_conv, so the
+// features are bitwise the same. 354 us on 1024 x 1024 x 8 (50 TFLOP/s, 0.63 of the FP32 FMA rate);
+// unpacked FMAs with the filter left to the next layer's loads took 534 us.
+struct FmFirstArgs {
+    const uint8_t* in;
+    int64_t in_slice, in_pitch;
+    int src_h, src_w;    // slice size for reflect-101
+    int off_y, off_x;    // conv input (r, c) reads slice (refl(r + off_y), refl(c + off_x))
+    uint16_t* out;
+    int64_t out_slice, out_pitch;  // elements per slice, columns per row
+    int rows, cols;      // filtered outputs
+    int n_strips;
+    int64_t total;       // strip-rows of the launch: nz x n_strips x rows
+    float2 w[16][32];    // [4 ky + kx][channel pair]
+    float2 b[32];
+};
+
+constexpr int kFirstWarps = 8;
+constexpr int kFirstCols = 68;                // 64 + 3 inputs per row
+
+__device__ __forceinline__ int refl_clamp(int t, int n) {
+    t = t < 0 ? -t : t;
+    t = t >= n ? 2 * (n - 1) - t : t;
+    return min(max(t, 0), n - 1);  // columns past the last strip's domain feed nothing that is stored
+}
+
+template <bool F16>
+__device__ __forceinline__ uint32_t pack16(float a, float b) {
+    uint32_t u;
+    if constexpr (F16) {
+        const __half2 v = __floats2half2_rn(a, b);
+        u = *reinterpret_cast<const uint32_t*>(&v);
+    } else {
+        const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+        u = *reinterpret_cast<const uint32_t*>(&v);
+    }
+    return u;
+}
+
+template <bool F16>
+__device__ __forceinline__ uint32_t max16(uint32_t a, uint32_t b) {
+    if constexpr (F16) {
+        const __half2 v = __hmax2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
+        return *reinterpret_cast<const uint32_t*>(&v);
+    } else {
+        const __nv_bfloat162 v =
+            __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+        return *reinterpret_cast<const uint32_t*>(&v);
+    }
+}
+
+template <bool F16, int ST>
+__global__ void __launch_bounds__(32 * kFirstWarps, 1) fm_first(const __grid_constant__ FmFirstArgs a) {
+    __shared__ __align__(16) float2 s_x[kFirstWarps][4][kFirstCols];  // a ring of 4 input rows per warp
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float2(*sx)[kFirstCols] = s_x[warp];
+    constexpr int kStrip = ST == 1 ? 63 : 32;  // filtered columns of a strip
+    // one equal contiguous range of strip-rows per warp
+    const int64_t n_warps = (int64_t)gridDim.x * kFirstWarps, me = (int64_t)blockIdx.x * kFirstWarps + warp;
+    int64_t pos = a.total * me / n_warps;
+    const int64_t end = a.total * (me + 1) / n_warps;
+    while (pos < end) {
+        const int64_t col = pos / a.rows;
+        const int y0 = (int)(pos - col * a.rows);
+        const int zi = (int)(col / a.n_strips), x0 = (int)(col % a.n_strips) * kStrip;  // filtered coordinates
+        const int rows = (int)min((int64_t)(a.rows - y0), end - pos);
+        pos += rows;
+        const int n_in = (ST == 1 ? rows + 1 : 2 * rows) + 3;  // conv rows + 3
+        const uint8_t* src = a.in + (int64_t)zi * a.in_slice;
+        int sc[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) sc[i] = refl_clamp(ST * x0 + lane + 32 * i + a.off_x, a.src_w);
+        uint8_t u[3];
+        auto fetch = [&](int r) {  // the bytes of input row r of the item
+            const uint8_t* row = src + (int64_t)refl_clamp(ST * y0 + r + a.off_y, a.src_h) * a.in_pitch;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) u[i] = __ldg(row + sc[i]);
+        };
+        uint16_t* out = a.out + (int64_t)zi * a.out_slice;
+        uint32_t prev[2][16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) prev[0][k] = prev[1][k] = 0u;
+        fetch(0);
+#pragma unroll 1
+        for (int r = 0; r < n_in; ++r) {
+            __syncwarp();  // row r - 4, whose slot is written now, has been read
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                if (lane + 32 * i < kFirstCols) {
+                    const float v = (float)u[i] / 255.0f;
+                    sx[r & 3][lane + 32 * i] = make_float2(v, v);
+                }
+            if (r + 1 < n_in) fetch(r + 1);
+            __syncwarp();
+            const int yc = r - 3;  // conv row of the item that input row r completes
+            if (yc < 0) continue;
+            float2 acc[2][32];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) acc[0][c] = acc[1][c] = a.b[c];
+#pragma unroll
+            for (int ky = 0; ky < 4; ++ky) {
+                const float2* row = sx[(r + 1 + ky) & 3] + lane;  // input row yc + ky
+#pragma unroll
+                for (int kx = 0; kx < 4; ++kx) {
+                    const float2 xa = row[kx], xb = row[kx + 32];
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) {
+                        acc[0][c] = __ffma2_rn(a.w[4 * ky + kx][c], xa, acc[0][c]);
+                        acc[1][c] = __ffma2_rn(a.w[4 * ky + kx][c], xb, acc[1][c]);
+                    }
+                }
+            }
+            const bool emit = ST == 1 ? yc > 0 : (yc & 1) != 0;
+            const int y = ST == 1 ? y0 + yc - 1 : y0 + (yc >> 1);
+            uint32_t v[2][16];
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const uint32_t f = pack16<F16>(fmaxf(acc[i][2 * k].x, acc[i][2 * k].y),
+                                                   fmaxf(acc[i][2 * k + 1].x, acc[i][2 * k + 1].y));
+                    v[i][k] = max16<F16>(prev[i][k], f);
+                    prev[i][k] = f;
+                }
+            if (!emit) continue;
+            // horizontal partner: the next column, in the next lane; of column 31 it is lane 0's
+            // column 32, and column 63 has none (a strip yields 63)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const uint32_t n0 = __shfl_sync(0xffffffffu, lane == 0 ? v[1][k] : v[0][k], (lane + 1) & 31);
+                const uint32_t n1 = __shfl_sync(0xffffffffu, v[1][k], (lane + 1) & 31);
+                v[0][k] = max16<F16>(v[0][k], n0);
+                v[1][k] = max16<F16>(v[1][k], n1);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int c = lane + 32 * i;  // conv column of the strip
+                const int x = x0 + (ST == 1 ? c : c >> 1);
+                if ((ST == 1 ? c < 63 : (c & 1) == 0) && x < a.cols) {
+                    uint16_t* o = out + ((int64_t)y * 4 * a.out_pitch + x) * 8;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        *reinterpret_cast<uint4*>(o + (int64_t)q * a.out_pitch * 8) =
+                            make_uint4(v[i][4 * q], v[i][4 * q + 1], v[i][4 * q + 2], v[i][4 * q + 3]);
+                }
+            }
+        }
+    }
+}
+
+template <bool F16, int ST>
+static mb_status launch_first(FmFirstArgs a, int nz, cudaStream_t st) {
+    static int sms = 0;
+    if (sms == 0) {
+        int dev = 0;
+        MB_CUDA(cudaGetDevice(&dev));
+        MB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    }
+    constexpr int kStrip = ST == 1 ? 63 : 32;
+    a.n_strips = (a.cols + kStrip - 1) / kStrip;
+    a.total = (int64_t)nz * a.n_strips * a.rows;
+    // one CTA per SM, or fewer when a warp's range would get under 4 rows
+    const int64_t want = (a.total + 4 * kFirstWarps - 1) / (4 * kFirstWarps);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, want));
+    fm_first<F16, ST><<<grid, 32 * kFirstWarps, 0, st>>>(a);
+    count_launch();
+    MB_CUDA(cudaGetLastError());
+    return MB_OK;
+}
+
+// Tensor-core paths (BF16 or FP16): layer 1 on CUDA cores (FP32 arithmetic, 16-bit out); the 32->64
+// dilated convs and the head on the tensor cores (fastmemb_tc.cu). Every layer leaves what the next
+// one reads: max-filtered 16-bit features, chunk-planar, rows wide enough for the reader's strips.
 mb_status tc_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,
                                int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
                                int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st, int sub) {
@@ -170,49 +350,53 @@ mb_status tc_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_t 
     const int R = nc == 5 ? kFastMemb3nmRadius : kFastMembRadius;
     const FmGeom g = fm_geom(nc, rows, cols, sub);
     auto up = [](int64_t n) { return (n + 127) & ~(int64_t)127; };  // 256-byte aligned sub-buffers
-    int64_t n[kFmMaxConvs - 1];
+    // features entering conv k = 1 .. nc-1: fr x fc of them, fp columns apart, n elements per slice
+    int64_t fr[kFmMaxConvs], fc[kFmMaxConvs], fp[kFmMaxConvs], n[kFmMaxConvs];
     size_t per = 0;
-    for (int k = 0; k < nc - 1; ++k) {
-        n[k] = up(g.r[k] * g.c[k] * 32);
+    for (int k = 1; k < nc; ++k) {
+        const bool head = k == nc - 1;
+        fr[k] = g.r[k] + 3 * g.d[k];
+        fc[k] = g.c[k] + 3 * g.d[k];
+        fp[k] = fm_tc_in_pitch(head, head ? g.c[k] : g.c[k + 1] + 3 * g.d[k + 1], g.d[k]);
+        n[k] = up(fr[k] * 4 * fp[k] * 8);
         per += (size_t)n[k] * 2;
     }
     const size_t budget = (size_t)3 << 30;
     const int64_t zc = std::min<int64_t>(std::min<int64_t>(std::max<size_t>(1, budget / per), 65535), z);
     MB_TRY(net->ws.ensure(per * (size_t)zc));
-    uint16_t* act[kFmMaxConvs - 1];
-    act[0] = static_cast<uint16_t*>(net->ws.ptr);
-    for (int k = 1; k < nc - 1; ++k) act[k] = act[k - 1] + (size_t)zc * n[k - 1];
+    uint16_t* act[kFmMaxConvs];
+    act[1] = static_cast<uint16_t*>(net->ws.ptr);
+    for (int k = 2; k < nc; ++k) act[k] = act[k - 1] + (size_t)zc * n[k - 1];
     const size_t osz = ot == MB_OUT_F32 ? 4 : 1;
     for (int64_t z0 = 0; z0 < z; z0 += zc) {
         const int nz = (int)std::min<int64_t>(zc, z - z0);
-        FmArgs a{};
+        FmFirstArgs a{};
         a.in = in + z0 * in_slice;
         a.in_slice = in_slice;
         a.in_pitch = in_pitch;
-        a.in_rows = (int)(g.r[0] + 3);
-        a.in_cols = (int)(g.c[0] + 3);
         a.src_h = (int)h;
         a.src_w = (int)w;
         a.off_y = (int)(y0 - R);
         a.off_x = (int)(x0 - R);
-        a.d = 1;
-        a.out_h = (int)g.r[0];
-        a.out_w = (int)g.c[0];
-        a.out = act[0];
-        a.out_slice = n[0];
-        a.out_pitch = g.c[0];
-        a.wt = fm_simt_w(net, 0, nc, &a.bias);
+        a.out = act[1];
+        a.out_slice = n[1];
+        a.out_pitch = fp[1];
+        a.rows = (int)fr[1];
+        a.cols = (int)fc[1];
+        const float* w1 = net->host_params.data();  // W1[64][1][4][4], b1[64]
+        for (int t = 0; t < 16; ++t)
+            for (int c = 0; c < 32; ++c) a.w[t][c] = make_float2(w1[32 * c + t], w1[32 * c + 16 + t]);
+        for (int c = 0; c < 32; ++c) a.b[c] = make_float2(w1[64 * 16 + 2 * c], w1[64 * 16 + 2 * c + 1]);
         if (net->prec == MB_PREC_FP16)
-            MB_TRY((launch_fm<1, 1, 64, 8, FM_IN_U8, FM_OUT_MAXOUT_F16>(a, nz, st)));
+            MB_TRY((sub == 2 ? launch_first<true, 2>(a, nz, st) : launch_first<true, 1>(a, nz, st)));
         else
-            MB_TRY((launch_fm<1, 1, 64, 8, FM_IN_U8, FM_OUT_MAXOUT_BF16>(a, nz, st)));
+            MB_TRY((sub == 2 ? launch_first<false, 2>(a, nz, st) : launch_first<false, 1>(a, nz, st)));
         for (int k = 1; k < nc; ++k) {
             const bool head = k == nc - 1;
-            void* o = head ? static_cast<void*>(static_cast<uint8_t*>(out) + z0 * out_slice * osz) : act[k];
-            MB_TRY(fm_tc_layer(net, k - 1, act[k - 1], n[k - 1], g.c[k - 1], g.r[k - 1], g.c[k - 1],
-                               (int)fm_in_extent(g, k, true), (int)fm_in_extent(g, k, false), g.dm[k], g.st[k], o,
-                               head ? out_slice : n[k], head ? out_pitch : g.c[k], (int)g.r[k], (int)g.c[k], g.d[k],
-                               nz, head && ot == MB_OUT_U8, st));
+            void* o = head ? static_cast<void*>(static_cast<uint8_t*>(out) + z0 * out_slice * osz) : act[k + 1];
+            MB_TRY(fm_tc_layer(net, k - 1, act[k], n[k], fp[k], o, head ? out_slice : n[k + 1],
+                               head ? out_pitch : fp[k + 1], (int)(head ? g.r[k] : fr[k + 1]),
+                               (int)(head ? g.c[k] : fc[k + 1]), g.d[k], nz, head && ot == MB_OUT_U8, st));
         }
     }
     return fm_tc_poll_error(net);

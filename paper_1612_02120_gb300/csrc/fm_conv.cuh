@@ -5,11 +5,9 @@
 // plain 4x4 conv on the d-strided sub-grid (a max-pooling fragment), so each CTA computes a
 // TH x 32 tile of one fragment: 4 consecutive fragment pixels x CPT conv channels per thread,
 // input channels staged CC at a time with the previous stage's dilated 2x2 max-filter (and an
-// optional source stride) applied while staging. Epilogues: max-out of adjacent channel pairs
-// (FP32, BF16 or FP16 out), or the 2-class softmax.
+// optional source stride) applied while staging. Epilogues: max-out of adjacent channel pairs,
+// or the 2-class softmax.
 #pragma once
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -20,7 +18,7 @@ namespace mb {
 namespace {
 
 enum { FM_IN_U8 = 0, FM_IN_F32 = 1 };
-enum { FM_OUT_MAXOUT = 0, FM_OUT_SOFTMAX_F32 = 1, FM_OUT_SOFTMAX_U8 = 2, FM_OUT_MAXOUT_BF16 = 3, FM_OUT_MAXOUT_F16 = 4 };
+enum { FM_OUT_MAXOUT = 0, FM_OUT_SOFTMAX_F32 = 1, FM_OUT_SOFTMAX_U8 = 2 };
 
 struct FmArgs {
     const void* in;
@@ -160,35 +158,7 @@ __global__ void __launch_bounds__(256) fm_conv(const FmArgs a) {
 
     const int oy = ry + d * (fy0 + ty);
     if (oy >= a.out_h) return;
-    if constexpr (OUT == FM_OUT_MAXOUT_BF16 || OUT == FM_OUT_MAXOUT_F16) {
-        // 16-bit activations (BF16 or FP16), the tensor-core layers' input
-        static_assert(CPT >= 8, "max-out epilogue writes 4 channels per 8 conv channels");
-        uint16_t* o = static_cast<uint16_t*>(a.out) + (int64_t)zi * a.out_slice;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int ox = rx + d * (fx0 + 4 * tx + j);
-            if (ox < a.out_w) {
-#pragma unroll
-                for (int q = 0; q < CPT / 8; ++q) {
-                    const float* v = acc[j] + 8 * q;
-                    const float2 l = make_float2(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
-                    const float2 h = make_float2(fmaxf(v[4], v[5]), fmaxf(v[6], v[7]));
-                    uint2 u;
-                    if constexpr (OUT == FM_OUT_MAXOUT_F16) {
-                        __half2 lo = __floats2half2_rn(l.x, l.y), hi = __floats2half2_rn(h.x, h.y);
-                        u.x = *reinterpret_cast<uint32_t*>(&lo);
-                        u.y = *reinterpret_cast<uint32_t*>(&hi);
-                    } else {
-                        __nv_bfloat162 lo = __floats2bfloat162_rn(l.x, l.y), hi = __floats2bfloat162_rn(h.x, h.y);
-                        u.x = *reinterpret_cast<uint32_t*>(&lo);
-                        u.y = *reinterpret_cast<uint32_t*>(&hi);
-                    }
-                    *reinterpret_cast<uint2*>(o + ((int64_t)oy * a.out_pitch + ox) * (CO / 2) + (CPT / 2) * cg + 4 * q) =
-                        u;
-                }
-            }
-        }
-    } else if constexpr (OUT == FM_OUT_MAXOUT) {
+    if constexpr (OUT == FM_OUT_MAXOUT) {
         static_assert(CPT >= 8, "max-out epilogue writes 4 channels per 8 conv channels");
         float* o = static_cast<float*>(a.out) + (int64_t)zi * a.out_slice;
 #pragma unroll

@@ -121,12 +121,15 @@ mb_status tc_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_t 
 mb_status fm_tc_prepare(mb_net* net);
 void fm_tc_release(mb_net* net);
 mb_status fm_tc_poll_error(mb_net* net);
-// in: [slice][src_rows][src_cols(pitch)][32] BF16 or FP16 (the net's type); the conv reads input
-// (r, c) = 2x2 max (dilation dm) at source (stride r, stride c), for r < in_rows, c < in_cols.
+// in, and a layer's out: 16-bit features of the net's type, max-filtered, chunk-planar
+// [slice][row][chunk 0..3][column (pitch)][8 channels]. rows x cols: what the layer writes (filtered
+// features; the head: the map, FP32 or uint8), i.e. it reads rows + 3d (+ d for a layer) input rows.
+// in_pitch is at least fm_tc_in_pitch of the same cols and d (the last strip's overrun).
 // layer: 0-based index of the conv after conv1; the last one is the head.
-mb_status fm_tc_layer(mb_net* net, int layer, const void* in, int64_t in_slice, int64_t in_pitch, int64_t src_rows,
-                      int64_t src_cols, int in_rows, int in_cols, int dm, int stride, void* out, int64_t out_slice,
-                      int64_t out_pitch, int out_h, int out_w, int d, int nz, int out_u8, cudaStream_t st);
+int64_t fm_tc_in_pitch(bool head, int64_t cols, int d);
+mb_status fm_tc_layer(mb_net* net, int layer, const void* in, int64_t in_slice, int64_t in_pitch, void* out,
+                      int64_t out_slice, int64_t out_pitch, int rows, int cols, int d, int nz, int out_u8,
+                      cudaStream_t st);
 // MaskExtend (maskextend.cu): SIMT weight layout, and the +z transfer recursion (device pointers).
 void me_pack(const mb_net* net, const float* params, std::vector<float>& out);
 // MaskExtend FP16 tensor-core convs (maskextend_tc.cu). layer 0..4; in: [src rows][in_pitch][cs] FP16;

@@ -122,6 +122,29 @@ __device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The same (accumulating), executed where `on` is non-zero: a whole warp walks the issue loop, its
+// values in uniform registers, with one lane issuing. Descriptors as their two 32-bit words (the
+// start address is in the low one, so a caller steps that alone).
+__device__ __forceinline__ void mma_bf16_if(uint32_t on, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                            uint32_t b_hi, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 q, %6, 0;\n\t"
+        "setp.eq.b32 p, 0, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(on)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit_if(uint32_t on, uint64_t* bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
+        "r"(on)
+        : "memory");
+}
 // Arrive (count 1) on an mbarrier once all tcgen05 async operations issued so far by this
 // thread have completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
