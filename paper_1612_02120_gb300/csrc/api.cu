@@ -528,6 +528,7 @@ mb_status mb_net_destroy(mb_net* net) {
         fm_tc_release(net);
         me_tc_release(net);
         st_tc_release(net);
+        x3_release(net);
         dev_free(net->d_params);
         dev_free(net->d_simt);
         dev_free(net->d_queue);
@@ -590,7 +591,7 @@ mb_status mb_load_weights(mb_net* net, const float* params, int64_t n_params) {
     if (is_fastmemb(net->family) && (net->prec == MB_PREC_BF16 || net->prec == MB_PREC_FP16))
         MB_TRY(fm_tc_prepare(net));
     if (net->family == FAMILY_MASKEXTEND && net->prec == MB_PREC_FP16) MB_TRY(me_tc_prepare(net));
-    return MB_OK;
+    return x3_prepare(net);
 }
 
 mb_status mb_get_weights(const mb_net* net, float* params, int64_t n_params) {

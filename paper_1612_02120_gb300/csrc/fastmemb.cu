@@ -94,6 +94,7 @@ mb_status simt_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_
                                int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
                                int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st, int sub) {
     if (z == 0 || rows == 0 || cols == 0) return MB_OK;
+    MB_TRY(x3_poll_error(net));
     const int nc = fastmemb_convs(net->family);
     const int R = nc == 5 ? kFastMemb3nmRadius : kFastMembRadius;
     const FmGeom g = fm_geom(nc, rows, cols, sub);
@@ -142,7 +143,27 @@ mb_status simt_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_
                 b.out = act[k];
                 b.out_slice = g.r[k] * g.c[k] * 32;
                 b.out_pitch = g.c[k];
-                MB_TRY((launch_fm<32, 8, 64, 8, FM_IN_F32, FM_OUT_MAXOUT>(b, nz, st)));
+                if (net->x3_ok) {
+                    X3Layer a3{};
+                    a3.in = act[k - 1];
+                    a3.in_slice = b.in_slice;
+                    a3.in_pitch = b.in_pitch;
+                    a3.in_rows = b.in_rows;
+                    a3.in_cols = b.in_cols;
+                    a3.src_cols = g.c[k - 1];
+                    a3.d = b.d;
+                    a3.dm = b.dm;
+                    a3.stride = b.in_stride;
+                    a3.out = act[k];
+                    a3.out_slice = b.out_slice;
+                    a3.out_pitch = b.out_pitch;
+                    a3.out_h = b.out_h;
+                    a3.out_w = b.out_w;
+                    a3.nz = nz;
+                    MB_TRY(x3_layer(net, k - 1, a3, st));
+                } else {
+                    MB_TRY((launch_fm<32, 8, 64, 8, FM_IN_F32, FM_OUT_MAXOUT>(b, nz, st)));
+                }
             } else {
                 b.out_slice = out_slice;
                 b.out_pitch = out_pitch;
@@ -156,7 +177,7 @@ mb_status simt_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_
             }
         }
     }
-    return MB_OK;
+    return x3_poll_error(net);
 }
 
 // Layer 1 of the tensor-core paths: conv 4x4 1 -> 64 from the uint8 slice in FP32, max-out over

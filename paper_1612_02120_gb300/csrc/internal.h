@@ -77,6 +77,8 @@ struct mb_net {
     void* tc_state = nullptr;    // tensor-core path state (packed operands, constants), tc_conv.cu
     void* fm_state = nullptr;    // FastMemb tensor-core state (packed operands, error word), fastmemb_tc.cu
     void* me_state = nullptr;    // MaskExtend tensor-core state (packed operands, error word), maskextend_tc.cu
+    void* x3_state = nullptr;    // FP32 tensor-core layers (packed split operands, error word), f32_tc.cu
+    bool x3_ok = false;          // its activations are bounded: those layers run on the tensor cores
     void* st_state = nullptr;    // student tensor-core state (packed operands, error word), student_tc.cu
     float fp8_amax[2][32] = {};
     mb::Workspace ws;            // layered FP32 path activations
@@ -154,6 +156,30 @@ void st_tc_release(mb_net* net);
 mb_status student_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,
                          int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
                          int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st);
+// FP32 layers on the tensor cores (f32_tc.cu): 5x5 32 -> 32 of the teacher (layer 0: ReLU, FP32 out;
+// layer 1: ReLU, head, sigmoid, FP32 or uint8 map out), 4x4 32 -> 64 with max-out of FastMemb (layer =
+// 0-based conv after conv1). in and feature outputs: FP32 [slice][row][column (pitch)][32]; the conv
+// reads input (r, c) = 2x2 max (dilation dm; 0: none) at source (stride r, stride c), r < in_rows,
+// c < in_cols. x3_prepare packs at load time and sets net->x3_ok; where it is false the CUDA-core
+// kernels run.
+struct X3Layer {
+    const float* in;
+    int64_t in_slice, in_pitch;
+    int in_rows, in_cols;
+    int64_t src_cols;
+    int d, dm, stride;
+    void* out;
+    int64_t out_slice, out_pitch;
+    int out_h, out_w, nz, out_u8;
+};
+mb_status x3_prepare(mb_net* net);
+void x3_release(mb_net* net);
+mb_status x3_poll_error(mb_net* net);
+mb_status x3_layer(const mb_net* net, int layer, const X3Layer& a, cudaStream_t st);
+// Layers 2 and 3 of the FP32 teacher for nz slices: act1 [nz][rows + 10][cols + 10][32] -> act2
+// [nz][rows + 5][cols + 5][32] -> the map; on the tensor cores, or (x3_ok false) on CUDA cores.
+mb_status teacher_fp32_deep(const mb_net* net, const float* act1, float* act2, int nz, int64_t rows, int64_t cols,
+                            void* out, int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st);
 // FP32 teacher activations after the two max-filters: per-channel amax over n slices (device out[64]).
 mb_status simt_teacher_amax(mb_net* net, const uint8_t* in, int64_t n, int64_t h, int64_t w, float* d_amax,
                             cudaStream_t st);

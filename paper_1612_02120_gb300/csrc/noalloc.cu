@@ -60,16 +60,9 @@ static size_t band_floats(int64_t nz, int64_t rows, int64_t cols) {
 // activations in `scratch`.
 static mb_status noalloc_band(const mb_net* net, const uint8_t* in, int nz, int64_t h, int64_t w, int64_t y0,
                               int64_t rows, void* out, mb_out_type ot, float* scratch, cudaStream_t st) {
-    const int64_t cols = w, r1 = rows + 10, c1 = cols + 10, r2 = rows + 5, c2 = cols + 5;
+    const int64_t cols = w, r1 = rows + 10, c1 = cols + 10;
     float* act1 = scratch;
     float* act2 = act1 + (size_t)nz * r1 * c1 * 32;
-    const float* w1 = net->d_simt;
-    const float* b1 = w1 + 25 * 32;
-    const float* w2 = b1 + 32;
-    const float* b2 = w2 + 25 * 32 * 32;
-    const float* w3 = b2 + 32;
-    const float* b3 = w3 + 25 * 32 * 32;
-    const float* hw = b3 + 32;
     ConvArgs a{};
     a.in = in;
     a.in_slice = h * w;
@@ -85,44 +78,11 @@ static mb_status noalloc_band(const mb_net* net, const uint8_t* in, int nz, int6
     a.out = act1;
     a.out_slice = r1 * c1 * 32;
     a.out_pitch = c1;
-    a.wt = w1;
-    a.bias = b1;
+    a.wt = net->d_simt;
+    a.bias = net->d_simt + 25 * 32;
     MB_TRY((launch_conv<5, 1, 32, 1, IN_U8, OUT_ACT>(a, nz, st)));
-    ConvArgs b{};
-    b.in = act1;
-    b.in_slice = r1 * c1 * 32;
-    b.in_pitch = c1;
-    b.in_rows = (int)(r2 + 4);
-    b.in_cols = (int)(c2 + 4);
-    b.out_h = (int)r2;
-    b.out_w = (int)c2;
-    b.out = act2;
-    b.out_slice = r2 * c2 * 32;
-    b.out_pitch = c2;
-    b.wt = w2;
-    b.bias = b2;
-    MB_TRY((launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_ACT>(b, nz, st)));
-    ConvArgs c{};
-    c.in = act2;
-    c.in_slice = r2 * c2 * 32;
-    c.in_pitch = c2;
-    c.in_rows = (int)(rows + 4);
-    c.in_cols = (int)(cols + 4);
-    c.out_h = (int)rows;
-    c.out_w = (int)cols;
-    c.out_slice = h * w;
-    c.out_pitch = w;
-    c.wt = w3;
-    c.bias = b3;
-    c.head_w = hw;
-    if (ot == MB_OUT_F32) {
-        c.out = static_cast<float*>(out) + y0 * w;
-        MB_TRY((launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_HEAD_F32>(c, nz, st)));
-    } else {
-        c.out = static_cast<uint8_t*>(out) + y0 * w;
-        MB_TRY((launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_HEAD_U8>(c, nz, st)));
-    }
-    return MB_OK;
+    const size_t osz = ot == MB_OUT_F32 ? 4 : 1;
+    return teacher_fp32_deep(net, act1, act2, nz, rows, cols, static_cast<uint8_t*>(out) + y0 * w * osz, w, h * w, ot, st);
 }
 
 }  // namespace mb
@@ -165,6 +125,7 @@ extern "C" mb_status mb_infer_volume_noalloc(mb_net* net, const uint8_t* in, int
         return MB_ERR_SHAPE;
     }
     if (z == 0) return MB_OK;
+    MB_TRY(x3_poll_error(net));
     int prev = -1;
     cudaGetDevice(&prev);
     if (prev != net->device) {

@@ -75,21 +75,86 @@ static int64_t chunk_slices(size_t per_slice, int64_t z) {
     return std::min<int64_t>(zc, z);
 }
 
+mb_status teacher_fp32_deep(const mb_net* net, const float* act1, float* act2, int nz, int64_t rows, int64_t cols,
+                            void* out, int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st) {
+    const int64_t r1 = rows + 10, c1 = cols + 10, r2 = rows + 5, c2 = cols + 5;
+    if (net->x3_ok) {
+        X3Layer a{};
+        a.in = act1;
+        a.in_slice = r1 * c1 * 32;
+        a.in_pitch = c1;
+        a.in_rows = (int)(r2 + 4);
+        a.in_cols = (int)(c2 + 4);
+        a.src_cols = c1;
+        a.d = 1;
+        a.dm = 1;
+        a.out = act2;
+        a.out_slice = r2 * c2 * 32;
+        a.out_pitch = c2;
+        a.out_h = (int)r2;
+        a.out_w = (int)c2;
+        a.nz = nz;
+        MB_TRY(x3_layer(net, 0, a, st));
+        a.in = act2;
+        a.in_slice = r2 * c2 * 32;
+        a.in_pitch = c2;
+        a.in_rows = (int)(rows + 4);
+        a.in_cols = (int)(cols + 4);
+        a.src_cols = c2;
+        a.out = out;
+        a.out_slice = out_slice;
+        a.out_pitch = out_pitch;
+        a.out_h = (int)rows;
+        a.out_w = (int)cols;
+        a.out_u8 = ot == MB_OUT_U8;
+        return x3_layer(net, 1, a, st);
+    }
+    const float* w2 = net->d_simt + 25 * 32 + 32;
+    const float* b2 = w2 + 25 * 32 * 32;
+    const float* w3 = b2 + 32;
+    const float* b3 = w3 + 25 * 32 * 32;
+    ConvArgs b{};
+    b.in = act1;
+    b.in_slice = r1 * c1 * 32;
+    b.in_pitch = c1;
+    b.in_rows = (int)(r2 + 4);
+    b.in_cols = (int)(c2 + 4);
+    b.out_h = (int)r2;
+    b.out_w = (int)c2;
+    b.out = act2;
+    b.out_slice = r2 * c2 * 32;
+    b.out_pitch = c2;
+    b.wt = w2;
+    b.bias = b2;
+    MB_TRY((launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_ACT>(b, nz, st)));
+    ConvArgs c{};
+    c.in = act2;
+    c.in_slice = r2 * c2 * 32;
+    c.in_pitch = c2;
+    c.in_rows = (int)(rows + 4);
+    c.in_cols = (int)(cols + 4);
+    c.out_h = (int)rows;
+    c.out_w = (int)cols;
+    c.out = out;
+    c.out_slice = out_slice;
+    c.out_pitch = out_pitch;
+    c.wt = w3;
+    c.bias = b3;
+    c.head_w = b3 + 32;
+    if (ot == MB_OUT_F32) return launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_HEAD_F32>(c, nz, st);
+    return launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_HEAD_U8>(c, nz, st);
+}
+
 mb_status simt_teacher_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,
                               int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
                               int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st) {
-    const int64_t r1 = rows + 10, c1 = cols + 10, r2 = rows + 5, c2 = cols + 5;
+    MB_TRY(x3_poll_error(net));
+    const int64_t r1 = rows + 10, c1 = cols + 10;
     const int64_t zc = chunk_slices(teacher_ws_per_slice(rows, cols), z);
     MB_TRY(net->ws.ensure(teacher_ws_per_slice(rows, cols) * (size_t)zc));
     float* act1 = static_cast<float*>(net->ws.ptr);
     float* act2 = act1 + (size_t)zc * r1 * c1 * 32;
-    const float* w1 = net->d_simt;
-    const float* b1 = w1 + 25 * 32;
-    const float* w2 = b1 + 32;
-    const float* b2 = w2 + 25 * 32 * 32;
-    const float* w3 = b2 + 32;
-    const float* b3 = w3 + 25 * 32 * 32;
-    const float* hw = b3 + 32;
+    const size_t osz = ot == MB_OUT_F32 ? 4 : 1;
     for (int64_t z0 = 0; z0 < z; z0 += zc) {
         const int nz = (int)std::min<int64_t>(zc, z - z0);
         ConvArgs a{};
@@ -107,49 +172,17 @@ mb_status simt_teacher_region(mb_net* net, const uint8_t* in, int64_t z, int64_t
         a.out = act1;
         a.out_slice = r1 * c1 * 32;
         a.out_pitch = c1;
-        a.wt = w1;
-        a.bias = b1;
+        a.wt = net->d_simt;
+        a.bias = net->d_simt + 25 * 32;
         MB_TRY((launch_conv<5, 1, 32, 1, IN_U8, OUT_ACT>(a, nz, st)));
-
-        ConvArgs b{};
-        b.in = act1;
-        b.in_slice = r1 * c1 * 32;
-        b.in_pitch = c1;
-        b.in_rows = (int)(r2 + 4);
-        b.in_cols = (int)(c2 + 4);
-        b.out_h = (int)r2;
-        b.out_w = (int)c2;
-        b.out = act2;
-        b.out_slice = r2 * c2 * 32;
-        b.out_pitch = c2;
-        b.wt = w2;
-        b.bias = b2;
-        MB_TRY((launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_ACT>(b, nz, st)));
-
-        ConvArgs c{};
-        c.in = act2;
-        c.in_slice = r2 * c2 * 32;
-        c.in_pitch = c2;
-        c.in_rows = (int)(rows + 4);
-        c.in_cols = (int)(cols + 4);
-        c.out_h = (int)rows;
-        c.out_w = (int)cols;
-        c.out_slice = out_slice;
-        c.out_pitch = out_pitch;
-        c.wt = w3;
-        c.bias = b3;
-        c.head_w = hw;
-        if (ot == MB_OUT_F32) {
-            c.out = static_cast<float*>(out) + z0 * out_slice;
-            MB_TRY((launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_HEAD_F32>(c, nz, st)));
-        } else {
-            c.out = static_cast<uint8_t*>(out) + z0 * out_slice;
-            MB_TRY((launch_conv<5, 32, 32, 8, IN_F32_MAXF, OUT_HEAD_U8>(c, nz, st)));
-        }
+        MB_TRY(teacher_fp32_deep(net, act1, act2, nz, rows, cols, static_cast<uint8_t*>(out) + z0 * out_slice * osz,
+                                 out_pitch, out_slice, ot, st));
     }
-    return MB_OK;
+    return x3_poll_error(net);
 }
 
+// (The FP8 scales come from these activations: the CUDA-core kernels compute them, so that a
+// calibrated net's quantisation does not move with the kernel that serves FP32 maps.)
 mb_status simt_teacher_amax(mb_net* net, const uint8_t* in, int64_t n, int64_t h, int64_t w, float* d_amax,
                             cudaStream_t st) {
     const int64_t r1 = h + 10, c1 = w + 10, r2 = h + 5, c2 = w + 5;
