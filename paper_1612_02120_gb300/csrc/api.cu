@@ -492,6 +492,7 @@ mb_status mb_net_create(const mb_layer_desc* layers, int32_t n_layers, mb_precis
     net->device = device;
     net->family = fam;
     net->prec = prec;
+    if (prec == MB_PREC_FP8) net->stages = 6;
     net->layers.assign(layers, layers + n_layers);
     int64_t np = 0;
     for (const auto& L : net->layers)

@@ -484,8 +484,8 @@ mb_status launch_x3(XParams& p, cudaStream_t st) {
         MB_CUDA(cudaFuncSetAttribute(x3_conv<K, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem));
         attr = true;
     }
-    // one range per SM, or fewer when a range would get under 4 rows
-    const int64_t per_half = std::max<int64_t>(1, std::min<int64_t>(n_sms / p.halves, (p.total_rows + 3) / 4));
+    // one range per SM, or fewer when a range would get under 2 rows (each costs K - 1 more staged rows)
+    const int64_t per_half = std::max<int64_t>(1, std::min<int64_t>(n_sms / p.halves, (p.total_rows + 1) / 2));
     x3_conv<K, OUT><<<(unsigned)(per_half * p.halves), C::kThreads, C::kSmem, st>>>(p);
     count_launch();
     MB_CUDA(cudaGetLastError());

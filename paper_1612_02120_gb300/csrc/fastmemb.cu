@@ -350,8 +350,9 @@ static mb_status launch_first(FmFirstArgs a, int nz, cudaStream_t st) {
     constexpr int kStrip = ST == 1 ? 63 : 32;
     a.n_strips = (a.cols + kStrip - 1) / kStrip;
     a.total = (int64_t)nz * a.n_strips * a.rows;
-    // one CTA per SM, or fewer when a warp's range would get under 4 rows
-    const int64_t want = (a.total + 4 * kFirstWarps - 1) / (4 * kFirstWarps);
+    // one CTA per SM, or fewer where a warp would get no row (a row costs 2 conv rows at the start of
+    // a range, so short ranges cost throughput only where the launch is too small to fill the chip)
+    const int64_t want = (a.total + kFirstWarps - 1) / kFirstWarps;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, want));
     fm_first<F16, ST><<<grid, 32 * kFirstWarps, 0, st>>>(a);
     count_launch();

@@ -571,8 +571,9 @@ mb_status launch_fm_tc(const FmTcParams& p, cudaStream_t st) {
         MB_CUDA(cudaFuncSetAttribute(fm_tc_conv<HEAD, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem));
         attr = true;
     }
-    // one range per resident CTA, or fewer when a range would get under 8 rows
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)n_sms * C::kCtas, (p.total_rows + 7) / 8));
+    // one range per resident CTA, or fewer when a range would get under 2 rows (each costs 4 more
+    // staged rows: a launch this small is latency, not throughput)
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)n_sms * C::kCtas, (p.total_rows + 1) / 2));
     fm_tc_conv<HEAD, F16><<<grid, C::kThreads, C::kSmem, st>>>(p);
     count_launch();
     MB_CUDA(cudaGetLastError());
