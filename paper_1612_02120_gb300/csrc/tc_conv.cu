@@ -309,59 +309,53 @@ __device__ __forceinline__ void store_eighth(uint8_t* slot, int c, int h, const 
     }
 }
 
-// Issue the MMAs of groups [g_lo, g_hi) of one input row r for one layer: output rows j = r-4+i of
-// the layer for the valid blocks i (0 <= j < n_out). Every MMA accumulates; the epilogue zeroes an accumulator after
+// Issue the MMAs of one input row r for one layer: output rows j = r-4+i of the layer for the valid
+// blocks i (0 <= j < n_out). Every MMA accumulates; the epilogue zeroes an accumulator after
 // draining it, so a row's first contribution adds to zero. Blocks go to ring slots
-// (base + r - 4 + i) mod kAcc; runs of contiguous slots are one MMA each.
-template <bool FP8>
-__device__ __forceinline__ void issue_row(uint32_t tcol0, uint32_t acc_base_seq, int r, int n_out, uint64_t adesc0,
-                                          uint64_t bdesc0, int g_lo, int g_hi) {
+// (base + r - 4 + i) mod kAcc; runs of contiguous slots are one MMA each. The whole warp executes
+// this on uniform values, the lane with `on` issuing; `between(g)` runs after the MMAs of group g.
+// The issuing thread bounds a row as much as the tensor pipe does, so the full window in one piece is
+// straight-line code of a fixed shape.
+template <bool FP8, class Between>
+__device__ __forceinline__ void issue_row(uint32_t on, uint32_t tcol0, uint32_t acc_base_seq, int r, int n_out,
+                                          uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, Between between) {
     using C = Cfg<FP8>;
     constexpr int G = C::kGroups;
     constexpr int K = C::kAcc;
     constexpr uint32_t fmt = FP8 ? ptx::kFmtE4M3 : ptx::kFmtBF16;
-    const int ilo = max(0, 4 - r);
-    const int ihi = min(4, n_out + 3 - r);
-    if (ilo > ihi) return;
+    auto mma = [](uint32_t go, uint32_t d, uint32_t al, uint32_t ah, uint32_t bl, uint32_t bh, uint32_t id) {
+        if (FP8)
+            ptx::mma_e4m3_if(go, d, al, ah, bl, bh, id);
+        else
+            ptx::mma_bf16_if(go, d, al, ah, bl, bh, id);
+    };
+    auto a_of = [&](int g) {  // operand start of group g = (dx, K-half): in units of 16 bytes
+        const int dx = FP8 ? g : (g >> 1), hk = FP8 ? 0 : (g & 1);
+        return a_lo + (uint32_t)(hk * 2 * kPitch + dx);
+    };
+    const int ilo = max(0, 4 - r), ihi = min(4, n_out + 3 - r);
     const int s_lo = (int)((acc_base_seq + (uint32_t)(r - 4 + ilo)) % K);
-    uint32_t d[2], boff[2], idesc[2];
-    int nrun;
-    if (K == 5 && ilo == 0 && ihi == 4) {
-        // full window: slots 0..4, B rows rotated so slot 0 receives block (5 - s_lo) mod 5
-        const int i0 = (5 - s_lo) % 5;
-        d[0] = tcol0;
-        boff[0] = (uint32_t)(i0 * 32 * 16) >> 4;
-        idesc[0] = ptx::idesc_f32acc(fmt, 128, 160);
-        nrun = 1;
-    } else {
-        const int iw = ilo + (K - s_lo);  // first block whose slot wrapped to 0
-        const int hi0 = iw <= ihi ? iw - 1 : ihi;
-        d[0] = tcol0 + 32u * (uint32_t)s_lo;
-        boff[0] = (uint32_t)(ilo * 32 * 16) >> 4;
-        idesc[0] = ptx::idesc_f32acc(fmt, 128, (uint32_t)(32 * (hi0 - ilo + 1)));
-        nrun = 1;
-        if (iw <= ihi) {
-            d[1] = tcol0;
-            boff[1] = (uint32_t)(iw * 32 * 16) >> 4;
-            idesc[1] = ptx::idesc_f32acc(fmt, 128, (uint32_t)(32 * (ihi - iw + 1)));
-            nrun = 2;
+    if (ilo == 0 && ihi == 4 && (K == 5 || s_lo + 4 < K)) {
+        // full window. Ring of 5: slots 0..4, B rows rotated so slot 0 receives block (5 - s_lo) mod 5
+        constexpr uint32_t id = ptx::idesc_f32acc(fmt, 128, 160);
+        const uint32_t d = K == 5 ? tcol0 : tcol0 + 32u * (uint32_t)s_lo;
+        const uint32_t b0 = K == 5 ? b_lo + (uint32_t)((5 - s_lo) % 5 * 32) : b_lo;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            mma(on, d, a_of(g), a_hi, b0 + (uint32_t)((g * C::kGroupB) >> 4), b_hi, id);
+            between(g);
         }
-    }
+    } else {
+        const int n = ihi - ilo + 1, n1 = min(n, K - s_lo);  // blocks before the ring wraps
+        const uint32_t id0 = ptx::idesc_f32acc(fmt, 128, 0);
+        const uint32_t id1 = id0 | (uint32_t)(4 * n1) << 17, id2 = id0 | (uint32_t)(4 * (n - n1)) << 17;
+        const uint32_t on1 = n > 0 ? on : 0u, on2 = n1 < n ? on : 0u;
+        const uint32_t d = tcol0 + 32u * (uint32_t)s_lo, b1 = b_lo + (uint32_t)(ilo * 32), b2 = b1 + (uint32_t)(n1 * 32);
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        if (g < g_lo || g >= g_hi) continue;
-        const int dx = FP8 ? g : (g >> 1);
-        const int hk = FP8 ? 0 : (g & 1);
-        const uint64_t ad = adesc0 + (uint64_t)((hk * 2 * kPitch * 16 + dx * 16) >> 4);
-        const uint64_t bg = bdesc0 + (uint64_t)((g * C::kGroupB) >> 4);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            if (k < nrun) {
-                if (FP8)
-                    ptx::mma_e4m3(d[k], ad, bg + boff[k], idesc[k], 1u);
-                else
-                    ptx::mma_bf16(d[k], ad, bg + boff[k], idesc[k], 1u);
-            }
+        for (int g = 0; g < G; ++g) {
+            mma(on1, d, a_of(g), a_hi, b1 + (uint32_t)((g * C::kGroupB) >> 4), b_hi, id1);
+            mma(on2, tcol0, a_of(g), a_hi, b2 + (uint32_t)((g * C::kGroupB) >> 4), b_hi, id2);
+            between(g);
         }
     }
 }
@@ -390,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
     const float* cst = reinterpret_cast<const float*>(smem + C::oConst);
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // warp: known to be uniform
 
     // ---- set-up: barriers, B operands, ring padding, TMEM ------------------------------------
     if (tid == 0) {
@@ -457,8 +451,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
         if (warp == 0 || warp == 2) {
         // ================= MMA issuers: warp 0 lane 0 for layer 2, warp 2 lane 0 for layer 3 ======
         // Each issuer commits (and finally drains) only its own MMAs.
-        if (lane == 0) {
             const bool l2 = warp == 0;
+            const uint32_t lead = lane == 0;
             uint32_t in_seq = 0, acc_seq = 0;  // A-ring rows consumed, accumulator rows completed
             bool ok = true;
             // ring slot i of the layer's A operand: base descriptor + i slots (start-address field)
@@ -469,12 +463,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
             uint64_t* empty = l2 ? B.m1_empty : B.m2_empty;
             uint64_t* afree = l2 ? B.a2_free : B.a3_free;
             uint64_t* afull = l2 ? B.a2_full : B.a3_full;
-            // The waits for input row r+1 are taken between the two halves of row r's MMAs, while the
-            // first half still queues in the tensor pipe (a poll competes with the operand reads for
-            // the shared-memory pipe). The accumulator of output row r+1 shares its slot with output
-            // row r+1-kAcc, completed by input row r+5-kAcc: mid-row for the ring of 8 (BF16), but
-            // only at the end of row r itself for the ring of 5 (FP8), where that wait stays after
-            // the row's commits.
+            // The waits for input row r+1 are taken between row r's MMAs, while some of them still
+            // queue in the tensor pipe, and (ring of 8) the commits of row r between the MMAs of row
+            // r+1. The accumulator of output row r+1 shares its slot with output row r+1-kAcc,
+            // completed by input row r+5-kAcc: mid-row for the ring of 8 (BF16), but only at the end
+            // of row r itself for the ring of 5 (FP8), where the commits and that wait stay behind
+            // the row's MMAs.
             constexpr int G = C::kGroups;
             constexpr bool kEarlyAcc = C::kAcc >= 6;
             auto wait_in = [&](uint32_t q) {
@@ -490,29 +484,33 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
                 const int NR = it.rows;
                 const int n_in = l2 ? NR + 9 : NR + 4;   // input rows of this layer
                 const int n_out = l2 ? NR + 5 : NR;      // output rows of this layer
+                auto commit_row = [&](int r) {
+                    ptx::mma_commit_if(lead, &empty[(in_seq + r) % kRing]);
+                    if (r >= 4) ptx::mma_commit_if(lead, &afull[(acc_seq + r - 4) % C::kAcc]);
+                };
                 wait_in(in_seq);
-                if (n_out > 0) wait_acc(acc_seq);
+                wait_acc(acc_seq);
                 ptx::tc_fence_after();
                 for (int r = 0; r < n_in; ++r) {
-                    const uint32_t q = in_seq + r, s = q % kRing;
-                    const uint64_t arow = ad + (uint64_t)(s * (C::kSlotBytes >> 4));
-                    if (ok) issue_row<FP8>(tcol, acc_seq, r, n_out, arow, bd, 0, G / 2);
-                    if (r + 1 < n_in) {
-                        wait_in(q + 1);
-                        if (kEarlyAcc && r + 1 < n_out) wait_acc(acc_seq + r + 1);
-                        ptx::tc_fence_after();
+                    const uint32_t s = (in_seq + r) % kRing;
+                    issue_row<FP8>(ok ? lead : 0u, tcol, acc_seq, r, n_out, (uint32_t)ad + s * (C::kSlotBytes >> 4),
+                                   (uint32_t)(ad >> 32), (uint32_t)bd, (uint32_t)(bd >> 32), [&](int g) {
+                                       if (kEarlyAcc && g == 0 && r > 0) commit_row(r - 1);
+                                       if (g == G / 2 && r + 1 < n_in) wait_in(in_seq + r + 1);
+                                       if (kEarlyAcc && g == G / 2 + 1 && r + 1 < n_out) wait_acc(acc_seq + r + 1);
+                                   });
+                    if (!kEarlyAcc) {
+                        commit_row(r);
+                        if (r + 1 < n_out) wait_acc(acc_seq + r + 1);
                     }
-                    if (ok) issue_row<FP8>(tcol, acc_seq, r, n_out, arow, bd, G / 2, G);
-                    ptx::mma_commit(&empty[s]);
-                    if (r >= 4 && r - 4 < n_out) ptx::mma_commit(&afull[(acc_seq + r - 4) % C::kAcc]);
-                    if (!kEarlyAcc && r + 1 < n_in && r + 1 < n_out) {
-                        wait_acc(acc_seq + r + 1);
-                        ptx::tc_fence_after();
-                    }
+                    ptx::tc_fence_after();
                 }
+                if (kEarlyAcc) commit_row(n_in - 1);
                 in_seq += n_in;
                 acc_seq += n_out;
             }
+        if (lane == 0) {
+            const bool l2 = warp == 0;
             // drain: all of this issuer's MMAs complete before TMEM is released
             uint64_t* fin = B.fin + (l2 ? 0 : 1);
             ptx::mma_commit(fin);

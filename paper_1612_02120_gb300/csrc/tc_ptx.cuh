@@ -137,7 +137,19 @@ __device__ __forceinline__ void mma_bf16_if(uint32_t on, uint32_t d_tmem, uint32
         "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(on)
         : "memory");
 }
-// The same with the accumulate flag given (0: D is overwritten).
+__device__ __forceinline__ void mma_e4m3_if(uint32_t on, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                            uint32_t b_hi, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 q, %6, 0;\n\t"
+        "setp.eq.b32 p, 0, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(on)
+        : "memory");
+}
+// The BF16 form with the accumulate flag given (0: D is overwritten).
 __device__ __forceinline__ void mma_bf16_acc(uint32_t on, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
                                              uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
