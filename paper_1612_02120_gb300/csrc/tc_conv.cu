@@ -33,6 +33,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <chrono>
 #include <string>
 #include <vector>
@@ -101,8 +102,7 @@ struct Cfg {
     static constexpr int oR1 = oB + 2 * kLayerB;
     static constexpr int oR2 = oR1 + kRing * kSlotBytes;
     static constexpr int oIn = oR2 + kRing * kSlotBytes;
-    static constexpr int oSt1 = oIn + kInRing * kPitch * 4;
-    static constexpr int oSt2 = oSt1 + 2 * 4 * 32 * 4;
+    static constexpr int oSt2 = oIn + kInRing * kPitch * 4;
     static constexpr int oConst = oSt2 + 2 * 4 * 32 * 4;
     static constexpr int oBar = oConst + kConsts * 4;
     static constexpr int kBars = 2 * kInRing + 4 * kRing + 4 * 8 + 2;
@@ -213,100 +213,46 @@ __device__ __forceinline__ bool range_next(const TcParams& p, RangeIter& s, Item
     return true;
 }
 
-// Pack 8 consecutive channels (BF16) or 16 (E4M3) of one pixel into a 16-byte ring row.
-template <bool FP8>
-__device__ __forceinline__ void store_pixel(uint8_t* slot, int c, const float (&m)[32], const float* q) {
-    if (!FP8) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            uint4 u;
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(m[8 * k + 0], m[8 * k + 1]);
-            __nv_bfloat162 h1 = __floats2bfloat162_rn(m[8 * k + 2], m[8 * k + 3]);
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(m[8 * k + 4], m[8 * k + 5]);
-            __nv_bfloat162 h3 = __floats2bfloat162_rn(m[8 * k + 6], m[8 * k + 7]);
-            u.x = *reinterpret_cast<uint32_t*>(&h0);
-            u.y = *reinterpret_cast<uint32_t*>(&h1);
-            u.z = *reinterpret_cast<uint32_t*>(&h2);
-            u.w = *reinterpret_cast<uint32_t*>(&h3);
-            *reinterpret_cast<uint4*>(slot + (k * kPitch + c) * 16) = u;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            uint32_t w[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int ch = 16 * k + 4 * j;
-                __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(
-                    make_float2(m[ch] * q[ch], m[ch + 1] * q[ch + 1]), __NV_SATFINITE, __NV_E4M3);
-                __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(
-                    make_float2(m[ch + 2] * q[ch + 2], m[ch + 3] * q[ch + 3]), __NV_SATFINITE, __NV_E4M3);
-                w[j] = (uint32_t)lo | ((uint32_t)hi << 16);
-            }
-            *reinterpret_cast<uint4*>(slot + (k * kPitch + c) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    }
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ uint32_t max_bf16(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 v =
+        __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// Store 16 channels (one half h of the 32) of one pixel: BF16 chunks 2h and 2h+1, or E4M3 chunk h.
-template <bool FP8>
-__device__ __forceinline__ void store_half(uint8_t* slot, int c, int h, const float (&m)[16], const float* q) {
-    if (!FP8) {
+// Store the 32 channels of one pixel, scaled by q, as two E4M3 chunks.
+__device__ __forceinline__ void store_pixel_e4m3(uint8_t* slot, int c, const float (&m)[32], const float* q) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            uint4 u;
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(m[8 * k + 0], m[8 * k + 1]);
-            __nv_bfloat162 h1 = __floats2bfloat162_rn(m[8 * k + 2], m[8 * k + 3]);
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(m[8 * k + 4], m[8 * k + 5]);
-            __nv_bfloat162 h3 = __floats2bfloat162_rn(m[8 * k + 6], m[8 * k + 7]);
-            u.x = *reinterpret_cast<uint32_t*>(&h0);
-            u.y = *reinterpret_cast<uint32_t*>(&h1);
-            u.z = *reinterpret_cast<uint32_t*>(&h2);
-            u.w = *reinterpret_cast<uint32_t*>(&h3);
-            *reinterpret_cast<uint4*>(slot + ((2 * h + k) * kPitch + c) * 16) = u;
-        }
-    } else {
+    for (int k = 0; k < 2; ++k) {
         uint32_t w[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int ch = 4 * j;
+            const int ch = 16 * k + 4 * j;
             __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(make_float2(m[ch] * q[ch], m[ch + 1] * q[ch + 1]),
                                                                __NV_SATFINITE, __NV_E4M3);
             __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(
                 make_float2(m[ch + 2] * q[ch + 2], m[ch + 3] * q[ch + 3]), __NV_SATFINITE, __NV_E4M3);
             w[j] = (uint32_t)lo | ((uint32_t)hi << 16);
         }
-        *reinterpret_cast<uint4*>(slot + (h * kPitch + c) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(slot + (k * kPitch + c) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
-// Store channels 8h .. 8h+7 of one pixel: BF16 chunk h (16 B), or the half h & 1 of E4M3 chunk h >> 1.
-template <bool FP8>
-__device__ __forceinline__ void store_eighth(uint8_t* slot, int c, int h, const float (&m)[8], const float* q) {
-    if (!FP8) {
-        uint4 u;
-        __nv_bfloat162 h0 = __floats2bfloat162_rn(m[0], m[1]);
-        __nv_bfloat162 h1 = __floats2bfloat162_rn(m[2], m[3]);
-        __nv_bfloat162 h2 = __floats2bfloat162_rn(m[4], m[5]);
-        __nv_bfloat162 h3 = __floats2bfloat162_rn(m[6], m[7]);
-        u.x = *reinterpret_cast<uint32_t*>(&h0);
-        u.y = *reinterpret_cast<uint32_t*>(&h1);
-        u.z = *reinterpret_cast<uint32_t*>(&h2);
-        u.w = *reinterpret_cast<uint32_t*>(&h3);
-        *reinterpret_cast<uint4*>(slot + (h * kPitch + c) * 16) = u;
-    } else {
-        uint32_t w[2];
+// Store channels 8h .. 8h+7 of one pixel as half h & 1 of E4M3 chunk h >> 1 (layer 1 arrives already
+// scaled: the scale is folded into its weights and bias).
+__device__ __forceinline__ void store_eighth_e4m3(uint8_t* slot, int c, int h, const float (&m)[8]) {
+    uint32_t w[2];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int ch = 4 * j;
-            // (layer 1 arrives already scaled: the scale is folded into its weights and bias)
-            __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(make_float2(m[ch], m[ch + 1]), __NV_SATFINITE, __NV_E4M3);
-            __nv_fp8x2_storage_t hi =
-                __nv_cvt_float2_to_fp8x2(make_float2(m[ch + 2], m[ch + 3]), __NV_SATFINITE, __NV_E4M3);
-            w[j] = (uint32_t)lo | ((uint32_t)hi << 16);
-        }
-        *reinterpret_cast<uint2*>(slot + ((h >> 1) * kPitch + c) * 16 + (h & 1) * 8) = make_uint2(w[0], w[1]);
+    for (int j = 0; j < 2; ++j) {
+        const int ch = 4 * j;
+        __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(make_float2(m[ch], m[ch + 1]), __NV_SATFINITE, __NV_E4M3);
+        __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(make_float2(m[ch + 2], m[ch + 3]), __NV_SATFINITE, __NV_E4M3);
+        w[j] = (uint32_t)lo | ((uint32_t)hi << 16);
     }
+    *reinterpret_cast<uint2*>(slot + ((h >> 1) * kPitch + c) * 16 + (h & 1) * 8) = make_uint2(w[0], w[1]);
 }
 
 // Issue the MMAs of one input row r for one layer: output rows j = r-4+i of the layer for the valid
@@ -569,15 +515,26 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
         // ================= layer-2 epilogue: bias, ReLU, max-filter -> A ring of layer 3 =======
         const int c = tid - 128;
         const int pw = warp - 4;
-        float* stage = reinterpret_cast<float*>(smem + C::oSt2);
         uint32_t a2_seq = 0, m2_seq = 0;
-        float prev[32];
         // per-channel constants in registers (the waits are compiler barriers, so reads from shared
         // memory would repeat every row, beside the MMA operand traffic)
         // (FP8 reads its scales from shared memory: registers would not hold them as well)
         float b2[32];
 #pragma unroll
         for (int ch = 0; ch < 32; ++ch) b2[ch] = cst[kCE2B + ch];
+        // BF16 rounds first and filters packed pairs (the maxima of rounded values are the rounded
+        // maxima): half the registers, shuffles and exchanged bytes. E4M3 has no packed maximum.
+        using T = typename std::conditional<FP8, float, uint32_t>::type;
+        constexpr int NV = FP8 ? 32 : 16;
+        auto vmax = [](T x, T y) -> T {
+            if constexpr (FP8)
+                return fmaxf(x, y);
+            else
+                return max_bf16(x, y);
+        };
+        uint4* stage = reinterpret_cast<uint4*>(smem + C::oSt2);  // [2 rows in turn][4 warps][NV values]
+        T prev[NV];
+        uint32_t turn = 0;
         RangeIter range = range_begin(p);
         ItemInfo it;
         for (int k = blockIdx.x; RNG ? range_next(p, range, it) : k < p.n_items; k += gridDim.x) {
@@ -596,29 +553,59 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                 for (int ch = 0; ch < 32; ++ch)  // BF16: the scales are 1
                     v[ch] = fmaxf(FP8 ? fmaf(v[ch], cst[kCE2S + ch], b2[ch]) : v[ch] + b2[ch], 0.f);
-                if (j > 0) {
-                    float (&m)[32] = prev;  // vertical max in place; prev is reloaded from v below
+                T cur[NV];
 #pragma unroll
-                    for (int ch = 0; ch < 32; ++ch) m[ch] = fmaxf(prev[ch], v[ch]);
-                    float* st = stage + (j & 1) * 128;
+                for (int i = 0; i < NV; ++i) {
+                    if constexpr (FP8)
+                        cur[i] = v[i];
+                    else
+                        cur[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
+                }
+                if (j > 0) {
+                    T(&m)[NV] = prev;  // vertical max in place; prev is reloaded from cur below
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) m[i] = vmax(prev[i], cur[i]);
+                    // lane 31's right neighbour is the next warp's lane 0: 16-byte pieces through
+                    // shared memory
+                    uint4* st = stage + turn * 4 * (NV / 4);
+                    turn ^= 1;  // two buffers in turn, over item boundaries too
                     if (lane == 0)
 #pragma unroll
-                        for (int ch = 0; ch < 32; ++ch) st[pw * 32 + ch] = m[ch];
+                        for (int i = 0; i < NV / 4; ++i) {
+                            uint4 w;
+                            memcpy(&w, &m[4 * i], 16);
+                            st[pw * (NV / 4) + i] = w;
+                        }
                     asm volatile("bar.sync 2, 128;" ::: "memory");
+                    T nx[NV];
 #pragma unroll
-                    for (int ch = 0; ch < 32; ++ch) {
-                        float nb = __shfl_down_sync(0xffffffffu, m[ch], 1);
-                        if (lane == 31) nb = pw < 3 ? st[(pw + 1) * 32 + ch] : m[ch];
-                        m[ch] = fmaxf(m[ch], nb);
+                    for (int i = 0; i < NV / 4; ++i) {
+                        uint4 w = make_uint4(0, 0, 0, 0);
+                        if (lane == 31 && pw < 3) w = st[(pw + 1) * (NV / 4) + i];
+                        memcpy(&nx[4 * i], &w, 16);
+                    }
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) {
+                        T nb = __shfl_down_sync(0xffffffffu, m[i], 1);
+                        if (lane == 31) nb = pw < 3 ? nx[i] : m[i];
+                        m[i] = vmax(m[i], nb);
                     }
                     const uint32_t q2 = m2_seq + j - 1, s2 = q2 % kRing;
                     wait_phase(&B.m2_empty[s2], ((q2 / kRing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
-                    store_pixel<FP8>(smem + C::oR2 + s2 * C::kSlotBytes, c, m, cst + kCQ2);
+                    uint8_t* slot = smem + C::oR2 + s2 * C::kSlotBytes;
+                    if constexpr (FP8) {
+                        store_pixel_e4m3(slot, c, m, cst + kCQ2);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            *reinterpret_cast<uint4*>(slot + (i * kPitch + c) * 16) =
+                                make_uint4(m[4 * i], m[4 * i + 1], m[4 * i + 2], m[4 * i + 3]);
+                    }
                     ptx::fence_proxy_async_smem();
                     ptx::mbar_arrive(&B.m2_full[s2]);
                 }
 #pragma unroll
-                for (int ch = 0; ch < 32; ++ch) prev[ch] = v[ch];
+                for (int i = 0; i < NV; ++i) prev[i] = cur[i];
             }
             a2_seq += N2;
             m2_seq += N2 - 1;
@@ -676,7 +663,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
         const int h = warp - 12;
         const int c0 = 4 * lane;
         uint32_t in_seq = 0, m1_seq = 0;
-        float prev[4][8], cur[4][8];
+        // (BF16 rounds first and filters packed pairs, as the layer-2 epilogue)
+        using T = typename std::conditional<FP8, float, uint32_t>::type;
+        constexpr int NV = FP8 ? 8 : 4;
+        auto vmax = [](T x, T y) -> T {
+            if constexpr (FP8)
+                return fmaxf(x, y);
+            else
+                return max_bf16(x, y);
+        };
+        T prev[4][NV], cur[4][NV];
         RangeIter range = range_begin(p);
         ItemInfo it;
         for (int k = blockIdx.x; RNG ? range_next(p, range, it) : k < p.n_items; k += gridDim.x) {
@@ -739,8 +735,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
                 for (int c = 0; c < 4; ++c)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        cur[c][2 * j] = fmaxf(acc[c][j].x, 0.f);
-                        cur[c][2 * j + 1] = fmaxf(acc[c][j].y, 0.f);
+                        if constexpr (FP8) {
+                            cur[c][2 * j] = fmaxf(acc[c][j].x, 0.f);
+                            cur[c][2 * j + 1] = fmaxf(acc[c][j].y, 0.f);
+                        } else {
+                            cur[c][j] = pack_bf16(fmaxf(acc[c][j].x, 0.f), fmaxf(acc[c][j].y, 0.f));
+                        }
                     }
                 ptx::mbar_arrive(&B.in_empty[(in_seq + t + 1) % kInRing]);
                 if (t >= 0) {
@@ -748,27 +748,30 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
 #pragma unroll
-                        for (int ch = 0; ch < 8; ++ch) prev[c][ch] = fmaxf(prev[c][ch], cur[c][ch]);
+                        for (int i = 0; i < NV; ++i) prev[c][i] = vmax(prev[c][i], cur[c][i]);
                     // horizontal: column c0 + 3 pairs with the next lane's column c0 + 4; lane 31's
                     // column 127 only feeds discarded output columns and pairs with itself
                     const uint32_t q = m1_seq + t, s = q % kRing;
                     wait_phase(&B.m1_empty[s], ((q / kRing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
                     uint8_t* slot = smem + C::oR1 + s * C::kSlotBytes;
-                    float o[8];
+                    T o[NV];
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
 #pragma unroll
-                        for (int ch = 0; ch < 8; ++ch) {
-                            float nb;
+                        for (int i = 0; i < NV; ++i) {
+                            T nb;
                             if (c < 3) {
-                                nb = prev[c + 1][ch];
+                                nb = prev[c + 1][i];
                             } else {
-                                nb = __shfl_down_sync(0xffffffffu, prev[0][ch], 1);
-                                if (lane == 31) nb = prev[3][ch];
+                                nb = __shfl_down_sync(0xffffffffu, prev[0][i], 1);
+                                if (lane == 31) nb = prev[3][i];
                             }
-                            o[ch] = fmaxf(prev[c][ch], nb);
+                            o[i] = vmax(prev[c][i], nb);
                         }
-                        store_eighth<FP8>(slot, c0 + c, h, o, cst + kCQ1 + 8 * h);
+                        if constexpr (FP8)
+                            store_eighth_e4m3(slot, c0 + c, h, o);
+                        else
+                            *reinterpret_cast<uint4*>(slot + (h * kPitch + c0 + c) * 16) = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                     ptx::fence_proxy_async_smem();
                     ptx::mbar_arrive(&B.m1_full[s]);
@@ -776,7 +779,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
 #pragma unroll
-                    for (int ch = 0; ch < 8; ++ch) prev[c][ch] = cur[c][ch];
+                    for (int i = 0; i < NV; ++i) prev[c][i] = cur[c][i];
             }
             for (int u = M1 + 1; u < NR + 14; ++u) ptx::mbar_arrive(&B.in_empty[(in_seq + u) % kInRing]);
             in_seq += NR + 14;
