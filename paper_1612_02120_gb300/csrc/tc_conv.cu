@@ -33,7 +33,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <type_traits>
 #include <chrono>
 #include <string>
 #include <vector>
@@ -213,46 +212,42 @@ __device__ __forceinline__ bool range_next(const TcParams& p, RangeIter& s, Item
     return true;
 }
 
+// Filtered values are packed: BF16 pairs, or four E4M3 codes. The maxima of rounded values are the
+// rounded maxima, and after the ReLU (no sign) a code orders like an unsigned byte; its maximum is
+// taken on 16-bit lanes holding one byte each, so four codes are held as two registers ("split": the
+// even bytes, the odd bytes) and as one to move ("merged").
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
 }
-__device__ __forceinline__ uint32_t max_bf16(uint32_t a, uint32_t b) {
-    const __nv_bfloat162 v =
-        __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
-    return *reinterpret_cast<const uint32_t*>(&v);
+__device__ __forceinline__ uint32_t pack_e4m3(float a, float b, float c, float d) {
+    const __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3);
+    const __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(make_float2(c, d), __NV_SATFINITE, __NV_E4M3);
+    return (uint32_t)lo | ((uint32_t)hi << 16);
 }
-
-// Store the 32 channels of one pixel, scaled by q, as two E4M3 chunks.
-__device__ __forceinline__ void store_pixel_e4m3(uint8_t* slot, int c, const float (&m)[32], const float* q) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int ch = 16 * k + 4 * j;
-            __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(make_float2(m[ch] * q[ch], m[ch + 1] * q[ch + 1]),
-                                                               __NV_SATFINITE, __NV_E4M3);
-            __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(
-                make_float2(m[ch + 2] * q[ch + 2], m[ch + 3] * q[ch + 3]), __NV_SATFINITE, __NV_E4M3);
-            w[j] = (uint32_t)lo | ((uint32_t)hi << 16);
-        }
-        *reinterpret_cast<uint4*>(slot + (k * kPitch + c) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+template <bool FP8>
+__device__ __forceinline__ uint32_t vmax(uint32_t a, uint32_t b) {
+    if constexpr (FP8) {
+        return __vmaxu2(a, b);
+    } else {
+        const __nv_bfloat162 v =
+            __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+        return *reinterpret_cast<const uint32_t*>(&v);
     }
 }
-
-// Store channels 8h .. 8h+7 of one pixel as half h & 1 of E4M3 chunk h >> 1 (layer 1 arrives already
-// scaled: the scale is folded into its weights and bias).
-__device__ __forceinline__ void store_eighth_e4m3(uint8_t* slot, int c, int h, const float (&m)[8]) {
-    uint32_t w[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const int ch = 4 * j;
-        __nv_fp8x2_storage_t lo = __nv_cvt_float2_to_fp8x2(make_float2(m[ch], m[ch + 1]), __NV_SATFINITE, __NV_E4M3);
-        __nv_fp8x2_storage_t hi = __nv_cvt_float2_to_fp8x2(make_float2(m[ch + 2], m[ch + 3]), __NV_SATFINITE, __NV_E4M3);
-        w[j] = (uint32_t)lo | ((uint32_t)hi << 16);
+// N registers of values (BF16 pairs, or split codes: even and odd bytes in turn) <-> merged ones.
+template <bool FP8>
+__device__ __forceinline__ uint32_t merged(const uint32_t* v, int i) {
+    return FP8 ? v[2 * i] | v[2 * i + 1] : v[i];
+}
+template <bool FP8>
+__device__ __forceinline__ void max_merged(uint32_t* v, int i, uint32_t w) {
+    if constexpr (FP8) {
+        v[2 * i] = vmax<true>(v[2 * i], w & 0x00ff00ffu);
+        v[2 * i + 1] = vmax<true>(v[2 * i + 1], w & 0xff00ff00u);
+    } else {
+        v[i] = vmax<false>(v[i], w);
     }
-    *reinterpret_cast<uint2*>(slot + ((h >> 1) * kPitch + c) * 16 + (h & 1) * 8) = make_uint2(w[0], w[1]);
 }
 
 // Issue the MMAs of one input row r for one layer: output rows j = r-4+i of the layer for the valid
@@ -522,18 +517,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
         float b2[32];
 #pragma unroll
         for (int ch = 0; ch < 32; ++ch) b2[ch] = cst[kCE2B + ch];
-        // BF16 rounds first and filters packed pairs (the maxima of rounded values are the rounded
-        // maxima): half the registers, shuffles and exchanged bytes. E4M3 has no packed maximum.
-        using T = typename std::conditional<FP8, float, uint32_t>::type;
-        constexpr int NV = FP8 ? 32 : 16;
-        auto vmax = [](T x, T y) -> T {
-            if constexpr (FP8)
-                return fmaxf(x, y);
-            else
-                return max_bf16(x, y);
-        };
-        uint4* stage = reinterpret_cast<uint4*>(smem + C::oSt2);  // [2 rows in turn][4 warps][NV values]
-        T prev[NV];
+        // rounded first, filtered packed: a quarter to a half of the registers, shuffles and exchanged
+        // bytes of FP32 values
+        constexpr int NV = 16, NM = FP8 ? 8 : 16;  // registers of values, of merged values
+        uint4* stage = reinterpret_cast<uint4*>(smem + C::oSt2);  // [2 rows in turn][4 warps][NM merged values]
+        uint32_t prev[NV];
         uint32_t turn = 0;
         RangeIter range = range_begin(p);
         ItemInfo it;
@@ -553,54 +541,55 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                 for (int ch = 0; ch < 32; ++ch)  // BF16: the scales are 1
                     v[ch] = fmaxf(FP8 ? fmaf(v[ch], cst[kCE2S + ch], b2[ch]) : v[ch] + b2[ch], 0.f);
-                T cur[NV];
+                uint32_t cur[NV];
 #pragma unroll
-                for (int i = 0; i < NV; ++i) {
-                    if constexpr (FP8)
-                        cur[i] = v[i];
-                    else
-                        cur[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
+                for (int i = 0; i < 8; ++i) {
+                    if constexpr (FP8) {
+                        const float* q2c = cst + kCQ2 + 4 * i;
+                        const uint32_t w = pack_e4m3(v[4 * i] * q2c[0], v[4 * i + 1] * q2c[1], v[4 * i + 2] * q2c[2],
+                                                     v[4 * i + 3] * q2c[3]);
+                        cur[2 * i] = w & 0x007f007fu;  // (no sign bit: a code of -0 must not order as the largest)
+                        cur[2 * i + 1] = w & 0x7f007f00u;
+                    } else {
+                        cur[2 * i] = pack_bf16(v[4 * i], v[4 * i + 1]);
+                        cur[2 * i + 1] = pack_bf16(v[4 * i + 2], v[4 * i + 3]);
+                    }
                 }
                 if (j > 0) {
-                    T(&m)[NV] = prev;  // vertical max in place; prev is reloaded from cur below
+                    uint32_t(&m)[NV] = prev;  // vertical max in place; prev is reloaded from cur below
 #pragma unroll
-                    for (int i = 0; i < NV; ++i) m[i] = vmax(prev[i], cur[i]);
+                    for (int i = 0; i < NV; ++i) m[i] = vmax<FP8>(prev[i], cur[i]);
+                    uint32_t w[NM];
+#pragma unroll
+                    for (int i = 0; i < NM; ++i) w[i] = merged<FP8>(m, i);
                     // lane 31's right neighbour is the next warp's lane 0: 16-byte pieces through
                     // shared memory
-                    uint4* st = stage + turn * 4 * (NV / 4);
+                    uint4* st = stage + turn * 4 * (NM / 4);
                     turn ^= 1;  // two buffers in turn, over item boundaries too
                     if (lane == 0)
 #pragma unroll
-                        for (int i = 0; i < NV / 4; ++i) {
-                            uint4 w;
-                            memcpy(&w, &m[4 * i], 16);
-                            st[pw * (NV / 4) + i] = w;
-                        }
+                        for (int i = 0; i < NM / 4; ++i)
+                            st[pw * (NM / 4) + i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
                     asm volatile("bar.sync 2, 128;" ::: "memory");
-                    T nx[NV];
 #pragma unroll
-                    for (int i = 0; i < NV / 4; ++i) {
-                        uint4 w = make_uint4(0, 0, 0, 0);
-                        if (lane == 31 && pw < 3) w = st[(pw + 1) * (NV / 4) + i];
-                        memcpy(&nx[4 * i], &w, 16);
-                    }
+                    for (int i = 0; i < NM / 4; ++i) {
+                        uint4 e = make_uint4(0, 0, 0, 0);  // (column 127 pairs with nothing: it is discarded)
+                        if (lane == 31 && pw < 3) e = st[(pw + 1) * (NM / 4) + i];
+                        const uint32_t ee[4] = {e.x, e.y, e.z, e.w};
 #pragma unroll
-                    for (int i = 0; i < NV; ++i) {
-                        T nb = __shfl_down_sync(0xffffffffu, m[i], 1);
-                        if (lane == 31) nb = pw < 3 ? nx[i] : m[i];
-                        m[i] = vmax(m[i], nb);
+                        for (int k = 0; k < 4; ++k) {
+                            const uint32_t nb = __shfl_down_sync(0xffffffffu, w[4 * i + k], 1);
+                            max_merged<FP8>(m, 4 * i + k, lane == 31 ? ee[k] : nb);
+                        }
                     }
                     const uint32_t q2 = m2_seq + j - 1, s2 = q2 % kRing;
                     wait_phase(&B.m2_empty[s2], ((q2 / kRing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
                     uint8_t* slot = smem + C::oR2 + s2 * C::kSlotBytes;
-                    if constexpr (FP8) {
-                        store_pixel_e4m3(slot, c, m, cst + kCQ2);
-                    } else {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            *reinterpret_cast<uint4*>(slot + (i * kPitch + c) * 16) =
-                                make_uint4(m[4 * i], m[4 * i + 1], m[4 * i + 2], m[4 * i + 3]);
-                    }
+                    for (int i = 0; i < NM / 4; ++i)
+                        *reinterpret_cast<uint4*>(slot + (i * kPitch + c) * 16) =
+                            make_uint4(merged<FP8>(m, 4 * i), merged<FP8>(m, 4 * i + 1), merged<FP8>(m, 4 * i + 2),
+                                       merged<FP8>(m, 4 * i + 3));
                     ptx::fence_proxy_async_smem();
                     ptx::mbar_arrive(&B.m2_full[s2]);
                 }
@@ -663,16 +652,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
         const int h = warp - 12;
         const int c0 = 4 * lane;
         uint32_t in_seq = 0, m1_seq = 0;
-        // (BF16 rounds first and filters packed pairs, as the layer-2 epilogue)
-        using T = typename std::conditional<FP8, float, uint32_t>::type;
-        constexpr int NV = FP8 ? 8 : 4;
-        auto vmax = [](T x, T y) -> T {
-            if constexpr (FP8)
-                return fmaxf(x, y);
-            else
-                return max_bf16(x, y);
-        };
-        T prev[4][NV], cur[4][NV];
+        // (rounded first, filtered packed, as the layer-2 epilogue)
+        constexpr int NV = 4, NM = FP8 ? 2 : 4;
+        uint32_t prev[4][NV], cur[4][NV];
         RangeIter range = range_begin(p);
         ItemInfo it;
         for (int k = blockIdx.x; RNG ? range_next(p, range, it) : k < p.n_items; k += gridDim.x) {
@@ -734,12 +716,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if constexpr (FP8) {
-                            cur[c][2 * j] = fmaxf(acc[c][j].x, 0.f);
-                            cur[c][2 * j + 1] = fmaxf(acc[c][j].y, 0.f);
+                    for (int j = 0; j < 4; j += 2) {
+                        const float a0 = fmaxf(acc[c][j].x, 0.f), a1 = fmaxf(acc[c][j].y, 0.f);
+                        const float a2 = fmaxf(acc[c][j + 1].x, 0.f), a3 = fmaxf(acc[c][j + 1].y, 0.f);
+                        if constexpr (FP8) {  // already scaled: the scale is folded into layer 1's weights and bias
+                            const uint32_t w = pack_e4m3(a0, a1, a2, a3);
+                            cur[c][j] = w & 0x007f007fu;
+                            cur[c][j + 1] = w & 0x7f007f00u;
                         } else {
-                            cur[c][j] = pack_bf16(fmaxf(acc[c][j].x, 0.f), fmaxf(acc[c][j].y, 0.f));
+                            cur[c][j] = pack_bf16(a0, a1);
+                            cur[c][j + 1] = pack_bf16(a2, a3);
                         }
                     }
                 ptx::mbar_arrive(&B.in_empty[(in_seq + t + 1) % kInRing]);
@@ -748,30 +734,34 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
 #pragma unroll
-                        for (int i = 0; i < NV; ++i) prev[c][i] = vmax(prev[c][i], cur[c][i]);
+                        for (int i = 0; i < NV; ++i) prev[c][i] = vmax<FP8>(prev[c][i], cur[c][i]);
                     // horizontal: column c0 + 3 pairs with the next lane's column c0 + 4; lane 31's
                     // column 127 only feeds discarded output columns and pairs with itself
                     const uint32_t q = m1_seq + t, s = q % kRing;
                     wait_phase(&B.m1_empty[s], ((q / kRing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
                     uint8_t* slot = smem + C::oR1 + s * C::kSlotBytes;
-                    T o[NV];
+                    uint32_t right[NM];
+#pragma unroll
+                    for (int i = 0; i < NM; ++i) {
+                        right[i] = __shfl_down_sync(0xffffffffu, merged<FP8>(prev[0], i), 1);
+                        if (lane == 31) right[i] = merged<FP8>(prev[3], i);
+                    }
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
+                        if (c < 3) {
 #pragma unroll
-                        for (int i = 0; i < NV; ++i) {
-                            T nb;
-                            if (c < 3) {
-                                nb = prev[c + 1][i];
-                            } else {
-                                nb = __shfl_down_sync(0xffffffffu, prev[0][i], 1);
-                                if (lane == 31) nb = prev[3][i];
-                            }
-                            o[i] = vmax(prev[c][i], nb);
+                            for (int i = 0; i < NV; ++i) prev[c][i] = vmax<FP8>(prev[c][i], prev[c + 1][i]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < NM; ++i) max_merged<FP8>(prev[3], i, right[i]);
                         }
+                        // channels 8h .. 8h+7: BF16 chunk h, or half h & 1 of E4M3 chunk h >> 1
                         if constexpr (FP8)
-                            store_eighth_e4m3(slot, c0 + c, h, o);
+                            *reinterpret_cast<uint2*>(slot + ((h >> 1) * kPitch + c0 + c) * 16 + (h & 1) * 8) =
+                                make_uint2(merged<true>(prev[c], 0), merged<true>(prev[c], 1));
                         else
-                            *reinterpret_cast<uint4*>(slot + (h * kPitch + c0 + c) * 16) = make_uint4(o[0], o[1], o[2], o[3]);
+                            *reinterpret_cast<uint4*>(slot + (h * kPitch + c0 + c) * 16) =
+                                make_uint4(prev[c][0], prev[c][1], prev[c][2], prev[c][3]);
                     }
                     ptx::fence_proxy_async_smem();
                     ptx::mbar_arrive(&B.m1_full[s]);
