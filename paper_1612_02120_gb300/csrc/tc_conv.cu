@@ -76,6 +76,7 @@ struct TcParams {
     int64_t total_rows;     // FP8 split: strip-rows of the launch
     int fault_stall;        // test injection: the input loader withholds its arrivals
     uint64_t wait_ns;       // limit of every device-side wait
+    float4 w1[25][8];       // layer 1: [tap][channel quad]
     TcBlockDesc blk[kMaxBlocks];
 };
 
@@ -692,12 +693,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
                     const float4 xl = *reinterpret_cast<const float4*>(ir);
                     const float4 xh = *reinterpret_cast<const float4*>(ir + 4);
                     const float x[8] = {xl.x, xl.y, xl.z, xl.w, xh.x, xh.y, xh.z, xh.w};
-                    const float4* wrow = reinterpret_cast<const float4*>(cst + kCW1 + ky * 5 * 32 + 8 * h);
                     float4 w[5][2];
 #pragma unroll
                     for (int kx = 0; kx < 5; ++kx) {
-                        w[kx][0] = wrow[kx * 8];
-                        w[kx][1] = wrow[kx * 8 + 1];
+                        w[kx][0] = p.w1[ky * 5 + kx][2 * h];
+                        w[kx][1] = p.w1[ky * 5 + kx][2 * h + 1];
                     }
 #pragma unroll
                     for (int kx = 0; kx < 5; ++kx) {
@@ -917,6 +917,7 @@ mb_status tc_prepare(mb_net* net) {
             pack_layer<true>(Wp.data(), inv, pack.data() + l * layer_bytes);
         }
     }
+    memcpy(q.w1, cs.data() + kCW1, 800 * 4);
     if (!S->d_wpack) MB_TRY(dev_alloc((void**)&S->d_wpack, kWpackConstOff + kConsts * 4));
     if (!S->h_err) {
         if (fault_oom()) {
