@@ -755,13 +755,34 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                             for (int i = 0; i < NM; ++i) max_merged<FP8>(prev[3], i, right[i]);
                         }
+                    }
+                    // A lane's four columns are 64 B from its neighbours': stored in the same order by
+                    // all lanes, 16 lanes meet in each bank. Lane l starts with its column (l / 2) mod 4
+                    // instead (the order is rotated in registers, two conditional steps).
+                    uint32_t w[4][NM];
+                    const int turn = (lane >> 1) & 3;
+#pragma unroll
+                    for (int i = 0; i < NM; ++i) {
+                        uint32_t a[4];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) a[c] = merged<FP8>(prev[c], i);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) w[c][i] = (turn & 1) ? a[(c + 1) & 3] : a[c];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) a[c] = w[c][i];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) w[c][i] = (turn & 2) ? a[(c + 2) & 3] : a[c];
+                    }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const int col = c0 + ((c + turn) & 3);
                         // channels 8h .. 8h+7: BF16 chunk h, or half h & 1 of E4M3 chunk h >> 1
                         if constexpr (FP8)
-                            *reinterpret_cast<uint2*>(slot + ((h >> 1) * kPitch + c0 + c) * 16 + (h & 1) * 8) =
-                                make_uint2(merged<true>(prev[c], 0), merged<true>(prev[c], 1));
+                            *reinterpret_cast<uint2*>(slot + ((h >> 1) * kPitch + col) * 16 + (h & 1) * 8) =
+                                make_uint2(w[c][0], w[c][1]);
                         else
-                            *reinterpret_cast<uint4*>(slot + (h * kPitch + c0 + c) * 16) =
-                                make_uint4(prev[c][0], prev[c][1], prev[c][2], prev[c][3]);
+                            *reinterpret_cast<uint4*>(slot + (h * kPitch + col) * 16) =
+                                make_uint4(w[c][0], w[c][1], w[c][2], w[c][3]);
                     }
                     ptx::fence_proxy_async_smem();
                     ptx::mbar_arrive(&B.m1_full[s]);
