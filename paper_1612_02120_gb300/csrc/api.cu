@@ -530,6 +530,7 @@ mb_status mb_net_destroy(mb_net* net) {
         me_tc_release(net);
         st_tc_release(net);
         x3_release(net);
+        if (net->train_host) cudaFreeHost(net->train_host);
         dev_free(net->d_params);
         dev_free(net->d_simt);
         dev_free(net->d_queue);

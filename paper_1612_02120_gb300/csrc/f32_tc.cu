@@ -43,14 +43,13 @@
 #include <new>
 #include <vector>
 
+#include "f32_split.cuh"
 #include "internal.h"
-#include "tc_ptx.cuh"
 
 namespace mb {
 
 namespace {
 
-constexpr uint64_t kXWaitNs = 4000000000ull;
 enum { X_RELU = 0, X_HEAD = 1, X_MAXOUT = 2 };
 
 template <int K, int OUT>
@@ -98,31 +97,6 @@ struct XParams {
     uint64_t wait_ns;
 };
 
-__device__ __forceinline__ uint64_t gtime() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err,
-                                         uint64_t limit_ns) {
-    if (ptx::mbar_test(bar, parity)) return true;
-    if (*abort_flag) return false;
-    const uint64_t t0 = gtime();
-    uint32_t n = 0;
-    while (!ptx::mbar_test(bar, parity)) {
-        if ((++n & 255u) == 0) {
-            if (*abort_flag) return false;
-            if (gtime() - t0 > limit_ns) {
-                *abort_flag = 1;
-                *(volatile int*)err = MB_ERR_TIMEOUT;
-                return false;
-            }
-        }
-    }
-    return true;
-}
-
 struct XItem {
     int z, ry, x0, m0, rows;  // conv rows y = ry + d (m0 + j), j < rows
 };
@@ -159,14 +133,6 @@ __device__ __forceinline__ bool x_next(const XParams& p, XCursor& c, XItem& it) 
 
 __device__ __forceinline__ float4 max4(float4 a, float4 b) {
     return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), fmaxf(a.w, b.w));
-}
-
-// The leading 8 significant bits of two floats as a BF16 pair; the floats keep what is left (exact).
-__device__ __forceinline__ uint32_t take_part(float& a, float& b) {
-    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
-    a -= __uint_as_float(ua & 0xffff0000u);
-    b -= __uint_as_float(ub & 0xffff0000u);
-    return __byte_perm(ua, ub, 0x7632);
 }
 
 template <int K, int OUT>
@@ -231,8 +197,8 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
             uint32_t q = 0;
             bool ok = true;
             auto wait_row = [&](uint32_t r) {
-                ok = ok && wait_bar(&row_full[r % C::kRing], (r / C::kRing) & 1, abort_flag, p.err, p.wait_ns);
-                ok = ok && wait_bar(&acc_free[r % C::kBufs], ((r / C::kBufs) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
+                ok = ok && x_wait(&row_full[r % C::kRing], (r / C::kRing) & 1, abort_flag, p.err, p.wait_ns);
+                ok = ok && x_wait(&acc_free[r % C::kBufs], ((r / C::kBufs) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
             };
             auto commit_row = [&](uint32_t r) {
                 ptx::mma_commit_if(lead, &row_empty[r % C::kRing]);
@@ -267,16 +233,7 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
                 }
                 commit_row(q - 1);
             }
-            if (lane == 0) {
-                ptx::mma_commit(fin);
-                const uint64_t t0 = gtime();
-                while (!ptx::mbar_test(fin, 0)) {
-                    if (gtime() - t0 > p.wait_ns) {
-                        *(volatile int*)p.err = MB_ERR_TIMEOUT;
-                        break;
-                    }
-                }
-            }
+            if (lane == 0) x_drain(fin, p.err, p.wait_ns);
             __syncwarp();
         }
     } else if (warp < 12) {
@@ -298,7 +255,7 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
                 for (int c = 0; c < 16; ++c) sum[k][c] = 0.f;
             for (int u = 0; u < nst; ++u, ++q) {
                 const uint32_t bf = q % C::kBufs;
-                wait_bar(&acc_full[bf], (q / C::kBufs) & 1, abort_flag, p.err, p.wait_ns);
+                x_wait(&acc_full[bf], (q / C::kBufs) & 1, abort_flag, p.err, p.wait_ns);
                 ptx::tc_fence_after();
                 const uint32_t ta = tbase + lanes + bf * C::kN + 16u * g;
                 float done[16];
@@ -407,7 +364,7 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
                         }
                     }
                 }
-                wait_bar(&row_empty[s], ((q / C::kRing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
+                x_wait(&row_empty[s], ((q / C::kRing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
                 uint8_t* dst = smem + C::oRing + s * C::kSlot;
 #pragma unroll
                 for (int i = 0; i < kTasks; ++i) {

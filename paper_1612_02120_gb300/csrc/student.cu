@@ -28,12 +28,10 @@
 
 #include "internal.h"
 #include "simt_conv.cuh"
+#include "student_x3.h"
 
 namespace mb {
 
-// Parameter offsets (API layout): W1[16][1][3][3] b1[16] W2[16][16][3][3] b2[16] Wh[16] bh.
-constexpr int kSW1 = 0, kSB1 = 144, kSW2 = 160, kSB2 = 2464, kSWH = 2480, kSBH = 2496, kSN = 2497;
-// Forward (SIMT) layout: W1t[1][3][3][16] b1 | W2t[16][3][3][16] b2 | Wh bh  (same block offsets)
 // Backward data layout: W2f[co][ky][kx][ci] = W2[co][ci][2-ky][2-kx]  (2304 floats)
 constexpr int kGridHead = 1184;   // 8 x 148: fixed grids make the partial sums reproducible
 constexpr int kGridG2 = 592;
@@ -293,11 +291,14 @@ __global__ void reduce_partials(const float* partial, int ncta, int width, int c
 
 __device__ __forceinline__ float fwd_round(float v, int bf16) { return bf16 ? __bfloat162float(__float2bfloat16_rn(v)) : v; }
 
-// Forward and backward-data layouts from the master weights.
-__global__ void student_pack(const float* master, float* fwd, float* w2f, int bf16) {
+// Forward and backward-data layouts from the master weights, and (x3) the B operands of the tensor-core
+// passes: per column tap kx blocks [chunk of 8 inputs][144 rows][8 BF16], row 48 part + 16 row tap +
+// output channel, parts 0..2 the leading, middle and trailing 8 significant bits of a weight. Forward:
+// outputs co, inputs ci; backward (at x3 + kX3StudentPack): outputs ci, inputs co, taps flipped.
+__global__ void student_pack(const float* master, float* fwd, float* w2f, int bf16, uint8_t* x3) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kSN) return;
-    const float v = fwd_round(master[i], bf16);
+    float v = fwd_round(master[i], bf16);
     if (i < kSB1) {  // W1[co][0][ky][kx] -> W1t[tap][co]
         const int co = i / 9, tap = i % 9;
         fwd[tap * 16 + co] = v;
@@ -307,6 +308,17 @@ __global__ void student_pack(const float* master, float* fwd, float* w2f, int bf
         const int j = i - kSW2, co = j / 144, ci = (j / 9) % 16, tap = j % 9, ky = tap / 3, kx = tap % 3;
         fwd[kSW2 + (ci * 9 + tap) * 16 + co] = v;
         w2f[(co * 9 + (2 - ky) * 3 + (2 - kx)) * 16 + ci] = v;
+        if (!x3) return;
+        uint8_t* bwd = x3 + kX3StudentPack;
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+            const uint32_t u = __float_as_uint(v) & 0xffff0000u;
+            v -= __uint_as_float(u);
+            const uint16_t h = (uint16_t)(u >> 16);
+            *reinterpret_cast<uint16_t*>(x3 + ((kx * 2 + (ci >> 3)) * 144 + 48 * part + 16 * ky + co) * 16 + 2 * (ci & 7)) = h;
+            *reinterpret_cast<uint16_t*>(bwd + (((2 - kx) * 2 + (co >> 3)) * 144 + 48 * part + 16 * (2 - ky) + ci) * 16 +
+                                         2 * (co & 7)) = h;
+        }
     } else {
         fwd[i] = v;
     }
@@ -365,21 +377,69 @@ struct StudentBufs {
     float* v = nullptr;
     int* zmap = nullptr;
     float* losses = nullptr;
+    // tensor-core pass (null where the CUDA-core kernels run)
+    uint16_t* mask = nullptr;  // [B][H+2][W+2]
+    uint8_t* x3 = nullptr;     // B operands
 };
 
-static size_t part_floats() {
+static size_t part_floats(bool x3) {
+    if (x3) return (size_t)kX3Grid * (kX3FwdWidth + 160) + (size_t)kX3GridG2 * 2304;
     return std::max<size_t>({(size_t)kGridHead * 18, (size_t)kGridG2 * 2320, (size_t)kGridG1 * 160});
+}
+
+// Whether the training passes may run on the tensor cores: their three-part split needs finite values
+// with room for the sums, so every weight must stay below 2^30 (activations then below 2^70). `drift`
+// bounds how far a run can move a weight.
+static bool train_bounded(const float* params, double drift) {
+    for (int i = 0; i < kSN; ++i)
+        if (!((double)std::fabs(params[i]) + drift < 1073741824.0)) return false;
+    return true;
+}
+
+// A bound on sum |dw| of `steps` Adam steps: |m_t| <= c sqrt(v_t) for the moments (Cauchy-Schwarz over
+// their geometric weights, r = beta1^2 / beta2 < 1) with c = (1 - beta1) / sqrt((1 - beta2)(1 - r)), and
+// the bias corrections raise |m_t / c1| / sqrt(v_t / c2) by at most sqrt(c2) / c1 <= 1 / (1 - beta1). The
+// centred layer 1 moves its biases by up to half of nine weight steps more.
+static double adam_drift(const mb_train_cfg* c) {
+    const double b1 = c->beta1, b2 = c->beta2;
+    if (!(b1 >= 0 && b1 < 1 && b2 > 0 && b2 < 1 && b1 * b1 < b2 && std::isfinite(c->lr) && c->eps >= 0)) return INFINITY;
+    const double bound = 1.0 / std::sqrt((1 - b2) * (1 - b1 * b1 / b2));
+    return 5.5 * std::fabs((double)c->lr) * bound * c->steps;
+}
+
+static mb_status train_words(mb_net* s) {
+    if (s->train_host) return MB_OK;
+    if (fault_oom()) {
+        set_error("pinned allocation failed (MB_FAULT_OOM injected)");
+        return MB_ERR_OOM;
+    }
+    MB_CUDA(cudaHostAlloc((void**)&s->train_host, 2 * sizeof(int), cudaHostAllocMapped));
+    s->train_host[0] = s->train_host[1] = 0;
+    MB_CUDA(cudaHostGetDevicePointer((void**)&s->train_dev, s->train_host, 0));
+    return MB_OK;
+}
+
+// The error word after a synchronisation.
+static mb_status train_error(mb_net* s) {
+    if (s->train_host && *(volatile int*)s->train_host) {
+        *(volatile int*)s->train_host = 0;
+        set_error("a training launch gave up waiting (device-side wait limit)");
+        return MB_ERR_TIMEOUT;
+    }
+    return MB_OK;
 }
 
 // Carves the training workspace; every sub-buffer starts on a 256-byte boundary (the convolution
 // kernels read weights and activations as float4).
-static mb_status ensure_bufs(mb_net* s, int64_t B, int64_t H, int64_t W, int64_t steps, StudentBufs& b) {
+static mb_status ensure_bufs(mb_net* s, int64_t B, int64_t H, int64_t W, int64_t steps, bool x3, StudentBufs& b) {
     auto up = [](size_t n) { return (n + 63) & ~(size_t)63; };  // floats, rounded to 256 bytes
     const size_t nst = (size_t)std::max<int64_t>(steps, 1);
     const size_t f_h1 = up((size_t)B * (H + 2) * (W + 2) * 16), f_h2 = up((size_t)B * H * W * 16);
-    const size_t f_part = up(part_floats()), f_grad = up(kSN), f_w2f = up(2304), f_zero = up(16), f_m = up(kSN),
+    const size_t f_part = up(part_floats(x3)), f_grad = up(kSN), f_w2f = up(2304), f_zero = up(16), f_m = up(kSN),
                  f_v = up(kSN), f_loss = up(nst), f_zmap = up(nst * (size_t)B);
-    const size_t floats = f_h1 + f_h2 + f_part + f_grad + f_w2f + f_zero + f_m + f_v + f_loss + f_zmap;
+    const size_t f_mask = x3 ? up(((size_t)B * (H + 2) * (W + 2) + 1) / 2) : 0, f_x3 = x3 ? up(2 * kX3StudentPack / 4) : 0;
+    const size_t floats = f_h1 + f_h2 + f_part + f_grad + f_w2f + f_zero + f_m + f_v + f_loss + f_zmap + f_mask + f_x3;
+    if (x3) MB_TRY(train_words(s));
     MB_TRY(s->ws2.ensure(floats * 4));
     float* p = static_cast<float*>(s->ws2.ptr);
     b.h1 = p;
@@ -401,6 +461,11 @@ static mb_status ensure_bufs(mb_net* s, int64_t B, int64_t H, int64_t W, int64_t
     b.losses = p;
     p += f_loss;
     b.zmap = reinterpret_cast<int*>(p);
+    p += f_zmap;
+    if (x3) {
+        b.mask = reinterpret_cast<uint16_t*>(p);
+        b.x3 = reinterpret_cast<uint8_t*>(p + f_mask);
+    }
     return MB_OK;
 }
 
@@ -410,6 +475,28 @@ static mb_status batch_grad(mb_net* s, const uint8_t* in, const float* tgt, cons
                             int64_t W, StudentBufs& b, float* loss_dev, cudaStream_t st) {
     const float* fwd = s->d_simt;
     const float inv_n = (float)(1.0 / ((double)B * H * W));
+    if (b.x3) {
+        StudentX3 a{};
+        a.in = in;
+        a.target = tgt;
+        a.zmap = zmap;
+        a.B = (int)B;
+        a.H = (int)H;
+        a.W = (int)W;
+        a.fw = fwd;
+        a.h1 = b.h1;
+        a.mask = b.mask;
+        a.dy2 = b.h2;
+        a.pack = b.x3;
+        a.part_fwd = b.part;
+        a.part_bwd = a.part_fwd + (size_t)kX3Grid * kX3FwdWidth;
+        a.part_g2 = a.part_bwd + (size_t)kX3Grid * 160;
+        a.inv_n = inv_n;
+        a.grad = b.grad;
+        a.loss = loss_dev;
+        a.err = s->train_dev;
+        return student_x3_grad(a, st);
+    }
     // forward layer 1 -> h1, layer 2 -> h2 (post-ReLU)
     ConvArgs a{};
     a.in = in;
@@ -483,8 +570,8 @@ static mb_status batch_grad(mb_net* s, const uint8_t* in, const float* tgt, cons
 }
 
 static mb_status pack_forward(mb_net* s, StudentBufs& b, cudaStream_t st) {
-    MB_CUDA(cudaMemsetAsync(b.zero, 0, 16 * sizeof(float), st));
-    student_pack<<<(kSN + 255) / 256, 256, 0, st>>>(s->d_params, s->d_simt, b.w2f, s->prec == MB_PREC_BF16);
+    if (!b.x3) MB_CUDA(cudaMemsetAsync(b.zero, 0, 16 * sizeof(float), st));
+    student_pack<<<(kSN + 255) / 256, 256, 0, st>>>(s->d_params, s->d_simt, b.w2f, s->prec == MB_PREC_BF16, b.x3);
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;
@@ -493,8 +580,17 @@ static mb_status pack_forward(mb_net* s, StudentBufs& b, cudaStream_t st) {
 mb_status student_loss_grad(mb_net* s, const uint8_t* in, const float* tgt, int64_t n, int64_t h, int64_t w,
                             double* loss, float* grad, cudaStream_t st) {
     StudentBufs b;
-    MB_TRY(ensure_bufs(s, n, h, w, 1, b));
+    const bool x3 = train_bounded(s->host_params.data(), 0.0);
+    MB_TRY(ensure_bufs(s, n, h, w, 1, x3, b));
     MB_TRY(pack_forward(s, b, st));
+    if (x3) {  // straight into the caller's gradient; the loss through the mapped word
+        b.grad = grad;
+        MB_TRY(batch_grad(s, in, tgt, nullptr, n, h, w, b, reinterpret_cast<float*>(s->train_dev + 1), st));
+        MB_CUDA(cudaStreamSynchronize(st));
+        MB_TRY(train_error(s));
+        *loss = *reinterpret_cast<volatile float*>(s->train_host + 1);
+        return MB_OK;
+    }
     MB_TRY(batch_grad(s, in, tgt, nullptr, n, h, w, b, b.losses, st));
     MB_CUDA(cudaMemcpyAsync(grad, b.grad, kSN * sizeof(float), cudaMemcpyDeviceToDevice, st));
     float lh = 0.f;
@@ -565,8 +661,6 @@ static CkptRead read_ckpt(const char* path, CkptHeader& hd, std::vector<float>& 
 mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t n, int64_t h, int64_t w,
                         const mb_train_cfg* cfg, const char* ckpt, float* curve, cudaStream_t st) {
     const int64_t B = cfg->batch;
-    StudentBufs b;
-    MB_TRY(ensure_bufs(s, B, h, w, cfg->steps, b));
     CkptHeader hd;
     memset(&hd, 0, sizeof(hd));
     memcpy(hd.magic, "MBCKPT02", 8);
@@ -587,6 +681,11 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
             set_error("checkpoint %s does not match this run (seed or step count)", ckpt);
             return MB_ERR_INVALID_ARG;
         }
+    }
+    const bool x3 = train_bounded(found == CkptRead::kOk ? buf.data() : s->host_params.data(), adam_drift(cfg));
+    StudentBufs b;
+    MB_TRY(ensure_bufs(s, B, h, w, cfg->steps, x3, b));
+    if (found == CkptRead::kOk) {
         start = hd.step;
         MB_CUDA(cudaMemcpyAsync(s->d_params, buf.data(), kSN * 4, cudaMemcpyHostToDevice, st));
         MB_CUDA(cudaMemcpyAsync(b.m, buf.data() + kSN, kSN * 4, cudaMemcpyHostToDevice, st));
@@ -630,7 +729,7 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
     MB_CUDA(cudaStreamSynchronize(st));
     // the host master copy follows the device
     MB_CUDA(cudaMemcpy(s->host_params.data(), s->d_params, kSN * 4, cudaMemcpyDeviceToHost));
-    return MB_OK;
+    return train_error(s);
 }
 
 // ---- cascade -------------------------------------------------------------------------------------

@@ -1,0 +1,753 @@
+// student_x3.cu - the student's training convolutions on the tensor cores with FP32 accuracy, each fused
+// with what follows it: conv2 + ReLU + head + loss + dL/dy2 (st_x3<false>) and the data gradient +
+// ReLU mask + conv1's weight gradient (st_x3<true>); the first convolution (st_conv1) and conv2's weight
+// gradient (st_grad2) on packed FP32 FMAs.
+//
+// Numbers: the three-part BF16 split of f32_tc.cu (six of nine products, error below an FMA chain's).
+// With 16 channels the products of equal weight sit in columns of their own: part 1 of an input row
+// is multiplied by [w1 | w2 | w3] (N = 144: 3 parts x 3 row taps x 16), part 2 by [w1 | w2] into the
+// second and third column groups, part 3 by w1 into the third; the epilogue adds g1 + (g2 + g3) per row
+// tap and sums the row taps in FP32.
+//
+// st_x3 reads one 64-byte pixel of h1 or dy2 per output pixel, once, and the forward writes dy2 once
+// (h2 and dy1 exist in registers only): 128 px rows cost ~500 cycles of MMAs and 360-710 of HBM time.
+// The separate kernels (conv 865 us, head and loss 218, data gradient 1,023, conv1's weight gradient
+// 395 on a batch of 32 x 512 x 512) passed 3.2 GB through HBM at 0.47-0.55 of the FP32 FMA rate.
+//
+// Warp roles of st_x3 (512 threads, 1 CTA per SM, one equal contiguous range of strip-rows per CTA):
+//   warp 0        lane 0 issues the MMAs
+//   warps 4-11    epilogue, two groups of 8 channels, one pixel column per thread; sums over pixels
+//                 (loss, head, bias and conv1 weight gradients) stay in registers until the end
+//   warps 12-15   producers: load 8 channels of a pixel, split, store 3 x 16 B
+// The grids are fixed, so the partial sums, and with them a training run, are reproducible.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "f32_split.cuh"
+#include "internal.h"
+#include "student_x3.h"
+
+namespace mb {
+
+namespace {
+
+constexpr int kThreadsX = 512;
+constexpr int kP = 130;                       // pixels per staged row (2 mod 8: chunk planes on distinct banks)
+constexpr int kPart = 2 * kP * 16;            // one BF16 part of a staged row: [2 chunks][kP][16 B]
+constexpr int kSlotX = 3 * kPart;
+constexpr int kRingX = 6;
+constexpr int kNx = 144;                      // columns per accumulator: 3 weight groups x 3 row taps x 16
+constexpr int kBufsX = 3;
+constexpr int oBx = 0;
+constexpr int oRingX = oBx + kX3StudentPack;
+constexpr int oLut = oRingX + kRingX * kSlotX;    // u / 255 (backward)
+constexpr int oXch = oLut + 256 * 4;              // partial head sums: 2 rows in turn x 2 groups x 128
+constexpr int oRed = oXch + 2 * 2 * 128 * 4;      // [8 warps][80] partial sums at the end
+constexpr int oBarX = oRed + 8 * 80 * 4;
+constexpr int kBarsX = 2 * kRingX + 2 * kBufsX + 1;
+constexpr int oMiscX = oBarX + kBarsX * 8;
+constexpr int kSmemX = oMiscX + 16;
+static_assert(kSmemX <= 227 * 1024 && kBufsX * kNx <= 512, "resources");
+
+struct SxParams {
+    const float* in;       // h1 [B][H+2][W+2][16], or dy2 [B][H][W][16] read as zero-padded by 2
+    const uint8_t* wpack;  // student_pack's B operand of this pass: per column tap kx [2 chunks][144 rows][16 B]
+    const float* fw;       // forward parameters (b2, head)
+    int B, H, W;
+    // forward
+    const float* target;
+    const int* zmap;
+    float* dy2;
+    float inv_n;
+    // backward
+    const uint16_t* mask;  // h1 > 0 per channel, [B][H+2][W+2]
+    const uint8_t* img;    // [slices][H][W]
+    float* partial;
+    int64_t total_rows;
+    int n_strips, out_h, out_w;
+    int* err;
+    int fault_stall;
+    uint64_t wait_ns;
+};
+
+struct SxItem {
+    int z, x0, y0, rows;
+};
+
+__device__ __forceinline__ bool sx_next(const SxParams& p, int64_t& g, int64_t hi, SxItem& it) {
+    if (g >= hi) return false;
+    const int64_t col = g / p.out_h;
+    it.y0 = (int)(g - col * p.out_h);
+    it.z = (int)(col / p.n_strips);
+    it.x0 = (int)(col % p.n_strips) * 128;
+    it.rows = (int)min((int64_t)(p.out_h - it.y0), hi - g);
+    g += it.rows;
+    return true;
+}
+
+__device__ __forceinline__ int sx_refl(int t, int n) {
+    t = t < 0 ? -t : t;
+    t = t >= n ? 2 * (n - 1) - t : t;
+    return min(max(t, 0), n - 1);  // columns past the strip's domain feed nothing that counts
+}
+
+// Sums of N values over the 128 threads of an epilogue group, in a fixed order; valid in the group's
+// first warp's lane 0 order: out[i] written by thread i of the group.
+template <int N>
+__device__ __forceinline__ void group_sum(const float (&v)[N], float* red, int group, int warp_in, int lane, float* out) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        float s = v[i];
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+        if (lane == 0) red[(group * 4 + warp_in) * 80 + i] = s;
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(3 + group) : "memory");
+    const int t = warp_in * 32 + lane;
+    if (t < N) {
+        const float* r = red + group * 4 * 80 + t;
+        out[t] = (r[0] + r[80]) + (r[160] + r[240]);
+    }
+}
+
+template <bool BWD>
+__global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ SxParams p) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint64_t* row_full = reinterpret_cast<uint64_t*>(smem + oBarX);
+    uint64_t* row_empty = row_full + kRingX;
+    uint64_t* acc_full = row_empty + kRingX;
+    uint64_t* acc_free = acc_full + kBufsX;
+    uint64_t* fin = acc_free + kBufsX;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + oMiscX);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + oMiscX + 4);
+    float* lut = reinterpret_cast<float*>(smem + oLut);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+
+    if (tid == 0) {
+        for (int i = 0; i < kRingX; ++i) {
+            ptx::mbar_init(&row_full[i], 128);
+            ptx::mbar_init(&row_empty[i], 1);
+        }
+        for (int i = 0; i < kBufsX; ++i) {
+            ptx::mbar_init(&acc_full[i], 1);
+            ptx::mbar_init(&acc_free[i], 256);
+        }
+        ptx::mbar_init(fin, 1);
+        *abort_flag = 0;
+        ptx::mbar_fence_init();
+    }
+    {
+        const uint4* src = reinterpret_cast<const uint4*>(p.wpack);
+        uint4* dst = reinterpret_cast<uint4*>(smem + oBx);
+        for (int i = tid; i < kX3StudentPack / 16; i += kThreadsX) dst[i] = __ldg(src + i);
+        if (tid < 256) lut[tid] = (float)tid / 255.0f;
+    }
+    if (warp == 0) {
+        ptx::tmem_alloc(tmem_slot, 512);
+        ptx::tmem_relinquish();
+    }
+    ptx::fence_proxy_async_smem();
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    const uint32_t tbase = *tmem_slot;
+    const uint32_t sbase = ptx::smem_u32(smem);
+    int64_t pos = p.total_rows * (int64_t)blockIdx.x / gridDim.x;
+    const int64_t end = p.total_rows * (int64_t)(blockIdx.x + 1) / gridDim.x;
+    SxItem it;
+    static_assert(40 + 2 * 176 + 120 <= 4 * 128, "register budget exceeds the launch allocation");
+
+    if (warp < 4) {
+        ptx::setmaxnreg_dec<40>();
+        if (warp == 0) {
+            // ================= MMA issuer ============================================================
+            const uint64_t adesc = ptx::smem_desc(sbase + oRingX, kP * 16, 128);
+            const uint64_t bdesc = ptx::smem_desc(sbase + oBx, kNx * 16, 128);
+            const uint32_t a_hi = (uint32_t)(adesc >> 32), b_hi = (uint32_t)(bdesc >> 32);
+            const uint32_t lead = lane == 0;
+            uint32_t q = 0;
+            bool ok = true;
+            auto wait_row = [&](uint32_t r) {
+                ok = ok && x_wait(&row_full[r % kRingX], (r / kRingX) & 1, abort_flag, p.err, p.wait_ns);
+                ok = ok && x_wait(&acc_free[r % kBufsX], ((r / kBufsX) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
+            };
+            auto commit_row = [&](uint32_t r) {
+                ptx::mma_commit_if(lead, &row_empty[r % kRingX]);
+                ptx::mma_commit_if(lead, &acc_full[r % kBufsX]);
+            };
+            while (sx_next(p, pos, end, it)) {
+                const int nst = it.rows + 2;
+                wait_row(q);
+                for (int u = 0; u < nst; ++u, ++q) {
+                    ptx::tc_fence_after();
+                    const uint32_t on = ok ? lead : 0u, d = tbase + (q % kBufsX) * kNx;
+                    const uint32_t a = (uint32_t)adesc + (((q % kRingX) * kSlotX) >> 4);
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) {
+                        const uint32_t b = (uint32_t)bdesc + ((kx * 2 * kNx * 16) >> 4);
+                        ptx::mma_bf16_acc(on, d, a + kx, a_hi, b, b_hi, ptx::idesc_f32acc(ptx::kFmtBF16, 128, 144),
+                                          kx > 0 ? 1u : 0u);
+                        ptx::mma_bf16_if(on, d + 48, a + (kPart >> 4) + kx, a_hi, b, b_hi,
+                                         ptx::idesc_f32acc(ptx::kFmtBF16, 128, 96));
+                        ptx::mma_bf16_if(on, d + 96, a + (2 * kPart >> 4) + kx, a_hi, b, b_hi,
+                                         ptx::idesc_f32acc(ptx::kFmtBF16, 128, 48));
+                        if (kx == 0 && u > 0) commit_row(q - 1);
+                        if (kx == 1 && u + 1 < nst) wait_row(q + 1);
+                    }
+                }
+                commit_row(q - 1);
+            }
+            if (lane == 0) x_drain(fin, p.err, p.wait_ns);
+            __syncwarp();
+        }
+    } else if (warp < 12) {
+        ptx::setmaxnreg_inc<176>();
+        // ================= epilogue ===================================================================
+        const int px = tid & 127, g = (warp - 4) >> 2;  // channels 8 g .. 8 g + 7
+        const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
+        float* xch = reinterpret_cast<float*>(smem + oXch);
+        float* red = reinterpret_cast<float*>(smem + oRed);
+        uint32_t q = 0, turn = 0;
+        float s0[8], s1[8];  // conv rows u, u - 1 so far
+        // one staged row's contributions: the completed conv row u - 2 in `done`
+        auto row = [&](float (&done)[8]) {
+            const uint32_t bf = q % kBufsX;
+            x_wait(&acc_full[bf], (q / kBufsX) & 1, abort_flag, p.err, p.wait_ns);
+            ptx::tc_fence_after();
+            const uint32_t ta = tbase + lanes + bf * kNx + 8u * g;
+            float v[3][3][8];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int m = 0; m < 3; ++m) ptx::tmem_ld8_nowait(ta + (uint32_t)(48 * m + 16 * k), v[k][m]);
+            ptx::tmem_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int m = 0; m < 3; ++m) ptx::keep8(v[k][m]);
+            ptx::tc_fence_before();
+            ptx::mbar_arrive(&acc_free[bf]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                done[c] = s1[c] + (v[2][0][c] + (v[2][1][c] + v[2][2][c]));
+                s1[c] = s0[c] + (v[1][0][c] + (v[1][1][c] + v[1][2][c]));
+                s0[c] = v[0][0][c] + (v[0][1][c] + v[0][2][c]);
+            }
+        };
+        if constexpr (!BWD) {
+            float b2[8], hw[8], gw[8], db[8], loss = 0.f, gb = 0.f;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                b2[c] = __ldg(p.fw + kSB2 + 8 * g + c);
+                hw[c] = __ldg(p.fw + kSWH + 8 * g + c);
+                gw[c] = db[c] = 0.f;
+            }
+            const float hb = __ldg(p.fw + kSBH);
+            while (sx_next(p, pos, end, it)) {
+                const int nst = it.rows + 2, x = it.x0 + px;
+                const bool col_ok = x < p.W;
+                const int64_t pix0 = ((int64_t)it.z * p.H + it.y0) * p.W + x;  // conv row 0 of the item
+                const float* trow = p.target + ((int64_t)(p.zmap ? p.zmap[it.z] : it.z) * p.H + it.y0) * p.W + x;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) s0[c] = s1[c] = 0.f;
+                float t = 0.f;
+                for (int u = 0; u < nst; ++u, ++q) {
+                    const float t_next = col_ok && u >= 1 && u + 1 < nst ? __ldg(trow + (int64_t)(u - 1) * p.W) : 0.f;
+                    float h2[8];
+                    row(h2);
+                    if (u >= 2) {
+                        float z = 0.f;
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            h2[c] = fmaxf(h2[c] + b2[c], 0.f);
+                            z = fmaf(hw[c], h2[c], z);
+                        }
+                        // the groups' halves of the head sum meet; two buffers in turn, so that one
+                        // rendezvous per row keeps a row's readers from the next but one's writers
+                        float* xc = xch + turn * 256;
+                        turn ^= 1;
+                        xc[g * 128 + px] = z;
+                        asm volatile("bar.sync 2, 256;" ::: "memory");
+                        z = (xc[px] + xc[128 + px]) + hb;
+                        const float pr = 1.0f / (1.0f + expf(-z));
+                        const float e = pr - t;
+                        const float dz = col_ok ? 2.0f * p.inv_n * e * pr * (1.0f - pr) : 0.f;
+                        if (g == 0 && col_ok) {
+                            loss = fmaf(e, e, loss);
+                            gb += dz;
+                        }
+                        float dy[8];
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            gw[c] = fmaf(dz, h2[c], gw[c]);
+                            dy[c] = h2[c] > 0.f ? dz * hw[c] : 0.f;
+                            db[c] += dy[c];
+                        }
+                        if (col_ok && !*abort_flag) {
+                            float4* o = reinterpret_cast<float4*>(p.dy2 + (pix0 + (int64_t)(u - 2) * p.W) * 16 + 8 * g);
+                            o[0] = make_float4(dy[0], dy[1], dy[2], dy[3]);
+                            o[1] = make_float4(dy[4], dy[5], dy[6], dy[7]);
+                        }
+                    }
+                    t = t_next;
+                }
+            }
+            // partials per CTA: [loss, db2[16], dWh[16], dbh]
+            float all[18];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                all[c] = db[c];
+                all[8 + c] = gw[c];
+            }
+            all[16] = loss;
+            all[17] = gb;
+            float* out = reinterpret_cast<float*>(smem + oXch) + 128 * g;  // free: every row's exchange is over
+            asm volatile("bar.sync 2, 256;" ::: "memory");
+            group_sum(all, red, g, warp & 3, lane, out);
+            asm volatile("bar.sync %0, 128;" ::"r"(3 + g) : "memory");
+            float* part = p.partial + (int64_t)blockIdx.x * kX3FwdWidth;
+            if (px < 8) {
+                part[1 + 8 * g + px] = out[px];
+                part[17 + 8 * g + px] = out[8 + px];
+            }
+            if (g == 0 && px == 0) {
+                part[0] = out[16];
+                part[33] = out[17];
+            }
+        } else {
+            // dy1 = (h1 > 0) conv row; dW1[co][ky][kx] += dy1[co] x(y + ky, x + kx), channel pairs packed
+            float2 acc[9][4], db[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                db[c] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < 9; ++k) acc[k][c] = make_float2(0.f, 0.f);
+            }
+            while (sx_next(p, pos, end, it)) {
+                const int nst = it.rows + 2, x = it.x0 + px;
+                const bool col_ok = x < p.out_w;
+                const uint16_t* mrow = p.mask + ((int64_t)it.z * p.out_h + it.y0) * p.out_w + x;
+                const uint8_t* img = p.img + (int64_t)(p.zmap ? p.zmap[it.z] : it.z) * p.H * p.W;
+                int sc[3];
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) sc[kx] = sx_refl(x + kx - 2, p.W);
+                float w[3][3];  // x at input rows (of the conv row) ky, taps kx
+                uint8_t nb[3];
+                auto fetch = [&](int r) {  // image row that conv row r - 2's ky = 2 reads: y0 + r, mirrored by 2
+                    const uint8_t* src = img + (int64_t)sx_refl(it.y0 + r - 2, p.H) * p.W;
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) nb[kx] = __ldg(src + sc[kx]);
+                };
+#pragma unroll
+                for (int c = 0; c < 8; ++c) s0[c] = s1[c] = 0.f;
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) w[ky][kx] = 0.f;
+                fetch(0);
+                uint32_t m = 0;
+                for (int u = 0; u < nst; ++u, ++q) {
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) {
+                        w[0][kx] = w[1][kx];
+                        w[1][kx] = w[2][kx];
+                        w[2][kx] = lut[nb[kx]];  // row y0 + u
+                    }
+                    if (u + 1 < nst) fetch(u + 1);
+                    const uint32_t m_next = col_ok && u >= 1 && u + 1 < nst ? __ldg(mrow + (int64_t)(u - 1) * p.out_w) : 0u;
+                    float dy[8];
+                    row(dy);
+                    if (u >= 2) {
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) dy[c] = (m >> (8 * g + c)) & 1u ? dy[c] : 0.f;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const float2 d = make_float2(dy[2 * c], dy[2 * c + 1]);
+                            db[c].x += d.x;
+                            db[c].y += d.y;
+#pragma unroll
+                            for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+                                for (int kx = 0; kx < 3; ++kx)
+                                    acc[ky * 3 + kx][c] =
+                                        __ffma2_rn(d, make_float2(w[ky][kx], w[ky][kx]), acc[ky * 3 + kx][c]);
+                        }
+                    }
+                    m = m_next;
+                }
+            }
+            // partials per CTA: [144 (co, ky, kx)] then db1[16]
+            float all[80];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    all[(2 * c) * 9 + k] = acc[k][c].x;
+                    all[(2 * c + 1) * 9 + k] = acc[k][c].y;
+                }
+                all[72 + 2 * c] = db[c].x;
+                all[72 + 2 * c + 1] = db[c].y;
+            }
+            float* out = xch + 128 * g;
+            group_sum(all, red, g, warp & 3, lane, out);
+            asm volatile("bar.sync %0, 128;" ::"r"(3 + g) : "memory");
+            float* part = p.partial + (int64_t)blockIdx.x * 160;
+            if (px < 72) part[72 * g + px] = out[px];
+            if (px < 8) part[144 + 8 * g + px] = out[72 + px];
+        }
+    } else {
+        ptx::setmaxnreg_dec<120>();
+        // ================= producers ==================================================================
+        // Tasks e = pt + 128 i: 8 channels (e & 1) of pixel e >> 1. Each thread's loads of the row
+        // after next are issued before this row's are split (two rows in flight).
+        const int pt = tid - 384;
+        constexpr int kTasks = 3;  // ceil(2 * 130 / 128)
+        const int off = BWD ? -2 : 0, src_h = BWD ? p.H : p.H + 2, src_w = BWD ? p.W : p.W + 2;
+        uint32_t q = 0;
+        while (sx_next(p, pos, end, it)) {
+            const int nst = it.rows + 2;
+            const float* src = p.in + (int64_t)it.z * src_h * src_w * 16;
+            float4 v[2][kTasks][2];
+            auto load = [&](int u, float4 (&d)[kTasks][2]) {
+                const int y = it.y0 + u + off;
+#pragma unroll
+                for (int i = 0; i < kTasks; ++i) {
+                    const int e = pt + 128 * i, x = it.x0 + (e >> 1) + off;
+                    d[i][0] = d[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (e < 2 * 130 && u < nst && y >= 0 && y < src_h && x >= 0 && x < src_w) {
+                        const float4* a = reinterpret_cast<const float4*>(src + ((int64_t)y * src_w + x) * 16 + (e & 1) * 8);
+                        d[i][0] = __ldg(a);
+                        d[i][1] = __ldg(a + 1);
+                    }
+                }
+            };
+            auto put = [&](int u, float4 (&d)[kTasks][2]) {
+                if (u >= nst) return;
+                const uint32_t s = q % kRingX;
+                x_wait(&row_empty[s], ((q / kRingX) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
+                uint8_t* dst = smem + oRingX + s * kSlotX;
+#pragma unroll
+                for (int i = 0; i < kTasks; ++i) {
+                    const int e = pt + 128 * i;
+                    if (e < 2 * 130) {
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            uint4 w;
+                            w.x = take_part(d[i][0].x, d[i][0].y);
+                            w.y = take_part(d[i][0].z, d[i][0].w);
+                            w.z = take_part(d[i][1].x, d[i][1].y);
+                            w.w = take_part(d[i][1].z, d[i][1].w);
+                            *reinterpret_cast<uint4*>(dst + k * kPart + ((e & 1) * kP + (e >> 1)) * 16) = w;
+                        }
+                    }
+                }
+                ptx::fence_proxy_async_smem();
+                if (!p.fault_stall) ptx::mbar_arrive(&row_full[s]);
+                ++q;
+            };
+            load(0, v[0]);
+            load(1, v[1]);
+            for (int u = 0; u < nst; u += 2) {
+                put(u, v[0]);
+                load(u + 2, v[0]);
+                put(u + 1, v[1]);
+                load(u + 3, v[1]);
+            }
+        }
+    }
+
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    if (warp == 0) ptx::tmem_dealloc(tbase, 512);
+}
+
+// conv1 + ReLU from the uint8 slice: h1 [B][H+2][W+2][16] FP32 and its mask (bit c: h1[c] > 0). HBM
+// writes bound it (66 B per pixel). A warp walks down a 32-column strip; a lane keeps all 144 weights
+// (packed by channel pairs) and its 3x3 input window in registers.
+__global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int* zmap, int B, int H, int W, const float* fw,
+                                                   float* h1, uint16_t* mask, int n_strips, int64_t total) {
+    __shared__ float lut[256];
+    lut[threadIdx.x] = (float)threadIdx.x / 255.0f;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * 8, me = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    int64_t pos = total * me / nw;
+    const int64_t end = total * (me + 1) / nw;
+    const int H1 = H + 2, W1 = W + 2;
+    float2 w[9][8], b[8];  // fw: W1t[tap][co], b1
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        b[c] = make_float2(__ldg(fw + kSB1 + 2 * c), __ldg(fw + kSB1 + 2 * c + 1));
+#pragma unroll
+        for (int k = 0; k < 9; ++k) w[k][c] = make_float2(__ldg(fw + k * 16 + 2 * c), __ldg(fw + k * 16 + 2 * c + 1));
+    }
+    while (pos < end) {
+        const int64_t col = pos / H1;
+        const int y0 = (int)(pos - col * H1), z = (int)(col / n_strips), x = (int)(col % n_strips) * 32 + lane;
+        const int rows = (int)min((int64_t)(H1 - y0), end - pos);
+        pos += rows;
+        const uint8_t* src = in + (int64_t)(zmap ? zmap[z] : z) * H * W;
+        int sc[3];
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx) sc[kx] = sx_refl(x + kx - 2, W);
+        float win[3][3];
+        uint8_t nb[3];
+        auto fetch = [&](int r) {
+            const uint8_t* row = src + (int64_t)sx_refl(y0 + r - 2, H) * W;
+#pragma unroll
+            for (int kx = 0; kx < 3; ++kx) nb[kx] = __ldg(row + sc[kx]);
+        };
+#pragma unroll
+        for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+            for (int kx = 0; kx < 3; ++kx) win[ky][kx] = 0.f;
+        fetch(0);
+        for (int r = 0; r < rows + 2; ++r) {
+#pragma unroll
+            for (int kx = 0; kx < 3; ++kx) {
+                win[0][kx] = win[1][kx];
+                win[1][kx] = win[2][kx];
+                win[2][kx] = lut[nb[kx]];
+            }
+            if (r + 1 < rows + 2) fetch(r + 1);
+            if (r < 2) continue;
+            float2 acc[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[c] = b[c];
+#pragma unroll
+            for (int k = 0; k < 9; ++k)
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    acc[c] = __ffma2_rn(make_float2(win[k / 3][k % 3], win[k / 3][k % 3]), w[k][c], acc[c]);
+            if (x < W1) {
+                const int64_t pix = ((int64_t)z * H1 + y0 + r - 2) * W1 + x;
+                uint32_t m = 0;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    m |= (acc[c].x > 0.f ? 1u : 0u) << (2 * c) | (acc[c].y > 0.f ? 1u : 0u) << (2 * c + 1);
+                    acc[c] = make_float2(fmaxf(acc[c].x, 0.f), fmaxf(acc[c].y, 0.f));
+                }
+                float4* o = reinterpret_cast<float4*>(h1 + pix * 16);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) o[c] = make_float4(acc[2 * c].x, acc[2 * c].y, acc[2 * c + 1].x, acc[2 * c + 1].y);
+                mask[pix] = (uint16_t)m;
+            }
+        }
+    }
+}
+
+// conv2's weight gradient dW2[co][ci][ky][kx] = sum dy2[co](y, x) h1[ci](y + ky, x + kx) over 16x16
+// pixel tiles. FP32 FMA issue bounds it (2,304 per pixel). Thread: input channel t & 15, output channels
+// 4 ((t >> 4) & 3) .. + 3 as two pairs, tile rows 4 (t >> 6) .. + 3: 18 packed FMAs per pixel for three
+// window loads and one 16-byte load (scalar FMAs, two channels: 18 for five loads, 1,192 us on a batch
+// of 32 x 512 x 512). The next tile's 37 KB arrive by asynchronous copies meanwhile; 2 CTAs per SM.
+constexpr int kG2H = 18 * 18 * 16, kG2D = 16 * 16 * 16;  // floats per tile buffer
+constexpr int kG2Smem = 2 * (kG2H + kG2D) * 4;
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool on) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(on ? 16 : 0)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(256, 2) st_grad2(const float* dy2, const float* h1, int B, int H, int W, float* partial) {
+    extern __shared__ __align__(16) float sm[];
+    const int t = threadIdx.x, ci = t & 15, cg = (t >> 4) & 3, rg = t >> 6;
+    float2 acc[9][2];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k][0] = acc[k][1] = make_float2(0.f, 0.f);
+    const int tx_n = (W + 15) / 16, ty_n = (H + 15) / 16;
+    const int64_t tiles = (int64_t)B * tx_n * ty_n;
+    auto stage = [&](int64_t tile, int buf) {
+        if (tile < tiles) {
+            const int zi = (int)(tile / ((int64_t)tx_n * ty_n));
+            const int rem = (int)(tile - (int64_t)zi * tx_n * ty_n);
+            const int y0 = (rem / tx_n) * 16, x0 = (rem % tx_n) * 16;
+            float* sh = sm + buf * (kG2H + kG2D);
+            float* sd = sh + kG2H;
+            for (int e = t; e < 256 * 4; e += 256) {
+                const int px = e >> 2, y = y0 + (px >> 4), x = x0 + (px & 15);
+                const bool on = y < H && x < W;
+                cp_async16(sd + 4 * e, on ? dy2 + (((int64_t)zi * H + y) * W + x) * 16 + 4 * (e & 3) : dy2, on);
+            }
+            for (int e = t; e < 18 * 18 * 4; e += 256) {
+                const int px = e >> 2, y = y0 + px / 18, x = x0 + px % 18;
+                const bool on = y < H + 2 && x < W + 2;
+                cp_async16(sh + 4 * e, on ? h1 + (((int64_t)zi * (H + 2) + y) * (W + 2) + x) * 16 + 4 * (e & 3) : h1, on);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int buf = 0;
+    stage(blockIdx.x, 0);
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
+        stage(tile + gridDim.x, buf ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        const float* sh = sm + buf * (kG2H + kG2D) + ci;
+        const float* sd = sm + buf * (kG2H + kG2D) + kG2H + 4 * cg;
+#pragma unroll 1
+        for (int py = 4 * rg; py < 4 * rg + 4; ++py) {
+            float w[3][3];  // h1 at rows py + ky, columns px + kx
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+                for (int kx = 0; kx < 2; ++kx) w[ky][kx + 1] = sh[((py + ky) * 18 + kx) * 16];
+#pragma unroll
+            for (int px = 0; px < 16; ++px) {
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) {
+                    w[ky][0] = w[ky][1];
+                    w[ky][1] = w[ky][2];
+                    w[ky][2] = sh[((py + ky) * 18 + px + 2) * 16];
+                }
+                const float4 d = *reinterpret_cast<const float4*>(sd + (py * 16 + px) * 16);
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const float2 ww = make_float2(w[k / 3][k % 3], w[k / 3][k % 3]);
+                    acc[k][0] = __ffma2_rn(make_float2(d.x, d.y), ww, acc[k][0]);
+                    acc[k][1] = __ffma2_rn(make_float2(d.z, d.w), ww, acc[k][1]);
+                }
+            }
+        }
+        __syncthreads();  // the buffer is filled again in the next turn
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    // the four row groups' sums, in order
+    float* x = sm + (t & 63) * 37;
+    for (int r = 1; r < 4; ++r) {
+        if (rg == r)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                x[4 * k] = acc[k][0].x;
+                x[4 * k + 1] = acc[k][0].y;
+                x[4 * k + 2] = acc[k][1].x;
+                x[4 * k + 3] = acc[k][1].y;
+            }
+        __syncthreads();
+        if (rg == 0)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                acc[k][0].x += x[4 * k];
+                acc[k][0].y += x[4 * k + 1];
+                acc[k][1].x += x[4 * k + 2];
+                acc[k][1].y += x[4 * k + 3];
+            }
+        __syncthreads();
+    }
+    if (rg == 0) {
+        float* out = partial + (int64_t)blockIdx.x * 2304;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            out[((4 * cg + 0) * 16 + ci) * 9 + k] = acc[k][0].x;
+            out[((4 * cg + 1) * 16 + ci) * 9 + k] = acc[k][0].y;
+            out[((4 * cg + 2) * 16 + ci) * 9 + k] = acc[k][1].x;
+            out[((4 * cg + 3) * 16 + ci) * 9 + k] = acc[k][1].y;
+        }
+    }
+}
+
+// Every parameter's gradient and the loss from the CTAs' partial sums, in FP64 and a fixed order: thread
+// (o, j) of a block adds CTAs j, j + 8, ... of output o (32 consecutive outputs per block, so that the
+// loads are coalesced), then the eight are added in order.
+__global__ void __launch_bounds__(256) st_reduce(const float* fwd, const float* g2, const float* bwd, float inv_n,
+                                                 float* grad, float* loss) {
+    __shared__ double sh[8][32];
+    const int l = threadIdx.x & 31, j = threadIdx.x >> 5, o = blockIdx.x * 32 + l;
+    const float* src = nullptr;
+    int n = kX3Grid, width = 0;
+    if (o < kSW2) {  // W1, b1
+        src = bwd + o;
+        width = 160;
+    } else if (o < kSB2) {
+        src = g2 + (o - kSW2);
+        n = kX3GridG2;
+        width = 2304;
+    } else if (o <= kSN) {  // b2, head; the loss after the last parameter
+        src = fwd + (o == kSN ? 0 : 1 + o - kSB2);
+        width = kX3FwdWidth;
+    }
+    double s = 0.0;
+    if (src) {
+#pragma unroll 8
+        for (int c = j; c < n; c += 8) s += (double)__ldg(src + (int64_t)c * width);
+    }
+    sh[j][l] = s;
+    __syncthreads();
+    if (j == 0 && src) {
+#pragma unroll
+        for (int k = 1; k < 8; ++k) s += sh[k][l];
+        if (o == kSN)
+            *loss = (float)(s * (double)inv_n);
+        else
+            grad[o] = (float)s;
+    }
+}
+
+template <bool BWD>
+mb_status launch_sx(const SxParams& q, cudaStream_t st) {
+    static bool attr = false;
+    if (!attr) {
+        MB_CUDA(cudaFuncSetAttribute(st_x3<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemX));
+        attr = true;
+    }
+    SxParams p = q;
+    p.out_h = BWD ? p.H + 2 : p.H;
+    p.out_w = BWD ? p.W + 2 : p.W;
+    p.n_strips = (p.out_w + 127) / 128;
+    p.total_rows = (int64_t)p.B * p.n_strips * p.out_h;
+    const char* stall = getenv("MB_FAULT_STALL");
+    p.fault_stall = (stall && stall[0] == '1') ? 1 : 0;
+    p.wait_ns = p.fault_stall ? 200000000ull : kXWaitNs;
+    st_x3<BWD><<<kX3Grid, kThreadsX, kSmemX, st>>>(p);
+    count_launch();
+    MB_CUDA(cudaGetLastError());
+    return MB_OK;
+}
+
+}  // namespace
+
+mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
+    const int strips = (a.W + 2 + 31) / 32;
+    st_conv1<<<kX3Grid, 256, 0, st>>>(a.in, a.zmap, a.B, a.H, a.W, a.fw, a.h1, a.mask, strips,
+                                      (int64_t)a.B * strips * (a.H + 2));
+    count_launch();
+    SxParams p{};
+    p.fw = a.fw;
+    p.B = a.B;
+    p.H = a.H;
+    p.W = a.W;
+    p.zmap = a.zmap;
+    p.err = a.err;
+    p.in = a.h1;
+    p.wpack = a.pack;
+    p.target = a.target;
+    p.dy2 = a.dy2;
+    p.inv_n = a.inv_n;
+    p.partial = a.part_fwd;
+    MB_TRY(launch_sx<false>(p, st));
+    static bool attr = false;
+    if (!attr) {
+        MB_CUDA(cudaFuncSetAttribute(st_grad2, cudaFuncAttributeMaxDynamicSharedMemorySize, kG2Smem));
+        attr = true;
+    }
+    st_grad2<<<kX3GridG2, 256, kG2Smem, st>>>(a.dy2, a.h1, a.B, a.H, a.W, a.part_g2);
+    count_launch();
+    p.in = a.dy2;
+    p.wpack = a.pack + kX3StudentPack;
+    p.mask = a.mask;
+    p.img = a.in;
+    p.partial = a.part_bwd;
+    MB_TRY(launch_sx<true>(p, st));
+    st_reduce<<<(kSN + 1 + 31) / 32, 256, 0, st>>>(a.part_fwd, a.part_g2, a.part_bwd, a.inv_n, a.grad, a.loss);
+    count_launch();
+    MB_CUDA(cudaGetLastError());
+    return MB_OK;
+}
+
+}  // namespace mb
