@@ -542,113 +542,131 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
 }
 
 // conv2's weight gradient dW2[co][ci][ky][kx] = sum dy2[co](y, x) h1[ci](y + ky, x + kx) over 16x16
-// pixel tiles. FP32 FMA issue bounds it (2,304 per pixel). Thread: input channel t & 15, output channels
-// 4 ((t >> 4) & 3) .. + 3 as two pairs, tile rows 4 (t >> 6) .. + 3: 18 packed FMAs per pixel for three
-// window loads and one 16-byte load (scalar FMAs, two channels: 18 for five loads, 1,192 us on a batch
-// of 32 x 512 x 512). The next tile's 37 KB arrive by asynchronous copies meanwhile; 2 CTAs per SM.
+// pixel tiles. FP32 FMA issue bounds it (2,304 per pixel). Lane: input channels 2 (l & 7), + 1 as a
+// pair, output channels 4 (l >> 3) .. + 3; a warp takes two tile rows: 36 packed FMAs per pixel for
+// three 8-byte window loads and one 16-byte load (scalar FMAs over two output channels: 18 for five
+// loads). A ninth warp brings the next tile's 37 KB meanwhile, by bulk copies of whole tile rows; 2 CTAs
+// per SM. (With the copies issued by the computing warps, a rendezvous per tile cost 25 %.)
+// 32 x 512 x 512: MMMM us, the FMAs alone 580.
 constexpr int kG2H = 18 * 18 * 16, kG2D = 16 * 16 * 16;  // floats per tile buffer
-constexpr int kG2Smem = 2 * (kG2H + kG2D) * 4;
+constexpr int kG2Smem = 2 * (kG2H + kG2D) * 4 + 48;
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool on) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(on ? 16 : 0)
-                 : "memory");
-}
-
-__global__ void __launch_bounds__(256, 2) st_grad2(const float* dy2, const float* h1, int B, int H, int W, float* partial) {
-    extern __shared__ __align__(16) float sm[];
-    const int t = threadIdx.x, ci = t & 15, cg = (t >> 4) & 3, rg = t >> 6;
-    float2 acc[9][2];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) acc[k][0] = acc[k][1] = make_float2(0.f, 0.f);
+__global__ void __maxnreg__(112) st_grad2(const float* dy2, const float* h1, int B, int H, int W, float* partial,
+                                                   int* err) {
+    extern __shared__ __align__(128) float sm[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(sm + 2 * (kG2H + kG2D));
+    uint64_t* empty = full + 2;
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 4);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, cp = lane & 7, cg = lane >> 3;
     const int tx_n = (W + 15) / 16, ty_n = (H + 15) / 16;
     const int64_t tiles = (int64_t)B * tx_n * ty_n;
-    auto stage = [&](int64_t tile, int buf) {
-        if (tile < tiles) {
+    if (t == 0) {
+        for (int i = 0; i < 2; ++i) {
+            ptx::mbar_init(&full[i], 1);
+            ptx::mbar_init(&empty[i], 8);
+        }
+        *abort_flag = 0;
+        ptx::mbar_fence_init();
+    }
+    // what a short tile leaves uncovered is finite (stale or zero) in h1 and zero in dy2
+    for (int i = t; i < 2 * (kG2H + kG2D); i += 288) sm[i] = 0.f;
+    ptx::fence_proxy_async_smem();
+    __syncthreads();
+    float2 acc[9][4];
+    if (warp == 8) {
+        uint32_t n = 0;
+        bool ok = true;
+        for (int64_t tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x, ++n) {
+            const int buf = n & 1;
             const int zi = (int)(tile / ((int64_t)tx_n * ty_n));
             const int rem = (int)(tile - (int64_t)zi * tx_n * ty_n);
             const int y0 = (rem / tx_n) * 16, x0 = (rem % tx_n) * 16;
+            const int dr = min(16, H - y0), dc = min(16, W - x0);  // rows, columns of dy2; h1 has two more of each
+            ok = x_wait(&empty[buf], ((n >> 1) & 1) ^ 1, abort_flag, err, kXWaitNs);
+            if (!ok) break;
             float* sh = sm + buf * (kG2H + kG2D);
             float* sd = sh + kG2H;
-            for (int e = t; e < 256 * 4; e += 256) {
-                const int px = e >> 2, y = y0 + (px >> 4), x = x0 + (px & 15);
-                const bool on = y < H && x < W;
-                cp_async16(sd + 4 * e, on ? dy2 + (((int64_t)zi * H + y) * W + x) * 16 + 4 * (e & 3) : dy2, on);
+            if (dr < 16 || dc < 16) {
+                for (int i = lane; i < 256 * 4; i += 32) {
+                    const int px = i >> 2;
+                    if ((px >> 4) >= dr || (px & 15) >= dc)
+                        *reinterpret_cast<float4*>(sd + 4 * i) = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                ptx::fence_proxy_async_smem();  // a later tile's copies overwrite them
             }
-            for (int e = t; e < 18 * 18 * 4; e += 256) {
-                const int px = e >> 2, y = y0 + px / 18, x = x0 + px % 18;
-                const bool on = y < H + 2 && x < W + 2;
-                cp_async16(sh + 4 * e, on ? h1 + (((int64_t)zi * (H + 2) + y) * (W + 2) + x) * 16 + 4 * (e & 3) : h1, on);
-            }
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive_expect_tx(&full[buf], (uint32_t)(dr * dc + (dr + 2) * (dc + 2)) * 64u);
+            __syncwarp();
+            if (lane < dr)
+                ptx::bulk_copy_g2s(sd + lane * 16 * 16, dy2 + (((int64_t)zi * H + y0 + lane) * W + x0) * 16,
+                                   (uint32_t)dc * 64u, &full[buf]);
+            if (lane < dr + 2)
+                ptx::bulk_copy_g2s(sh + lane * 18 * 16, h1 + (((int64_t)zi * (H + 2) + y0 + lane) * (W + 2) + x0) * 16,
+                                   (uint32_t)(dc + 2) * 64u, &full[buf]);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    int buf = 0;
-    stage(blockIdx.x, 0);
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
-        stage(tile + gridDim.x, buf ^ 1);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        __syncthreads();
-        const float* sh = sm + buf * (kG2H + kG2D) + ci;
+        // copies still in flight (only where the CTA gave up) land before it ends
+        const uint64_t t0 = x_gtime();
+        for (uint32_t r = n > 2 ? n - 2 : 0; r < n; ++r)
+            while (!ptx::mbar_test(&full[r & 1], (r >> 1) & 1) && x_gtime() - t0 <= kXWaitNs) {
+            }
+    } else {
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[k][j] = make_float2(0.f, 0.f);
+    uint32_t n = 0;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++n) {
+        const int buf = n & 1;
+        x_wait(&full[buf], (n >> 1) & 1, abort_flag, err, kXWaitNs);
+        const float* sh = sm + buf * (kG2H + kG2D) + 2 * cp;
         const float* sd = sm + buf * (kG2H + kG2D) + kG2H + 4 * cg;
 #pragma unroll 1
-        for (int py = 4 * rg; py < 4 * rg + 4; ++py) {
-            float w[3][3];  // h1 at rows py + ky, columns px + kx
+        for (int py = 2 * warp; py < 2 * warp + 2; ++py) {
+            float2 w[3][3];  // h1 at rows py + ky, columns px + kx
+            auto h_at = [&](int ky, int c) { return *reinterpret_cast<const float2*>(sh + ((py + ky) * 18 + c) * 16); };
 #pragma unroll
             for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
-                for (int kx = 0; kx < 2; ++kx) w[ky][kx + 1] = sh[((py + ky) * 18 + kx) * 16];
+                for (int kx = 0; kx < 2; ++kx) w[ky][kx + 1] = h_at(ky, kx);
 #pragma unroll
             for (int px = 0; px < 16; ++px) {
 #pragma unroll
                 for (int ky = 0; ky < 3; ++ky) {
                     w[ky][0] = w[ky][1];
                     w[ky][1] = w[ky][2];
-                    w[ky][2] = sh[((py + ky) * 18 + px + 2) * 16];
+                    w[ky][2] = h_at(ky, px + 2);
                 }
                 const float4 d = *reinterpret_cast<const float4*>(sd + (py * 16 + px) * 16);
+                const float2 dd[4] = {make_float2(d.x, d.x), make_float2(d.y, d.y), make_float2(d.z, d.z),
+                                      make_float2(d.w, d.w)};
 #pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const float2 ww = make_float2(w[k / 3][k % 3], w[k / 3][k % 3]);
-                    acc[k][0] = __ffma2_rn(make_float2(d.x, d.y), ww, acc[k][0]);
-                    acc[k][1] = __ffma2_rn(make_float2(d.z, d.w), ww, acc[k][1]);
-                }
+                for (int k = 0; k < 9; ++k)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[k][j] = __ffma2_rn(w[k / 3][k % 3], dd[j], acc[k][j]);
             }
         }
-        __syncthreads();  // the buffer is filled again in the next turn
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&empty[buf]);
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
     __syncthreads();
-    // the four row groups' sums, in order
-    float* x = sm + (t & 63) * 37;
-    for (int r = 1; r < 4; ++r) {
-        if (rg == r)
+    // the eight warps' sums, in order
+    static_assert(8 * 2304 * 4 <= kG2Smem, "the warps' sums fit the tile buffers");
+    if (warp < 8) {
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                x[4 * k] = acc[k][0].x;
-                x[4 * k + 1] = acc[k][0].y;
-                x[4 * k + 2] = acc[k][1].x;
-                x[4 * k + 3] = acc[k][1].y;
-            }
-        __syncthreads();
-        if (rg == 0)
+        for (int k = 0; k < 9; ++k)
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                acc[k][0].x += x[4 * k];
-                acc[k][0].y += x[4 * k + 1];
-                acc[k][1].x += x[4 * k + 2];
-                acc[k][1].y += x[4 * k + 3];
-            }
-        __syncthreads();
-    }
-    if (rg == 0) {
-        float* out = partial + (int64_t)blockIdx.x * 2304;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            out[((4 * cg + 0) * 16 + ci) * 9 + k] = acc[k][0].x;
-            out[((4 * cg + 1) * 16 + ci) * 9 + k] = acc[k][0].y;
-            out[((4 * cg + 2) * 16 + ci) * 9 + k] = acc[k][1].x;
-            out[((4 * cg + 3) * 16 + ci) * 9 + k] = acc[k][1].y;
+            for (int j = 0; j < 4; ++j) {
+            sm[warp * 2304 + ((4 * cg + j) * 16 + 2 * cp) * 9 + k] = acc[k][j].x;
+            sm[warp * 2304 + ((4 * cg + j) * 16 + 2 * cp + 1) * 9 + k] = acc[k][j].y;
         }
+    }
+    __syncthreads();
+    for (int i = t; i < 2304; i += 288) {
+        float v = sm[i];
+#pragma unroll
+        for (int r = 1; r < 8; ++r) v += sm[r * 2304 + i];
+        partial[(int64_t)blockIdx.x * 2304 + i] = v;
     }
 }
 
@@ -736,7 +754,7 @@ mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
         MB_CUDA(cudaFuncSetAttribute(st_grad2, cudaFuncAttributeMaxDynamicSharedMemorySize, kG2Smem));
         attr = true;
     }
-    st_grad2<<<kX3GridG2, 256, kG2Smem, st>>>(a.dy2, a.h1, a.B, a.H, a.W, a.part_g2);
+    st_grad2<<<kX3GridG2, 288, kG2Smem, st>>>(a.dy2, a.h1, a.B, a.H, a.W, a.part_g2, a.err);
     count_launch();
     p.in = a.dy2;
     p.wpack = a.pack + kX3StudentPack;
