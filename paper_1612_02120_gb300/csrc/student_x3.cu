@@ -10,7 +10,8 @@
 // tap and sums the row taps in FP32.
 //
 // st_x3 reads one 64-byte pixel of h1 or dy2 per output pixel, once, and the forward writes dy2 once
-// (h2 and dy1 exist in registers only): 128 px rows cost ~500 cycles of MMAs and 360-710 of HBM time.
+// (h2 and dy1 exist in registers only): a row of 128 pixels costs ~500 cycles of MMAs and 360-710 of
+// HBM time; 1,320-1,620 measured (370 us a pass on a batch of 32 x 512 x 512), the epilogue's chain.
 // The separate kernels (conv 865 us, head and loss 218, data gradient 1,023, conv1's weight gradient
 // 395 on a batch of 32 x 512 x 512) passed 3.2 GB through HBM at 0.47-0.55 of the FP32 FMA rate.
 //
@@ -467,8 +468,9 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
 }
 
 // conv1 + ReLU from the uint8 slice: h1 [B][H+2][W+2][16] FP32 and its mask (bit c: h1[c] > 0). HBM
-// writes bound it (66 B per pixel). A warp walks down a 32-column strip; a lane keeps all 144 weights
-// (packed by channel pairs) and its 3x3 input window in registers.
+// writes bound it (66 B per pixel: 85 us on a batch of 32 x 512 x 512; 154 measured, 205 with weights
+// broadcast from shared memory). A warp walks down a 32-column strip; a lane keeps all 144 weights
+// (packed by channel pairs), its 3x3 input window and the bytes of the next four rows in registers.
 __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int* zmap, int B, int H, int W, const float* fw,
                                                    float* h1, uint16_t* mask, int n_strips, int64_t total) {
     __shared__ float lut[256];
@@ -496,26 +498,28 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
 #pragma unroll
         for (int kx = 0; kx < 3; ++kx) sc[kx] = sx_refl(x + kx - 2, W);
         float win[3][3];
-        uint8_t nb[3];
-        auto fetch = [&](int r) {
+        uint8_t nb[4][3];  // four rows of bytes in flight
+        auto fetch = [&](int r, uint8_t (&n)[3]) {
             const uint8_t* row = src + (int64_t)sx_refl(y0 + r - 2, H) * W;
 #pragma unroll
-            for (int kx = 0; kx < 3; ++kx) nb[kx] = __ldg(row + sc[kx]);
+            for (int kx = 0; kx < 3; ++kx) n[kx] = __ldg(row + sc[kx]);
         };
 #pragma unroll
         for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
             for (int kx = 0; kx < 3; ++kx) win[ky][kx] = 0.f;
-        fetch(0);
-        for (int r = 0; r < rows + 2; ++r) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) fetch(i, nb[i]);
+        auto step = [&](int r, uint8_t (&n)[3]) {
+            if (r >= rows + 2) return;
 #pragma unroll
             for (int kx = 0; kx < 3; ++kx) {
                 win[0][kx] = win[1][kx];
                 win[1][kx] = win[2][kx];
-                win[2][kx] = lut[nb[kx]];
+                win[2][kx] = lut[n[kx]];
             }
-            if (r + 1 < rows + 2) fetch(r + 1);
-            if (r < 2) continue;
+            if (r + 4 < rows + 2) fetch(r + 4, n);
+            if (r < 2) return;
             float2 acc[8];
 #pragma unroll
             for (int c = 0; c < 8; ++c) acc[c] = b[c];
@@ -537,6 +541,13 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
                 for (int c = 0; c < 4; ++c) o[c] = make_float4(acc[2 * c].x, acc[2 * c].y, acc[2 * c + 1].x, acc[2 * c + 1].y);
                 mask[pix] = (uint16_t)m;
             }
+        };
+#pragma unroll 1
+        for (int r = 0; r < rows + 2; r += 4) {
+            step(r, nb[0]);
+            step(r + 1, nb[1]);
+            step(r + 2, nb[2]);
+            step(r + 3, nb[3]);
         }
     }
 }
@@ -547,7 +558,7 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
 // three 8-byte window loads and one 16-byte load (scalar FMAs over two output channels: 18 for five
 // loads). A ninth warp brings the next tile's 37 KB meanwhile, by bulk copies of whole tile rows; 2 CTAs
 // per SM. (With the copies issued by the computing warps, a rendezvous per tile cost 25 %.)
-// 32 x 512 x 512: MMMM us, the FMAs alone 580.
+// 32 x 512 x 512: 588 us, of which the FMAs are 517.
 constexpr int kG2H = 18 * 18 * 16, kG2D = 16 * 16 * 16;  // floats per tile buffer
 constexpr int kG2Smem = 2 * (kG2H + kG2D) * 4 + 48;
 
