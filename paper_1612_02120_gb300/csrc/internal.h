@@ -140,16 +140,17 @@ mb_status fm_tc_layer(mb_net* net, int layer, const void* in, int64_t in_slice, 
                       cudaStream_t st);
 // MaskExtend (maskextend.cu): SIMT weight layout, and the +z transfer recursion (device pointers).
 void me_pack(const mb_net* net, const float* params, std::vector<float>& out);
-// MaskExtend FP16 tensor-core convs (maskextend_tc.cu). layer 0..4; in: [src rows][in_pitch][cs] FP16;
-// the conv reads input (r, c) = 2x2 max (dilation dm) at source (r, c), r < in_rows, c < in_cols;
-// layers 0-3 write FP16 features [out_h][out_pitch][N/2]; layer 4 writes the 3 class probabilities
-// [3][out_h][out_pitch] (planes probs_plane apart).
+// MaskExtend FP16 tensor-core convs (maskextend_tc.cu). layer 0..4; in, and the out of layers 0-3: FP16
+// features, max-filtered, chunk-planar [row][chunk of 8 channels][column (pitch)][8] (2, 4, 5, 6, 7 chunks
+// into layers 0..4); rows x cols is what the layer writes (layer 4: the 3 class probabilities
+// [3][rows][out_pitch], planes probs_plane apart), i.e. it reads rows + 3 d (+ d for layers 0-3) rows.
+// in_pitch is at least me_tc_in_pitch of the layer and cols (the last strip's overrun).
+int64_t me_tc_in_pitch(int layer, int64_t cols);
 mb_status me_tc_prepare(mb_net* net);
 void me_tc_release(mb_net* net);
 mb_status me_tc_poll_error(mb_net* net);
-mb_status me_tc_layer(mb_net* net, int layer, const void* in, int64_t in_pitch, int cs, int in_rows, int in_cols,
-                      int dm, void* out, int64_t out_pitch, int out_h, int out_w, float* probs, int64_t probs_plane,
-                      cudaStream_t st);
+mb_status me_tc_layer(mb_net* net, int layer, const void* in, int64_t in_pitch, void* out, int64_t out_pitch, int rows,
+                      int cols, float* probs, int64_t probs_plane, cudaStream_t st);
 mb_status maskextend_run(mb_net* net, const uint8_t* em, const float* memb, int64_t zt, int64_t h, int64_t w,
                          const uint8_t* seeds, int64_t z0, int64_t n_steps, int dz, float thr, uint8_t* masks_out,
                          float* probs_out, cudaStream_t st);

@@ -36,44 +36,46 @@ struct MeMasks {
     const uint8_t* m[4];  // masks of sections z + dz k for k = -4 .. -1, [h][w]
 };
 
-// Mirror-padded input stack of section z: out[(r, c)][ch] for r < h + 108, c < w + 108, FP32 or
-// (for the tensor-core path) FP16. dz = +1 or -1 is the direction of travel: the maps at offset k
-// of the transfer equation are read from section z + dz k.
+// Mirror-padded input stack of section z, r < h + 108, c < w + 108: FP32 out[r][c][16], or (the
+// tensor-core path) FP16 in two chunk planes, out[r][chunk][pitch][8]. dz = +1 or -1 is the direction of
+// travel: the maps at offset k of the transfer equation are read from section z + dz k. Blocks of 128
+// columns of one row.
 template <typename T>
-__global__ void me_assemble(const uint8_t* __restrict__ em, const float* __restrict__ memb, MeMasks mk, int64_t z,
-                            int dz, int h, int w, T* __restrict__ out) {
-    const int pw = w + 2 * kMeR, ph = h + 2 * kMeR;
-    const int64_t n = (int64_t)ph * pw;
+__global__ void __launch_bounds__(128) me_assemble(const uint8_t* __restrict__ em, const float* __restrict__ memb, MeMasks mk,
+                                                   int64_t z, int dz, int h, int w, T* __restrict__ out, int64_t pitch) {
+    const int pw = w + 2 * kMeR, nb = (pw + 127) / 128;
+    const int r = blockIdx.x / nb, c = (blockIdx.x - r * nb) * 128 + threadIdx.x;
+    if (c >= pw) return;
     const int64_t hw = (int64_t)h * w;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)(i / pw), c = (int)(i - (i / pw) * pw);
-        const int y = refl101(r - kMeR, h), x = refl101(c - kMeR, w);
-        const int64_t o = (int64_t)y * w + x;
-        float v[16];
+    const int64_t o = (int64_t)refl101(r - kMeR, h) * w + refl101(c - kMeR, w);
+    float v[16];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = (float)em[(z + dz * (k - 1)) * hw + o] / 255.0f;
+    for (int k = 0; k < 3; ++k) v[k] = (float)em[(z + dz * (k - 1)) * hw + o] / 255.0f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[3 + k] = (float)mk.m[k][o];
+    for (int k = 0; k < 4; ++k) v[3 + k] = (float)mk.m[k][o];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) v[7 + k] = memb[(z + dz * (k - 2)) * hw + o];
+    for (int k = 0; k < 5; ++k) v[7 + k] = memb[(z + dz * (k - 2)) * hw + o];
 #pragma unroll
-        for (int k = 12; k < 16; ++k) v[k] = 0.f;
-        if constexpr (sizeof(T) == 4) {
-            float4* d = reinterpret_cast<float4*>(out + i * kMeCin);
+    for (int k = 12; k < 16; ++k) v[k] = 0.f;
+    if constexpr (sizeof(T) == 4) {
+        float4* d = reinterpret_cast<float4*>(out + ((int64_t)r * pitch + c) * kMeCin);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) d[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-        } else {
-            uint32_t hw[8];
+        for (int k = 0; k < 4; ++k) d[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    } else {
+        uint32_t q[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                __half2 h2 = __floats2half2_rn(v[2 * k], v[2 * k + 1]);
-                hw[k] = *reinterpret_cast<uint32_t*>(&h2);
-            }
-            uint4* d = reinterpret_cast<uint4*>(out + i * kMeCin);
-            d[0] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-            d[1] = make_uint4(hw[4], hw[5], hw[6], hw[7]);
+        for (int k = 0; k < 8; ++k) {
+            const __half2 h2 = __floats2half2_rn(v[2 * k], v[2 * k + 1]);
+            q[k] = *reinterpret_cast<const uint32_t*>(&h2);
         }
+        T* d = out + ((int64_t)2 * r * pitch + c) * 8;
+        *reinterpret_cast<uint4*>(d) = make_uint4(q[0], q[1], q[2], q[3]);
+        *reinterpret_cast<uint4*>(d + pitch * 8) = make_uint4(q[4], q[5], q[6], q[7]);
     }
+}
+
+static unsigned assemble_grid(int64_t h, int64_t w) {
+    return (unsigned)((w + 2 * kMeR + 127) / 128 * (h + 2 * kMeR));
 }
 
 // 1x1 head 64 -> 3 and the softmax: probs[cls][y][x] = exp(z_cls - max) / sum exp(z - max).
@@ -163,41 +165,44 @@ static mb_status maskextend_run_tc(mb_net* net, const uint8_t* em, const float* 
                                    const uint8_t* seeds, int64_t z0, int64_t n_steps, int dz, float thr,
                                    uint8_t* masks_out, float* probs_out, cudaStream_t st) {
     MB_TRY(me_tc_poll_error(net));  // a wait that timed out in an earlier call on this net
-    const int64_t r[5] = {h + 105, h + 98, h + 84, h + 56, h}, c[5] = {w + 105, w + 98, w + 84, w + 56, w};
-    const int d[5] = {1, 2, 4, 8, 16}, dm[5] = {0, 1, 2, 4, 8};
-    const int64_t feat[5] = {32, 40, 48, 56, 64};
+    // Layer k writes rows[k] x cols[k]: what layer k + 1 reads (its output + 3 d), the last the maps;
+    // its input has chunks[k] planes of pitch[k] columns.
+    const int d[5] = {1, 2, 4, 8, 16}, chunks[5] = {2, 4, 5, 6, 7};
+    int64_t rows[5], cols[5], pitch[5], n_in[5], total = 0;
+    rows[4] = h;
+    cols[4] = w;
+    for (int k = 3; k >= 0; --k) {  // layer k + 1's conv outputs are d rows more than what it writes (k + 1 < 4)
+        const int64_t more = 3 * d[k + 1] + (k + 1 < 4 ? d[k + 1] : 0);
+        rows[k] = rows[k + 1] + more;
+        cols[k] = cols[k + 1] + more;
+    }
     auto up = [](int64_t n) { return (n + 127) & ~(int64_t)127; };  // 256-byte aligned sub-buffers (FP16)
-    const int64_t n_in = up((h + 108) * (w + 108) * kMeCin);
-    int64_t n_act[4], total = n_in;
-    for (int k = 0; k < 4; ++k) {
-        n_act[k] = up(r[k] * c[k] * feat[k]);
-        total += n_act[k];
+    for (int k = 0; k < 5; ++k) {
+        pitch[k] = me_tc_in_pitch(k, cols[k]);
+        const int64_t in_rows = k == 0 ? h + 2 * kMeR : rows[k - 1];
+        if (k == 0) pitch[0] = std::max<int64_t>(pitch[0], w + 2 * kMeR);
+        n_in[k] = up(in_rows * chunks[k] * pitch[k] * 8);
+        total += n_in[k];
     }
     const int64_t n_prob = up(2 * 3 * h * w);  // FP32 probabilities, counted in FP16 units
     total += n_prob;
     MB_TRY(net->ws.ensure((size_t)total * sizeof(__half)));
-    __half* xin = static_cast<__half*>(net->ws.ptr);
-    __half* act[4];
-    act[0] = xin + n_in;
-    for (int k = 1; k < 4; ++k) act[k] = act[k - 1] + n_act[k - 1];
-    float* prob_tmp = reinterpret_cast<float*>(act[3] + n_act[3]);
+    __half* in[5];
+    in[0] = static_cast<__half*>(net->ws.ptr);
+    for (int k = 1; k < 5; ++k) in[k] = in[k - 1] + n_in[k - 1];
+    float* prob_tmp = reinterpret_cast<float*>(in[4] + n_in[4]);
     const int64_t hw = h * w;
     for (int64_t s = 0; s < n_steps; ++s) {
         const int64_t z = z0 + dz * s;
         MeMasks mk;
         me_masks(mk, seeds, masks_out, s, hw);
-        me_assemble<__half><<<me_grid((h + 108) * (w + 108)), 256, 0, st>>>(em, memb, mk, z, dz, (int)h, (int)w, xin);
+        me_assemble<__half><<<assemble_grid(h, w), 128, 0, st>>>(em, memb, mk, z, dz, (int)h, (int)w, in[0], pitch[0]);
         count_launch();
         MB_CUDA(cudaGetLastError());
         float* probs = probs_out ? probs_out + s * 3 * hw : prob_tmp;
-        for (int k = 0; k < 5; ++k) {
-            const void* in = k == 0 ? (const void*)xin : (const void*)act[k - 1];
-            const int64_t in_pitch = k == 0 ? w + 108 : c[k - 1];
-            const int cs = k == 0 ? kMeCin : (int)feat[k - 1];
-            MB_TRY(me_tc_layer(net, k, in, in_pitch, cs, (int)(r[k] + 3 * d[k]), (int)(c[k] + 3 * d[k]), dm[k],
-                               k < 4 ? (void*)act[k] : nullptr, k < 4 ? c[k] : w, (int)r[k], (int)c[k],
-                               k == 4 ? probs : nullptr, hw, st));
-        }
+        for (int k = 0; k < 5; ++k)
+            MB_TRY(me_tc_layer(net, k, in[k], pitch[k], k < 4 ? (void*)in[k + 1] : nullptr, k < 4 ? pitch[k + 1] : w,
+                               (int)rows[k], (int)cols[k], k == 4 ? probs : nullptr, hw, st));
         me_smooth_threshold<<<me_grid(hw), 256, 0, st>>>(probs, (int)h, (int)w, thr, masks_out + s * hw);
         count_launch();
         MB_CUDA(cudaGetLastError());
@@ -250,7 +255,7 @@ mb_status maskextend_run(mb_net* net, const uint8_t* em, const float* memb, int6
         const int64_t z = z0 + dz * s;
         MeMasks mk;
         me_masks(mk, seeds, masks_out, s, hw);
-        me_assemble<float><<<me_grid((h + 108) * (w + 108)), 256, 0, st>>>(em, memb, mk, z, dz, (int)h, (int)w, xin);
+        me_assemble<float><<<assemble_grid(h, w), 128, 0, st>>>(em, memb, mk, z, dz, (int)h, (int)w, xin, w + 2 * kMeR);
         count_launch();
         MB_CUDA(cudaGetLastError());
         for (int k = 0; k < 5; ++k) {

@@ -20,16 +20,24 @@
 // and per group: with the tensor pipe reading shared memory at its full rate, each poll or commit
 // costs tens of cycles of MMA issue.
 //
-// Warp roles (512 threads, 1 CTA per SM, persistent over work items):
+// Features in global memory are what the next conv reads, already max-filtered, chunk-planar:
+// [row][8-channel chunk][column][16 B], so a staged row is a few contiguous runs that one thread fetches
+// with bulk copies. (Eight producer warps gathering 4 x 16 B per pixel took ~9,000 cycles for a row of
+// the last layer, a quarter of its launch before the first group was staged, and while they ran an MMA
+// took 85-100 cycles of the issuing thread against 65 alone.) The epilogue owns the values the filter
+// needs: a CTA walks one residue class, so the vertical partner y + D is the next row it drains, and the
+// horizontal one x + D is in the same strip. A strip of 128 conv columns yields 128 - D filtered ones, an
+// item one conv row more than filtered rows. The maxima are of values already rounded to FP16, so the
+// maps are bitwise those of filtering on the load.
+//
+// Warp roles (384 threads, 1 CTA per SM, persistent over work items):
 //   warp 0       TMEM owner; lane 0 issues the MMAs
-//   warp 1       lane 0 streams the weight units into their ring with bulk asynchronous copies
-//                (completion counted on the unit's mbarrier)
-//   warps 4-7    epilogue: TMEM -> registers, + bias, max-out, FP16 store (head: the 1x1 conv to 3
-//                classes and the softmax, FP32 probabilities)
-//   warps 8-15   A producers, groups taking staged rows in turn (4 groups of 2 warps for the first
-//                layer, 2 of 4 after): the 2x2 max-filter (dilation dm) of the previous layer's
-//                output, or the assembled input stack, into the staged-row ring (as deep as shared
-//                memory allows, up to 12 rows)
+//   warp 1       lane 0 streams the weight units into their ring with bulk copies (completion counted
+//                on the unit's mbarrier)
+//   warp 2       lane 0 fetches the staged rows (as many ahead as shared memory allows, up to 12)
+//   warps 4-11   epilogue, two groups of 4 warps, each half of the feature chunks: TMEM -> registers,
+//                + bias, max-out, FP16, max-filter, store. Last layer: the first group alone, the 1x1
+//                conv to 3 classes and the softmax, FP32 probabilities
 // Every mbarrier wait is bounded (a global-timer limit), after which the CTA records
 // MB_ERR_TIMEOUT in a mapped host word, stops issuing work, waits (bounded) for its bulk copies in
 // flight and frees its TMEM.
@@ -49,22 +57,15 @@ namespace mb {
 
 namespace {
 
-constexpr int kMThreads = 512;
+constexpr int kMThreads = 384;
 constexpr int kMBRing = 3;   // weight units in flight (a unit is 4 or 2 tap tiles)
 constexpr uint64_t kMWaitNs = 4000000000ull;
-
-// Staged pixels per row: >= 128 + 3 D, and chosen so that the 8 threads of a quarter-warp, which
-// store consecutive (chunk, pixel) tasks, hit distinct 16-byte bank groups (pixel pitch of a chunk
-// plane = MP x 16 bytes).
-__host__ __device__ constexpr int me_mp(int chunks, int D) {
-    return chunks == 2 ? 132 : chunks == 4 ? 138 : D <= 4 ? 141 : D <= 8 ? 153 : 177;
-}
 
 template <int KC, int N, int D, bool HEAD>
 struct MCfg {
     static constexpr int kChunks = 2 * KC;              // 8-channel chunks per staged pixel
-    static constexpr int kMP = me_mp(kChunks, D);
-    static constexpr int kNpix = 128 + 3 * D;            // staged pixels a row needs
+    static constexpr int kMP = 128 + 3 * D;              // staged pixels per row
+    static constexpr int kOutChunks = N / 16;            // 8-feature chunks of the output
     static constexpr int kARow = kChunks * kMP * 16;     // bytes per staged row
     static constexpr int kBTap = kChunks * N * 16;       // bytes per tap tile [chunk][N][16 B]
     static constexpr int kConsts = N + (HEAD ? 3 * 64 + 3 : 0);  // biases (+ head W[3][64], b[3])
@@ -75,38 +76,38 @@ struct MCfg {
     static constexpr int kBU = KC == 4 ? 2 : 4;
     static constexpr int kBUnit = kBU * kBTap;
     // staged rows: kR in use by a step, the rest filled ahead (as many as fit, up to 12)
-    static constexpr int kFixed = kMBRing * kBUnit + kConsts * 4 + 16 + (2 * kMBRing + kR + 2) * 8 + 16;
+    // the strip-edge exchange: 2 rows in turn x output chunks x 4 warps x D pixels x 16 B
+    static constexpr int kXch = HEAD ? 0 : 2 * kOutChunks * 4 * D * 16;
+    static constexpr int kEpi = HEAD ? 128 : 256;        // epilogue threads
+    static constexpr int kStrip = HEAD ? 128 : 128 - D;  // output columns of a strip
+    static constexpr int kMore = HEAD ? 0 : 1;           // conv rows of an item beyond its output rows
+    static constexpr int kFixed = kMBRing * kBUnit + kXch + kConsts * 4 + 16 + (2 * kMBRing + kR + 2) * 8 + 16;
     static constexpr int kARing = (227 * 1024 - kFixed) / (kARow + 16) < 12 ? (227 * 1024 - kFixed) / (kARow + 16) : 12;
-    // producer groups taking staged rows in turn (more for the short rows of the first layer)
-    static constexpr int kGroups = KC == 1 ? 4 : 2;
-    static constexpr int kGThreads = 256 / kGroups;
     static constexpr int oA = 0;
     static constexpr int oB = oA + kARing * kARow;
-    static constexpr int oConst = oB + kMBRing * kBUnit;
+    static constexpr int oXch = oB + kMBRing * kBUnit;
+    static constexpr int oConst = oXch + kXch;
     static constexpr int oBar = oConst + ((kConsts * 4 + 15) & ~15);
     static constexpr int kBars = 2 * kARing + 2 * kMBRing + 1 + kR + 1;
     static constexpr int oMisc = oBar + kBars * 8;
     static constexpr int kSmem = oMisc + 16;
-    static constexpr int kATasks = (kNpix * kChunks + kGThreads - 1) / kGThreads;
-    static_assert(kNpix <= kMP, "staged row too short");
     static_assert(kARing >= kR + 1, "staged-row ring");
     static_assert(N % 16 == 0 && N <= 128, "MMA N");
     static_assert(kSmem <= 227 * 1024, "shared memory");
 };
 
 struct MeTcParams {
-    const __half* in;       // source [src rows][in_pitch][cs] FP16
-    __half* out;            // layers: [out_h][out_pitch][N/2] FP16
+    const __half* in;       // features [row][chunk][in_pitch][8] FP16, src_chunks chunks
+    __half* out;            // layers: features in the same layout, N / 16 chunks
     float* probs;           // head: [3][out_h][out_pitch] FP32, planes probs_plane apart
     const uint8_t* wpack;   // 16 tap tiles, then the FP32 constants
     int* err;
     int64_t in_pitch, out_pitch, probs_plane;  // pixels
-    int cs;                 // source channels (a multiple of 8, <= 16 KC)
-    int in_rows, in_cols;   // conv input domain: input (r, c) = 2x2 max (dilation dm) at source (r, c)
-    int out_h, out_w, dm;
+    int src_chunks;         // 8-channel chunks of the input (the operand's further ones stay zero)
+    int out_h, out_w;       // what is written: filtered features; the head: the maps
     int n_strips;
     int total_rows;         // strip-rows of the launch: n_strips x out_h (< 2^31, checked)
-    int fault_stall;        // test injection: producers withhold their arrivals
+    int fault_stall;        // test injection: the loaders withhold their copies
     uint64_t wait_ns;
 };
 
@@ -136,7 +137,7 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, volatil
 }
 
 struct MeItem {
-    int ry, x0, m0, rows;  // output rows y = ry + D (m0 + j), j < rows; rows may be 0
+    int ry, x0, m0, rows;  // written rows y = ry + D (m0 + j), j < rows
 };
 
 // Work split: the launch's strip-rows, in (residue class ry, strip, row) order, are cut into one
@@ -144,7 +145,8 @@ struct MeItem {
 // items are the parts of its range in one (ry, strip) column. Residue class ry has
 // hr = ceil((out_h - ry) / D) rows per strip, i.e. base + 1 for ry < rem and base after
 // (out_h = D base + rem), so n_strips (ry base + min(ry, rem)) strip-rows precede it. Every role of
-// a CTA walks the same sequence.
+// a CTA walks the same sequence. A layer's item of n filtered rows is n + 1 conv rows; an item of n
+// conv rows stages n + 3 input rows.
 struct MeCursor {
     int g, hi;  // next strip-row, end of this CTA's range
 };
@@ -156,7 +158,7 @@ __device__ __forceinline__ MeCursor me_begin(const MeTcParams& p) {
     return c;
 }
 
-template <int D>
+template <int D, int STRIP>
 __device__ __forceinline__ bool me_next(const MeTcParams& p, MeCursor& c, MeItem& it) {
     if (c.g >= c.hi) return false;
     const int base = p.out_h / D, rem = p.out_h % D;
@@ -167,7 +169,7 @@ __device__ __forceinline__ bool me_next(const MeTcParams& p, MeCursor& c, MeItem
     const int off = c.g - before(ry);
     const int strip = off / hr;
     it.ry = ry;
-    it.x0 = strip * 128;
+    it.x0 = strip * STRIP;
     it.m0 = off - strip * hr;
     it.rows = min(hr - it.m0, c.hi - c.g);
     c.g += it.rows;
@@ -198,11 +200,12 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::oMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::oMisc + 4);
     const float* cst = reinterpret_cast<const float*>(smem + C::oConst);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the same in all lanes
 
     if (tid == 0) {
         for (int i = 0; i < C::kARing; ++i) {
-            ptx::mbar_init(&a_full[i], C::kGThreads);
+            ptx::mbar_init(&a_full[i], 1);
             ptx::mbar_init(&a_empty[i], 1);
         }
         for (int i = 0; i < kMBRing; ++i) {
@@ -210,7 +213,7 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
             ptx::mbar_init(&b_empty[i], 1);
         }
         ptx::mbar_init(acc_full, 1);
-        for (int i = 0; i < C::kR; ++i) ptx::mbar_init(&acc_free[i], 128);
+        for (int i = 0; i < C::kR; ++i) ptx::mbar_init(&acc_free[i], C::kEpi);
         ptx::mbar_init(fin, 1);
         *abort_flag = 0;
         ptx::mbar_fence_init();
@@ -219,6 +222,12 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
         const float* src = reinterpret_cast<const float*>(p.wpack + 16 * C::kBTap);
         float* dst = reinterpret_cast<float*>(smem + C::oConst);
         for (int i = tid; i < C::kConsts; i += kMThreads) dst[i] = __ldg(src + i);
+        // channels that the operand has beyond the input's stay zero
+        uint4* a = reinterpret_cast<uint4*>(smem + C::oA);
+        const int pad = (C::kChunks - p.src_chunks) * C::kMP;
+        for (int i = tid; i < C::kARing * pad; i += kMThreads)
+            a[(i / pad) * (C::kARow / 16) + p.src_chunks * C::kMP + i % pad] = make_uint4(0, 0, 0, 0);
+        ptx::fence_proxy_async_smem();
     }
     if (warp == 0) {
         ptx::tmem_alloc(tmem_slot, 512);
@@ -232,9 +241,13 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
 
     if (warp == 0) {
         // ================= MMA issuer ================================================================
-        if (lane == 0) {
-            const uint64_t adesc0 = ptx::smem_desc(sbase + C::oA, C::kMP * 16, 128);
-            const uint64_t bdesc0 = ptx::smem_desc(sbase + C::oB, N * 16, 128);
+        // The whole warp walks the loop on uniform values, lane 0 issuing: a divergent branch would
+        // move every operand of every MMA through vector registers.
+            const uint64_t adesc = ptx::smem_desc(sbase + C::oA, C::kMP * 16, 128);
+            const uint64_t bdesc = ptx::smem_desc(sbase + C::oB, N * 16, 128);
+            const uint32_t adesc0 = (uint32_t)adesc, a_hi = (uint32_t)(adesc >> 32);
+            const uint32_t bdesc0 = (uint32_t)bdesc, b_hi = (uint32_t)(bdesc >> 32);
+            const uint32_t lead = lane == 0;
             constexpr uint32_t idesc = ptx::idesc_f32acc(ptx::kFmtF16, 128, N);
             constexpr int kR = C::kR, kBU = C::kBU;
             uint32_t a_seq = 0, u_seq = 0;
@@ -245,32 +258,34 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
             // before it). Rows are runtime loops and only taps and K chunks are unrolled (the tap
             // shift D kx and the chunk kc are compile-time offsets): a short issue loop stays in
             // the instruction cache beside the other roles' code.
-            auto mma_taps = [&](uint64_t ad, uint32_t dcol, uint64_t bd, auto kx0, auto ntaps, bool zero_first) {
+            auto mma_taps = [&](uint32_t ad, uint32_t dcol, uint32_t bd, auto kx0, auto ntaps, bool zero_first) {
+                const uint32_t on = ok ? lead : 0u;
 #pragma unroll
                 for (int t = 0; t < decltype(ntaps)::value; ++t)
 #pragma unroll
                     for (int kc = 0; kc < KC; ++kc) {
                         const int kx = decltype(kx0)::value + t;
-                        ptx::mma_bf16(dcol, ad + (uint64_t)((D * kx * 16 + kc * 2 * C::kMP * 16) >> 4),
-                                      bd + (uint64_t)(((kx % kBU) * C::kBTap + kc * 2 * N * 16) >> 4), idesc,
-                                      (zero_first && t == 0 && kc == 0) ? 0u : 1u);
+                        ptx::mma_bf16_acc(on, dcol, ad + (uint32_t)((D * kx * 16 + kc * 2 * C::kMP * 16) >> 4), a_hi,
+                                          bd + (uint32_t)(((kx % kBU) * C::kBTap + kc * 2 * N * 16) >> 4), b_hi, idesc,
+                                          (zero_first && t == 0 && kc == 0) ? 0u : 1u);
                     }
             };
-            auto unit_desc = [&](uint32_t q) { return bdesc0 + (uint64_t)(((q % kMBRing) * C::kBUnit) >> 4); };
+            auto unit_desc = [&](uint32_t q) { return bdesc0 + (((q % kMBRing) * C::kBUnit) >> 4); };
             auto wait_unit = [&](uint32_t q) {
                 ok = ok && wait_bar(&b_full[q % kMBRing], (q / kMBRing) & 1, abort_flag, p.err, p.wait_ns);
             };
             MeCursor cur = me_begin(p);
             MeItem it;
-            while (me_next<D>(p, cur, it)) {
-                const int groups = (it.rows + kR - 1) / kR;
+            while (me_next<D, C::kStrip>(p, cur, it)) {
+                const int rows = it.rows + C::kMore;
+                const int groups = (rows + kR - 1) / kR;
                 int a_known = 0;  // staged rows [0, a_known) of the item are known full
                 int a_rel = 0;    // staged rows [0, a_rel) are released
                 auto release_upto = [&](int last) {
-                    for (; a_rel <= last; ++a_rel) ptx::mma_commit(&a_empty[(a_seq + a_rel) % C::kARing]);
+                    for (; a_rel <= last; ++a_rel) ptx::mma_commit_if(lead, &a_empty[(a_seq + a_rel) % C::kARing]);
                 };
                 for (int g = 0; g < groups; ++g) {
-                    const int rg = min(kR, it.rows - kR * g);
+                    const int rg = min(kR, rows - kR * g);
                     for (int ky = 0; ky < 4; ++ky) {
                         const int s = kR * g + ky;  // staged rows s .. s + rg - 1
                         for (; a_known < s + rg; ++a_known) {
@@ -280,21 +295,21 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                         const uint32_t aslot0 = (a_seq + s) % C::kARing;
                         auto arow = [&](int j) {
                             const uint32_t sl = aslot0 + j < (uint32_t)C::kARing ? aslot0 + j : aslot0 + j - C::kARing;
-                            return adesc0 + (uint64_t)((sl * C::kARow) >> 4);
+                            return adesc0 + ((sl * C::kARow) >> 4);
                         };
                         if (ky == 0) {
                             // the step's weight units, then rows one after the other, each waiting
                             // only for its own accumulator
                             for (int u = 0; u < 4 / kBU; ++u) wait_unit(u_seq + u);
-                            const uint64_t bd0 = unit_desc(u_seq), bd1 = unit_desc(u_seq + (4 / kBU) - 1);
+                            const uint32_t bd0 = unit_desc(u_seq), bd1 = unit_desc(u_seq + (4 / kBU) - 1);
                             for (int j = 0; j < rg; ++j) {
                                 ok = ok && wait_bar(&acc_free[j], ((free_par >> j) & 1) ^ 1, abort_flag, p.err,
                                                     p.wait_ns);
                                 free_par ^= 1u << j;
                                 ptx::tc_fence_after();
-                                const uint64_t ad = arow(j);
+                                const uint32_t ad = arow(j);
                                 const uint32_t dcol = tbase + (uint32_t)(C::kAccStride * j);
-                                if (ok) {
+                                {
                                     if constexpr (kBU == 4) {
                                         mma_taps(ad, dcol, bd0, std::integral_constant<int, 0>{},
                                                  std::integral_constant<int, 4>{}, true);
@@ -306,16 +321,16 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                                     }
                                 }
                             }
-                            for (int u = 0; u < 4 / kBU; ++u) ptx::mma_commit(&b_empty[(u_seq + u) % kMBRing]);
+                            for (int u = 0; u < 4 / kBU; ++u) ptx::mma_commit_if(lead, &b_empty[(u_seq + u) % kMBRing]);
                             u_seq += 4 / kBU;
                         } else {
                             for (int u = 0; u < 4 / kBU; ++u) {
                                 wait_unit(u_seq);
                                 ptx::tc_fence_after();
-                                const uint64_t bd = unit_desc(u_seq);
-                                if (ok) {
+                                const uint32_t bd = unit_desc(u_seq);
+                                {
                                     for (int j = 0; j < rg; ++j) {
-                                        const uint64_t ad = arow(j);
+                                        const uint32_t ad = arow(j);
                                         const uint32_t dcol = tbase + (uint32_t)(C::kAccStride * j);
                                         if constexpr (kBU == 4) {
                                             mma_taps(ad, dcol, bd, std::integral_constant<int, 0>{},
@@ -329,49 +344,52 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                                         }
                                     }
                                 }
-                                ptx::mma_commit(&b_empty[u_seq % kMBRing]);
+                                ptx::mma_commit_if(lead, &b_empty[u_seq % kMBRing]);
                                 ++u_seq;
                             }
                         }
                         // staged row s is not read by any later step
                         release_upto(s);
                     }
-                    ptx::mma_commit(acc_full);
+                    ptx::mma_commit_if(lead, acc_full);
                     // rows before the next group's first are done; after the last group, all rows
-                    release_upto(g + 1 < groups ? kR * (g + 1) - 1 : it.rows + 2);
+                    release_upto(g + 1 < groups ? kR * (g + 1) - 1 : rows + 2);
                 }
-                a_seq += it.rows + 3;
+                a_seq += rows + 3;
             }
-            ptx::mma_commit(fin);
-            const uint64_t t0 = gtime();
-            while (!ptx::mbar_test(fin, 0)) {
-                if (gtime() - t0 > p.wait_ns) {
-                    *(volatile int*)p.err = MB_ERR_TIMEOUT;
-                    break;
+            if (lane == 0) {
+                ptx::mma_commit(fin);
+                const uint64_t t0 = gtime();
+                while (!ptx::mbar_test(fin, 0)) {
+                    if (gtime() - t0 > p.wait_ns) {
+                        *(volatile int*)p.err = MB_ERR_TIMEOUT;
+                        break;
+                    }
                 }
             }
-        }
         __syncwarp();
-    } else if (warp >= 4 && warp < 8) {
+    } else if (HEAD ? (warp >= 4 && warp < 8) : warp >= 4) {
         // ================= epilogue ===================================================================
-        const int px = tid - 128;  // TMEM lane = pixel of the strip
-        const uint32_t lanes = (uint32_t)(32 * (warp - 4)) << 16;
+        const int px = tid & 127;  // TMEM lane = pixel of the strip
+        const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
         uint32_t n_groups = 0;
         MeCursor cur = me_begin(p);
         MeItem it;
-        while (me_next<D>(p, cur, it)) {
-            const int x = it.x0 + px;
-            for (int j = 0; j < it.rows; ++j) {
-                if (j % C::kR == 0) {  // a new group: all its accumulators are complete together
-                    wait_bar(acc_full, n_groups & 1, abort_flag, p.err, p.wait_ns);
-                    ++n_groups;
-                    ptx::tc_fence_after();
-                }
-                const uint32_t s = j % C::kR;  // accumulator of this row
-                const uint32_t ta = tbase + lanes + (uint32_t)C::kAccStride * s;
-                const int y = it.ry + D * (it.m0 + j);
-                const bool store = x < p.out_w && y < p.out_h && !*abort_flag;
-                if constexpr (HEAD) {
+        auto wait_group = [&](int j) {  // at a group's first row: all its accumulators are complete together
+            if (j % C::kR == 0) {
+                wait_bar(acc_full, n_groups & 1, abort_flag, p.err, p.wait_ns);
+                ++n_groups;
+                ptx::tc_fence_after();
+            }
+        };
+        if constexpr (HEAD) {
+            while (me_next<D, C::kStrip>(p, cur, it)) {
+                const int x = it.x0 + px;
+                for (int j = 0; j < it.rows; ++j) {
+                    wait_group(j);
+                    const uint32_t s = j % C::kR;
+                    const uint32_t ta = tbase + lanes + (uint32_t)C::kAccStride * s;
+                    const int y = it.ry + D * (it.m0 + j);
                     // features c = 0..63 -> logits z_k = b_k + sum_c W[k][c] f_c, in order of c
                     const float* hw = cst + N;
                     float z0 = hw[192], z1 = hw[193], z2 = hw[194];
@@ -393,50 +411,81 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                     const float m = fmaxf(z0, fmaxf(z1, z2));
                     const float e0 = expf(z0 - m), e1 = expf(z1 - m), e2 = expf(z2 - m);
                     const float den = e0 + e1 + e2;
-                    if (store) {
+                    if (x < p.out_w && !*abort_flag) {
                         float* o = p.probs + (int64_t)y * p.out_pitch + x;
                         o[0] = e0 / den;
                         o[p.probs_plane] = e1 / den;
                         o[2 * p.probs_plane] = e2 / den;
                     }
-                } else {
-                    // conv channels 2c, 2c+1 -> feature c; N/2 FP16 features = N/16 16-byte words
-                    uint32_t w[N / 4];
-#pragma unroll
-                    for (int q = 0; q < N / 32; ++q) {
-                        float v[32];
-                        ptx::tmem_ld32(ta + 32u * q, v);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int n = 32 * q + 4 * i;
-                            const float f0 = fmaxf(v[4 * i] + cst[n], v[4 * i + 1] + cst[n + 1]);
-                            const float f1 = fmaxf(v[4 * i + 2] + cst[n + 2], v[4 * i + 3] + cst[n + 3]);
-                            __half2 h2 = __floats2half2_rn(f0, f1);
-                            w[8 * q + i] = *reinterpret_cast<uint32_t*>(&h2);
-                        }
-                    }
-                    if constexpr (N % 32 != 0) {
-                        constexpr int q = N / 32;
-                        float v[16];
-                        ptx::tmem_ld16(ta + 32u * q, v);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int n = 32 * q + 4 * i;
-                            const float f0 = fmaxf(v[4 * i] + cst[n], v[4 * i + 1] + cst[n + 1]);
-                            const float f1 = fmaxf(v[4 * i + 2] + cst[n + 2], v[4 * i + 3] + cst[n + 3]);
-                            __half2 h2 = __floats2half2_rn(f0, f1);
-                            w[8 * q + i] = *reinterpret_cast<uint32_t*>(&h2);
-                        }
-                    }
-                    ptx::tc_fence_before();
-                    ptx::mbar_arrive(&acc_free[s]);
-                    if (store) {
-                        uint4* o = reinterpret_cast<uint4*>(p.out + ((int64_t)y * p.out_pitch + x) * (N / 2));
-#pragma unroll
-                        for (int i = 0; i < N / 16; ++i) o[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
-                    }
                 }
             }
+        } else {
+            // chunks C0 .. C0 + NC - 1: conv channels 16 C0 .. -> features 8 C0 ..
+            auto run = [&](auto c0_, auto nc_) {
+                constexpr int C0 = decltype(c0_)::value, NC = decltype(nc_)::value;
+                const int pw = warp & 3, bar = 2 + (C0 > 0);
+                uint4* xch = reinterpret_cast<uint4*>(smem + C::oXch) + C0 * 4 * D;
+                uint4 prev[NC];
+                uint32_t turn = 0;
+                while (me_next<D, C::kStrip>(p, cur, it)) {
+                    const int x = it.x0 + px;
+                    const bool col_ok = px < C::kStrip && x < p.out_w;
+                    for (int j = 0; j <= it.rows; ++j) {
+                        wait_group(j);
+                        const uint32_t s = j % C::kR;
+                        const uint32_t ta = tbase + lanes + (uint32_t)C::kAccStride * s + 16u * C0;
+                        uint4 w[NC];
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) {
+                            float v[16];
+                            ptx::tmem_ld16(ta + 16u * c, v);
+                            uint32_t r[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const float4 b = *reinterpret_cast<const float4*>(cst + 16 * (C0 + c) + 4 * i);
+                                const __half2 h2 = __floats2half2_rn(fmaxf(v[4 * i] + b.x, v[4 * i + 1] + b.y),
+                                                                     fmaxf(v[4 * i + 2] + b.z, v[4 * i + 3] + b.w));
+                                r[i] = *reinterpret_cast<const uint32_t*>(&h2);
+                            }
+                            w[c] = make_uint4(r[0], r[1], r[2], r[3]);
+                        }
+                        ptx::tc_fence_before();
+                        ptx::mbar_arrive(&acc_free[s]);
+                        if (j > 0) {
+                            // vertical maximum; then the horizontal partner: D lanes on, for the last D
+                            // lanes of a warp the next warp's first ones, through shared memory (two
+                            // buffers in turn, over item boundaries too: one rendezvous per row)
+                            uint4* xc = xch + turn * C::kOutChunks * 4 * D;
+                            turn ^= 1;
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) {
+                                prev[c] = hmax4(prev[c], w[c]);
+                                if (lane < D) xc[(c * 4 + pw) * D + lane] = prev[c];
+                            }
+                            asm volatile("bar.sync %0, 128;" ::"r"(bar) : "memory");
+                            __half* o = p.out + (((int64_t)(it.ry + D * (it.m0 + j - 1)) * C::kOutChunks + C0) * p.out_pitch + x) * 8;
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) {
+                                uint4 nb;
+                                nb.x = __shfl_down_sync(0xffffffffu, prev[c].x, D);
+                                nb.y = __shfl_down_sync(0xffffffffu, prev[c].y, D);
+                                nb.z = __shfl_down_sync(0xffffffffu, prev[c].z, D);
+                                nb.w = __shfl_down_sync(0xffffffffu, prev[c].w, D);
+                                if (lane >= 32 - D && pw < 3) nb = xc[(c * 4 + pw + 1) * D + lane - (32 - D)];
+                                if (col_ok && !*abort_flag)
+                                    *reinterpret_cast<uint4*>(o + (int64_t)c * p.out_pitch * 8) = hmax4(prev[c], nb);
+                            }
+                        }
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) prev[c] = w[c];
+                    }
+                }
+            };
+            constexpr int kFirst = (C::kOutChunks + 1) / 2;
+            if (warp < 8)
+                run(std::integral_constant<int, 0>{}, std::integral_constant<int, kFirst>{});
+            else
+                run(std::integral_constant<int, kFirst>{}, std::integral_constant<int, C::kOutChunks - kFirst>{});
         }
     } else if (warp == 1) {
         // ================= B producer: weight units, in the issuer's order ==========================
@@ -445,8 +494,8 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
             bool go = true;
             MeCursor cur = me_begin(p);
             MeItem it;
-            while (go && me_next<D>(p, cur, it)) {
-                const int groups = (it.rows + C::kR - 1) / C::kR;
+            while (go && me_next<D, C::kStrip>(p, cur, it)) {
+                const int groups = (it.rows + C::kMore + C::kR - 1) / C::kR;
                 for (int g = 0; go && g < groups; ++g)
                     for (int t0 = 0; go && t0 < 16; t0 += C::kBU) {
                         const uint32_t slot = issued % kMBRing;
@@ -471,55 +520,34 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
             }
         }
         __syncwarp();
-    } else if (warp >= 8) {
-        // ================= A producers: staged input rows ===========================================
-        // Group grp (kGroups groups of 8 / kGroups warps) stages the rows u = grp mod kGroups. Task
-        // e = pt + kGThreads i: chunk e % kChunks of staged pixel e / kChunks (consecutive threads read
-        // consecutive 16-byte chunks of one source pixel). All loads of a row are issued before the
-        // slot wait so their latency overlaps it.
-        const int grp = (tid - 256) / C::kGThreads;
-        const int pt = tid - 256 - C::kGThreads * grp;
-        const int64_t dxo = (int64_t)p.dm * p.cs, dyo = (int64_t)p.dm * p.in_pitch * p.cs;
-        const int src_chunks = p.cs / 8;
-        uint32_t a_seq = 0;
-        MeCursor cur = me_begin(p);
-        MeItem it;
-        while (me_next<D>(p, cur, it)) {
-            for (int u = grp; u < it.rows + 3; u += C::kGroups) {
-                const uint32_t q = a_seq + u, slot = q % C::kARing;
-                const int yin = it.ry + D * (it.m0 + u);
-                uint4 v[C::kATasks];
-#pragma unroll
-                for (int i = 0; i < C::kATasks; ++i) {
-                    const int e = pt + C::kGThreads * i;
-                    const int c = e % C::kChunks, xin = it.x0 + e / C::kChunks;
-                    v[i] = make_uint4(0, 0, 0, 0);
-                    if (e < C::kNpix * C::kChunks && c < src_chunks && yin < p.in_rows && xin < p.in_cols) {
-                        const __half* a = p.in + ((int64_t)yin * p.in_pitch + xin) * p.cs + c * 8;
-                        const uint4 r0 = __ldg(reinterpret_cast<const uint4*>(a));
-                        if (p.dm > 0) {
-                            const uint4 r1 = __ldg(reinterpret_cast<const uint4*>(a + dxo));
-                            const uint4 r2 = __ldg(reinterpret_cast<const uint4*>(a + dyo));
-                            const uint4 r3 = __ldg(reinterpret_cast<const uint4*>(a + dyo + dxo));
-                            v[i] = hmax4(hmax4(r0, r1), hmax4(r2, r3));
-                        } else {
-                            v[i] = r0;
-                        }
-                    }
+    } else if (warp == 2) {
+        // ================= A loader: staged input rows ==============================================
+        if (lane == 0) {
+            uint32_t q = 0;
+            bool go = !p.fault_stall;
+            MeCursor cur = me_begin(p);
+            MeItem it;
+            while (go && me_next<D, C::kStrip>(p, cur, it)) {
+                const int nst = it.rows + C::kMore + 3;
+                for (int u = 0; u < nst; ++u, ++q) {
+                    const uint32_t slot = q % C::kARing;
+                    go = wait_bar(&a_empty[slot], ((q / C::kARing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
+                    if (!go) break;
+                    const __half* row =
+                        p.in + ((int64_t)(it.ry + D * (it.m0 + u)) * p.src_chunks * p.in_pitch + it.x0) * 8;
+                    ptx::mbar_arrive_expect_tx(&a_full[slot], (uint32_t)(p.src_chunks * C::kMP * 16));
+                    for (int c = 0; c < p.src_chunks; ++c)
+                        ptx::bulk_copy_g2s(smem + C::oA + slot * C::kARow + c * C::kMP * 16,
+                                           row + (int64_t)c * p.in_pitch * 8, C::kMP * 16, &a_full[slot]);
                 }
-                wait_bar(&a_empty[slot], ((q / C::kARing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
-                uint8_t* dst = smem + C::oA + slot * C::kARow;
-#pragma unroll
-                for (int i = 0; i < C::kATasks; ++i) {
-                    const int e = pt + C::kGThreads * i;
-                    if (e < C::kNpix * C::kChunks)
-                        *reinterpret_cast<uint4*>(dst + ((e % C::kChunks) * C::kMP + e / C::kChunks) * 16) = v[i];
-                }
-                ptx::fence_proxy_async_smem();
-                if (!p.fault_stall) ptx::mbar_arrive(&a_full[slot]);
             }
-            a_seq += it.rows + 3;
+            // the copies still in flight land before the CTA exits (bounded, abort or not)
+            const uint64_t t0 = gtime();
+            for (uint32_t r = q > (uint32_t)C::kARing ? q - C::kARing : 0; r < q; ++r)
+                while (!ptx::mbar_test(&a_full[r % C::kARing], (r / C::kARing) & 1) && gtime() - t0 <= p.wait_ns) {
+                }
         }
+        __syncwarp();
     }
 
     ptx::tc_fence_before();
@@ -569,8 +597,8 @@ mb_status launch_me_tc(const MeTcParams& p, cudaStream_t st) {
                                      C::kSmem));
         attr = true;
     }
-    // one range per SM, or fewer when a range would get under 8 rows
-    const int grid = std::max(1, std::min(n_sms, (p.total_rows + 7) / 8));
+    // one range per SM, or fewer when a range would get under 2 rows
+    const int grid = std::max(1, std::min(n_sms, (p.total_rows + 1) / 2));
     me_tc_conv<KC, N, D, HEAD><<<grid, kMThreads, C::kSmem, st>>>(p);
     count_launch();
     MB_CUDA(cudaGetLastError());
@@ -649,21 +677,27 @@ mb_status me_tc_poll_error(mb_net* net) {
     return MB_OK;
 }
 
-// Rows per work item: the cost of a launch is taken as waves x (rows + 5) staged-row steps (3 rows
-// of context and ~2 of pipeline fill per item); the smallest cost wins, ties to more rows.
+static const int kMeD[5] = {1, 2, 4, 8, 16};
 
-mb_status me_tc_layer(mb_net* net, int layer, const void* in, int64_t in_pitch, int cs, int in_rows, int in_cols,
-                      int dm, void* out, int64_t out_pitch, int out_h, int out_w, float* probs, int64_t probs_plane,
-                      cudaStream_t st) {
+static int me_tc_strips(int layer, int64_t cols) {
+    const int strip = layer == 4 ? 128 : 128 - kMeD[layer];
+    return (int)((cols + strip - 1) / strip);
+}
+
+int64_t me_tc_in_pitch(int layer, int64_t cols) {
+    const int d = kMeD[layer], strip = layer == 4 ? 128 : 128 - d;
+    return (int64_t)(me_tc_strips(layer, cols) - 1) * strip + 128 + 3 * d;
+}
+
+mb_status me_tc_layer(mb_net* net, int layer, const void* in, int64_t in_pitch, void* out, int64_t out_pitch, int rows,
+                      int cols, float* probs, int64_t probs_plane, cudaStream_t st) {
     MeTcState* S = reinterpret_cast<MeTcState*>(net->me_state);
     if (!S || !S->d_wpack[layer]) {
         set_error("MaskExtend tensor-core weights not prepared");
         return MB_ERR_NOT_READY;
     }
-    static const int kD[5] = {1, 2, 4, 8, 16};
-    const int d = kD[layer];
-    if (cs % 8 != 0 || cs > 16 * kMeKc[layer] || in_rows < out_h + 3 * d || in_cols < out_w + 3 * d) {
-        set_error("MaskExtend: inconsistent layer geometry");
+    if (in_pitch < me_tc_in_pitch(layer, cols)) {
+        set_error("MaskExtend: feature pitch too small");
         return MB_ERR_INVALID_ARG;
     }
     MeTcParams p{};
@@ -675,18 +709,15 @@ mb_status me_tc_layer(mb_net* net, int layer, const void* in, int64_t in_pitch, 
     p.in_pitch = in_pitch;
     p.out_pitch = out_pitch;
     p.probs_plane = probs_plane;
-    p.cs = cs;
-    p.in_rows = in_rows;
-    p.in_cols = in_cols;
-    p.out_h = out_h;
-    p.out_w = out_w;
-    p.dm = dm;
-    p.n_strips = (out_w + 127) / 128;
-    if ((int64_t)p.n_strips * out_h > 0x7fffffffLL) {
+    p.src_chunks = layer == 0 ? 2 : (kMeCin[layer] + 7) / 8;
+    p.out_h = rows;
+    p.out_w = cols;
+    p.n_strips = me_tc_strips(layer, cols);
+    if ((int64_t)p.n_strips * rows > 0x7fffffffLL) {
         set_error("MaskExtend: too many strip-rows for one launch");
         return MB_ERR_SHAPE;
     }
-    p.total_rows = p.n_strips * out_h;
+    p.total_rows = p.n_strips * rows;
     const char* stall = getenv("MB_FAULT_STALL");
     p.fault_stall = (stall && stall[0] == '1') ? 1 : 0;
     p.wait_ns = p.fault_stall ? 200000000ull : kMWaitNs;
