@@ -31,7 +31,7 @@
 // maps are bitwise those of filtering on the load.
 //
 // Warp roles (384 threads, 1 CTA per SM, persistent over work items):
-//   warp 0       TMEM owner; lane 0 issues the MMAs
+//   warps 0, 3   lane 0 issues the MMAs of the even / odd rows of a group (warp 0 also owns TMEM)
 //   warp 1       lane 0 streams the weight units into their ring with bulk copies (completion counted
 //                on the unit's mbarrier)
 //   warp 2       lane 0 fetches the staged rows (as many ahead as shared memory allows, up to 12)
@@ -81,14 +81,14 @@ struct MCfg {
     static constexpr int kEpi = HEAD ? 128 : 256;        // epilogue threads
     static constexpr int kStrip = HEAD ? 128 : 128 - D;  // output columns of a strip
     static constexpr int kMore = HEAD ? 0 : 1;           // conv rows of an item beyond its output rows
-    static constexpr int kFixed = kMBRing * kBUnit + kXch + kConsts * 4 + 16 + (2 * kMBRing + kR + 2) * 8 + 16;
+    static constexpr int kFixed = kMBRing * kBUnit + kXch + kConsts * 4 + 16 + (2 * kMBRing + kR + 3) * 8 + 16;
     static constexpr int kARing = (227 * 1024 - kFixed) / (kARow + 16) < 12 ? (227 * 1024 - kFixed) / (kARow + 16) : 12;
     static constexpr int oA = 0;
     static constexpr int oB = oA + kARing * kARow;
     static constexpr int oXch = oB + kMBRing * kBUnit;
     static constexpr int oConst = oXch + kXch;
     static constexpr int oBar = oConst + ((kConsts * 4 + 15) & ~15);
-    static constexpr int kBars = 2 * kARing + 2 * kMBRing + 1 + kR + 1;
+    static constexpr int kBars = 2 * kARing + 2 * kMBRing + 1 + kR + 2;
     static constexpr int oMisc = oBar + kBars * 8;
     static constexpr int kSmem = oMisc + 16;
     static_assert(kARing >= kR + 1, "staged-row ring");
@@ -107,6 +107,7 @@ struct MeTcParams {
     int out_h, out_w;       // what is written: filtered features; the head: the maps
     int n_strips;
     int total_rows;         // strip-rows of the launch: n_strips x out_h (< 2^31, checked)
+    int per_cta, extra;     // total_rows = per_cta x CTAs + extra: the first `extra` CTAs take one more
     int fault_stall;        // test injection: the loaders withhold their copies
     uint64_t wait_ns;
 };
@@ -153,8 +154,9 @@ struct MeCursor {
 
 __device__ __forceinline__ MeCursor me_begin(const MeTcParams& p) {
     MeCursor c;
-    c.g = (int)((int64_t)p.total_rows * blockIdx.x / gridDim.x);
-    c.hi = (int)((int64_t)p.total_rows * (blockIdx.x + 1) / gridDim.x);
+    const int b = blockIdx.x;
+    c.g = b * p.per_cta + min(b, p.extra);
+    c.hi = c.g + p.per_cta + (b < p.extra ? 1 : 0);
     return c;
 }
 
@@ -200,21 +202,23 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::oMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::oMisc + 4);
     const float* cst = reinterpret_cast<const float*>(smem + C::oConst);
+    ptx::grid_dep_launch();  // the next launch may set itself up on SMs that are done
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the same in all lanes
 
     if (tid == 0) {
         for (int i = 0; i < C::kARing; ++i) {
             ptx::mbar_init(&a_full[i], 1);
-            ptx::mbar_init(&a_empty[i], 1);
+            ptx::mbar_init(&a_empty[i], 2);
         }
         for (int i = 0; i < kMBRing; ++i) {
             ptx::mbar_init(&b_full[i], 1);
-            ptx::mbar_init(&b_empty[i], 1);
+            ptx::mbar_init(&b_empty[i], 2);
         }
-        ptx::mbar_init(acc_full, 1);
+        ptx::mbar_init(acc_full, 2);
         for (int i = 0; i < C::kR; ++i) ptx::mbar_init(&acc_free[i], C::kEpi);
         ptx::mbar_init(fin, 1);
+        ptx::mbar_init(fin + 1, 1);
         *abort_flag = 0;
         ptx::mbar_fence_init();
     }
@@ -239,10 +243,13 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
     const uint32_t tbase = *tmem_slot;
     const uint32_t sbase = ptx::smem_u32(smem);
 
-    if (warp == 0) {
-        // ================= MMA issuer ================================================================
+    if (warp == 0 || warp == 3) {
+        // ================= MMA issuers ================================================================
         // The whole warp walks the loop on uniform values, lane 0 issuing: a divergent branch would
-        // move every operand of every MMA through vector registers.
+        // move every operand of every MMA through vector registers. One thread issues an MMA per 80-93
+        // cycles, the tensor pipe takes one per 48 (N = 64) to 64 (N = 128); a row's accumulator is its
+        // own, so two warps share the rows of a group (each accumulator's MMAs stay in one thread's order).
+            const int odd = warp == 3;
             const uint64_t adesc = ptx::smem_desc(sbase + C::oA, C::kMP * 16, 128);
             const uint64_t bdesc = ptx::smem_desc(sbase + C::oB, N * 16, 128);
             const uint32_t adesc0 = (uint32_t)adesc, a_hi = (uint32_t)(adesc >> 32);
@@ -258,16 +265,19 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
             // before it). Rows are runtime loops and only taps and K chunks are unrolled (the tap
             // shift D kx and the chunk kc are compile-time offsets): a short issue loop stays in
             // the instruction cache beside the other roles' code.
-            auto mma_taps = [&](uint32_t ad, uint32_t dcol, uint32_t bd, auto kx0, auto ntaps, bool zero_first) {
+            auto mma_taps = [&](uint32_t ad, uint32_t dcol, uint32_t bd, auto kx0, auto ntaps, auto zero_first) {
                 const uint32_t on = ok ? lead : 0u;
 #pragma unroll
                 for (int t = 0; t < decltype(ntaps)::value; ++t)
 #pragma unroll
                     for (int kc = 0; kc < KC; ++kc) {
                         const int kx = decltype(kx0)::value + t;
-                        ptx::mma_bf16_acc(on, dcol, ad + (uint32_t)((D * kx * 16 + kc * 2 * C::kMP * 16) >> 4), a_hi,
-                                          bd + (uint32_t)(((kx % kBU) * C::kBTap + kc * 2 * N * 16) >> 4), b_hi, idesc,
-                                          (zero_first && t == 0 && kc == 0) ? 0u : 1u);
+                        const uint32_t al = ad + (uint32_t)((D * kx * 16 + kc * 2 * C::kMP * 16) >> 4);
+                        const uint32_t bl = bd + (uint32_t)(((kx % kBU) * C::kBTap + kc * 2 * N * 16) >> 4);
+                        if (decltype(zero_first)::value && t == 0 && kc == 0)
+                            ptx::mma_bf16_acc(on, dcol, al, a_hi, bl, b_hi, idesc, 0u);
+                        else
+                            ptx::mma_bf16_if(on, dcol, al, a_hi, bl, b_hi, idesc);
                     }
             };
             auto unit_desc = [&](uint32_t q) { return bdesc0 + (((q % kMBRing) * C::kBUnit) >> 4); };
@@ -302,7 +312,7 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                             // only for its own accumulator
                             for (int u = 0; u < 4 / kBU; ++u) wait_unit(u_seq + u);
                             const uint32_t bd0 = unit_desc(u_seq), bd1 = unit_desc(u_seq + (4 / kBU) - 1);
-                            for (int j = 0; j < rg; ++j) {
+                            for (int j = odd; j < rg; j += 2) {
                                 ok = ok && wait_bar(&acc_free[j], ((free_par >> j) & 1) ^ 1, abort_flag, p.err,
                                                     p.wait_ns);
                                 free_par ^= 1u << j;
@@ -312,12 +322,12 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                                 {
                                     if constexpr (kBU == 4) {
                                         mma_taps(ad, dcol, bd0, std::integral_constant<int, 0>{},
-                                                 std::integral_constant<int, 4>{}, true);
+                                                 std::integral_constant<int, 4>{}, std::true_type{});
                                     } else {
                                         mma_taps(ad, dcol, bd0, std::integral_constant<int, 0>{},
-                                                 std::integral_constant<int, 2>{}, true);
+                                                 std::integral_constant<int, 2>{}, std::true_type{});
                                         mma_taps(ad, dcol, bd1, std::integral_constant<int, 2>{},
-                                                 std::integral_constant<int, 2>{}, false);
+                                                 std::integral_constant<int, 2>{}, std::false_type{});
                                     }
                                 }
                             }
@@ -329,18 +339,18 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                                 ptx::tc_fence_after();
                                 const uint32_t bd = unit_desc(u_seq);
                                 {
-                                    for (int j = 0; j < rg; ++j) {
+                                    for (int j = odd; j < rg; j += 2) {
                                         const uint32_t ad = arow(j);
                                         const uint32_t dcol = tbase + (uint32_t)(C::kAccStride * j);
                                         if constexpr (kBU == 4) {
                                             mma_taps(ad, dcol, bd, std::integral_constant<int, 0>{},
-                                                     std::integral_constant<int, 4>{}, false);
+                                                     std::integral_constant<int, 4>{}, std::false_type{});
                                         } else if (u == 0) {
                                             mma_taps(ad, dcol, bd, std::integral_constant<int, 0>{},
-                                                     std::integral_constant<int, 2>{}, false);
+                                                     std::integral_constant<int, 2>{}, std::false_type{});
                                         } else {
                                             mma_taps(ad, dcol, bd, std::integral_constant<int, 2>{},
-                                                     std::integral_constant<int, 2>{}, false);
+                                                     std::integral_constant<int, 2>{}, std::false_type{});
                                         }
                                     }
                                 }
@@ -358,9 +368,10 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
                 a_seq += rows + 3;
             }
             if (lane == 0) {
-                ptx::mma_commit(fin);
+                uint64_t* my = fin + odd;
+                ptx::mma_commit(my);
                 const uint64_t t0 = gtime();
-                while (!ptx::mbar_test(fin, 0)) {
+                while (!ptx::mbar_test(my, 0)) {
                     if (gtime() - t0 > p.wait_ns) {
                         *(volatile int*)p.err = MB_ERR_TIMEOUT;
                         break;
@@ -522,26 +533,30 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
         __syncwarp();
     } else if (warp == 2) {
         // ================= A loader: staged input rows ==============================================
-        if (lane == 0) {
-            uint32_t q = 0;
-            bool go = !p.fault_stall;
-            MeCursor cur = me_begin(p);
-            MeItem it;
-            while (go && me_next<D, C::kStrip>(p, cur, it)) {
-                const int nst = it.rows + C::kMore + 3;
-                for (int u = 0; u < nst; ++u, ++q) {
-                    const uint32_t slot = q % C::kARing;
-                    go = wait_bar(&a_empty[slot], ((q / C::kARing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
-                    if (!go) break;
-                    const __half* row =
-                        p.in + ((int64_t)(it.ry + D * (it.m0 + u)) * p.src_chunks * p.in_pitch + it.x0) * 8;
-                    ptx::mbar_arrive_expect_tx(&a_full[slot], (uint32_t)(p.src_chunks * C::kMP * 16));
-                    for (int c = 0; c < p.src_chunks; ++c)
-                        ptx::bulk_copy_g2s(smem + C::oA + slot * C::kARow + c * C::kMP * 16,
-                                           row + (int64_t)c * p.in_pitch * 8, C::kMP * 16, &a_full[slot]);
-                }
+        // (lane c fetches chunk c: one thread's 2 to 7 copies per row took 540-950 cycles)
+        uint32_t q = 0;
+        bool go = !p.fault_stall;
+        ptx::grid_dep_wait();  // the rows are the previous launch's output
+        MeCursor cur = me_begin(p);
+        MeItem it;
+        while (go && me_next<D, C::kStrip>(p, cur, it)) {
+            const int nst = it.rows + C::kMore + 3;
+            for (int u = 0; u < nst; ++u, ++q) {
+                const uint32_t slot = q % C::kARing;
+                go = wait_bar(&a_empty[slot], ((q / C::kARing) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
+                go = __all_sync(0xffffffffu, go);
+                if (!go) break;
+                if (lane == 0) ptx::mbar_arrive_expect_tx(&a_full[slot], (uint32_t)(p.src_chunks * C::kMP * 16));
+                __syncwarp();
+                if (lane < p.src_chunks)
+                    ptx::bulk_copy_g2s(
+                        smem + C::oA + slot * C::kARow + lane * C::kMP * 16,
+                        p.in + (((int64_t)(it.ry + D * (it.m0 + u)) * p.src_chunks + lane) * p.in_pitch + it.x0) * 8,
+                        C::kMP * 16, &a_full[slot]);
             }
-            // the copies still in flight land before the CTA exits (bounded, abort or not)
+        }
+        // the copies still in flight land before the CTA exits (bounded, abort or not)
+        if (lane == 0) {
             const uint64_t t0 = gtime();
             for (uint32_t r = q > (uint32_t)C::kARing ? q - C::kARing : 0; r < q; ++r)
                 while (!ptx::mbar_test(&a_full[r % C::kARing], (r / C::kARing) & 1) && gtime() - t0 <= p.wait_ns) {
@@ -583,7 +598,7 @@ void me_tc_pack(const float* W, const float* b, int cin, int n, int kc, const fl
 }
 
 template <int KC, int N, int D, bool HEAD>
-mb_status launch_me_tc(const MeTcParams& p, cudaStream_t st) {
+mb_status launch_me_tc(const MeTcParams& q, cudaStream_t st) {
     using C = MCfg<KC, N, D, HEAD>;
     static int n_sms = 0;
     if (n_sms == 0) {
@@ -598,8 +613,23 @@ mb_status launch_me_tc(const MeTcParams& p, cudaStream_t st) {
         attr = true;
     }
     // one range per SM, or fewer when a range would get under 2 rows
-    const int grid = std::max(1, std::min(n_sms, (p.total_rows + 1) / 2));
-    me_tc_conv<KC, N, D, HEAD><<<grid, kMThreads, C::kSmem, st>>>(p);
+    const int grid = std::max(1, std::min(n_sms, (q.total_rows + 1) / 2));
+    MeTcParams p = q;
+    p.per_cta = q.total_rows / grid;
+    p.extra = q.total_rows % grid;
+    // the launch's set-up (barriers, constants, TMEM, the first weights) overlaps the end of the one
+    // before it; its rows are read after that one's completion (grid_dep_wait)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kMThreads);
+    cfg.dynamicSmemBytes = C::kSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    MB_CUDA(cudaLaunchKernelEx(&cfg, me_tc_conv<KC, N, D, HEAD>, p));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;

@@ -53,6 +53,13 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void* gptr, uint32_t byte
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gptr), "r"(bytes) : "memory");
 }
 
+// ---- programmatic dependent launch -----------------------------------------------------------------
+// The launch after this one in the stream may start on free SMs (it waits for this one's completion in
+// grid_dep_wait before it touches anything that this one reads or writes).
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Until every launch that this one depends on has completed and its writes are visible.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- proxy / tcgen05 fences ---------------------------------------------------------------------
 // Generic-proxy shared-memory writes become visible to the async proxy (tcgen05.mma operands).
 __device__ __forceinline__ void fence_proxy_async_smem() {
