@@ -412,15 +412,18 @@ void x3_pack(const float* W, const float* b, int c0, const float* head, std::vec
     out.resize(base + C::kBBytes + 256, 0);
     uint8_t* o = out.data() + base;
     for (int c = 0; c < 32; ++c)
-        for (int ci = 0; ci < 32; ++ci) {
-            const int h = ci / 16, kc = (ci % 16) / 8, e = ci % 8;
-            const float* w = W + ((size_t)(c0 + c) * 32 + ci) * K * K;
-            uint8_t* at = o + h * C::kBlock + kc * C::kN * 16 + c * 16 + 2 * e;
+        for (int g = 0; g < 4; ++g) {  // input channels 8 g .. 8 g + 7: one 16-byte chunk per (part, tap)
+            const float* w = W + ((size_t)(c0 + c) * 32 + 8 * g) * K * K;
+            uint8_t* at = o + (g / 2) * C::kBlock + (g % 2) * C::kN * 16 + c * 16;
             for (int ky = 0; ky < K; ++ky)
                 for (int kx = 0; kx < K; ++kx) {
-                    float v = w[ky * K + kx];
+                    uint16_t v[3][8];
+                    for (int e = 0; e < 8; ++e) {
+                        float f = w[e * K * K + ky * K + kx];
+                        for (int i = 0; i < 3; ++i) v[i][e] = part_bits(f);
+                    }
                     for (int i = 0; i < 3; ++i)
-                        *reinterpret_cast<uint16_t*>(at + (i * C::kGroups + kx * 2) * C::kBlock + 32 * ky * 16) = part_bits(v);
+                        memcpy(at + (i * C::kGroups + kx * 2) * C::kBlock + 32 * ky * 16, v[i], 16);
                 }
         }
     memcpy(o + C::kBBytes, b + c0, 32 * 4);
@@ -450,7 +453,7 @@ mb_status launch_x3(XParams& p, cudaStream_t st) {
 }
 
 struct X3State {
-    uint8_t* d_w[4] = {};  // the packed layers
+    uint8_t* d_w[4] = {};  // the packed layers, parts of one allocation (d_w[0])
     int* h_err = nullptr;
     int* d_err = nullptr;
     float hb = 0.f;
@@ -497,8 +500,9 @@ mb_status x3_prepare(mb_net* net) {
     if (!x3_bounded(net)) return MB_OK;
     const int n = teacher ? 2 : fastmemb_convs(net->family) - 2;
     const float* P = net->host_params.data() + (teacher ? 832 : 64 * 16 + 64);
+    std::vector<uint8_t> pk;
+    size_t at[5] = {};
     for (int l = 0; l < n; ++l) {
-        std::vector<uint8_t> pk;
         if (teacher) {
             x3_pack<5>(P, P + 25600, 0, l == 1 ? P + 25600 + 32 : nullptr, pk);
             P += 25600 + 32;
@@ -507,9 +511,11 @@ mb_status x3_prepare(mb_net* net) {
             x3_pack<4>(P, P + 64 * 32 * 16, 32, nullptr, pk);
             P += 64 * 32 * 16 + 64;
         }
-        if (!S->d_w[l]) MB_TRY(dev_alloc((void**)&S->d_w[l], pk.size()));
-        MB_CUDA(cudaMemcpy(S->d_w[l], pk.data(), pk.size(), cudaMemcpyHostToDevice));
+        at[l + 1] = pk.size();
     }
+    if (!S->d_w[0]) MB_TRY(dev_alloc((void**)&S->d_w[0], pk.size()));
+    for (int l = 1; l < n; ++l) S->d_w[l] = S->d_w[0] + at[l];
+    MB_CUDA(cudaMemcpy(S->d_w[0], pk.data(), pk.size(), cudaMemcpyHostToDevice));
     if (teacher) S->hb = P[32];
     if (!S->h_err) {
         if (fault_oom()) {
@@ -527,7 +533,7 @@ mb_status x3_prepare(mb_net* net) {
 void x3_release(mb_net* net) {
     X3State* S = x3_of(net);
     if (!S) return;
-    for (uint8_t* w : S->d_w) dev_free(w);
+    dev_free(S->d_w[0]);
     if (S->h_err) cudaFreeHost(S->h_err);
     delete S;
     net->x3_state = nullptr;

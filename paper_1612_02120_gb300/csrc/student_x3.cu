@@ -11,12 +11,14 @@
 //
 // st_x3 reads one 64-byte pixel of h1 or dy2 per output pixel, once, and the forward writes dy2 once
 // (h2 and dy1 exist in registers only): a row of 128 pixels costs ~500 cycles of MMAs and 360-710 of
-// HBM time; 1,320-1,620 measured (370 us a pass on a batch of 32 x 512 x 512), the epilogue's chain.
+// HBM time; 1,290-1,590 measured (forward 358 us, backward 364 on a batch of 32 x 512 x 512; 370 each with
+// remainders in the issue loop and a third turn for one producer warp): the issuing warp's and the epilogue's chains.
 // The separate kernels (conv 865 us, head and loss 218, data gradient 1,023, conv1's weight gradient
 // 395 on a batch of 32 x 512 x 512) passed 3.2 GB through HBM at 0.47-0.55 of the FP32 FMA rate.
 //
 // Warp roles of st_x3 (512 threads, 1 CTA per SM, one equal contiguous range of strip-rows per CTA):
-//   warp 0        lane 0 issues the MMAs
+//   warp 0        issues the MMAs (whole warp on uniform values, lane 0 issuing)
+//   warp 1        producer of the row's last two pixels
 //   warps 4-11    epilogue, two groups of 8 channels, one pixel column per thread; sums over pixels
 //                 (loss, head, bias and conv1 weight gradients) stay in registers until the end
 //   warps 12-15   producers: load 8 channels of a pixel, split, store 3 x 16 B
@@ -26,6 +28,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "f32_split.cuh"
 #include "internal.h"
@@ -130,12 +133,12 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
 
     if (tid == 0) {
         for (int i = 0; i < kRingX; ++i) {
-            ptx::mbar_init(&row_full[i], 128);
+            ptx::mbar_init(&row_full[i], 5);
             ptx::mbar_init(&row_empty[i], 1);
         }
         for (int i = 0; i < kBufsX; ++i) {
             ptx::mbar_init(&acc_full[i], 1);
-            ptx::mbar_init(&acc_free[i], 256);
+            ptx::mbar_init(&acc_free[i], 8);
         }
         ptx::mbar_init(fin, 1);
         *abort_flag = 0;
@@ -162,31 +165,105 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
     SxItem it;
     static_assert(40 + 2 * 176 + 120 <= 4 * 128, "register budget exceeds the launch allocation");
 
+    // Producer of kTasks tasks a thread, from e = first on, 128 apart: 8 channels (e & 1) of pixel e >> 1
+    // of every staged row. The loads of the row after next are issued before this row's are split (two
+    // rows in flight). Warps 12-15 take the 256 tasks of pixels 0..127, a lane each and two in turn; the four
+    // of pixels 128 and 129 are warp 1's (a third turn for them made one producer warp the slowest role).
+    auto produce = [&](auto tasks, int first) {
+        constexpr int kTasks = decltype(tasks)::value;
+        const int off = BWD ? -2 : 0, src_h = BWD ? p.H : p.H + 2, src_w = BWD ? p.W : p.W + 2;
+        uint32_t s = 0, ph = 0;
+        while (sx_next(p, pos, end, it)) {
+            const int nst = it.rows + 2;
+            const float* src = p.in + (int64_t)it.z * src_h * src_w * 16;
+            float4 v[2][kTasks][2];
+            auto load = [&](int u, float4 (&d)[kTasks][2]) {
+                const int y = it.y0 + u + off;
+#pragma unroll
+                for (int i = 0; i < kTasks; ++i) {
+                    const int e = first + 128 * i, x = it.x0 + (e >> 1) + off;
+                    d[i][0] = d[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (e < 2 * 130 && u < nst && y >= 0 && y < src_h && x >= 0 && x < src_w) {
+                        const float4* a = reinterpret_cast<const float4*>(src + ((int64_t)y * src_w + x) * 16 + (e & 1) * 8);
+                        d[i][0] = __ldg(a);
+                        d[i][1] = __ldg(a + 1);
+                    }
+                }
+            };
+            auto put = [&](int u, float4 (&d)[kTasks][2]) {
+                if (u >= nst) return;
+                x_wait(&row_empty[s], ph ^ 1, abort_flag, p.err, p.wait_ns);
+                uint8_t* dst = smem + oRingX + s * kSlotX;
+#pragma unroll
+                for (int i = 0; i < kTasks; ++i) {
+                    const int e = first + 128 * i;
+                    if (e < 2 * 130) {
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            uint4 w;
+                            w.x = take_part(d[i][0].x, d[i][0].y);
+                            w.y = take_part(d[i][0].z, d[i][0].w);
+                            w.z = take_part(d[i][1].x, d[i][1].y);
+                            w.w = take_part(d[i][1].z, d[i][1].w);
+                            *reinterpret_cast<uint4*>(dst + k * kPart + ((e & 1) * kP + (e >> 1)) * 16) = w;
+                        }
+                    }
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0 && !p.fault_stall) ptx::mbar_arrive(&row_full[s]);
+                if (++s == kRingX) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            };
+            load(0, v[0]);
+            load(1, v[1]);
+            for (int u = 0; u < nst; u += 2) {
+                put(u, v[0]);
+                load(u + 2, v[0]);
+                put(u + 1, v[1]);
+                load(u + 3, v[1]);
+            }
+        }
+    };
+
     if (warp < 4) {
         ptx::setmaxnreg_dec<40>();
+        if (warp == 1) produce(std::integral_constant<int, 1>{}, 256 + lane);
         if (warp == 0) {
             // ================= MMA issuer ============================================================
             const uint64_t adesc = ptx::smem_desc(sbase + oRingX, kP * 16, 128);
             const uint64_t bdesc = ptx::smem_desc(sbase + oBx, kNx * 16, 128);
             const uint32_t a_hi = (uint32_t)(adesc >> 32), b_hi = (uint32_t)(bdesc >> 32);
             const uint32_t lead = lane == 0;
-            uint32_t q = 0;
+            // running ring positions (slot and phase): this warp's own chain of instructions is what
+            // bounds a row once the producers keep up, and a remainder or quotient costs several
+            uint32_t rs = 0, rph = 0, as = 0, aph = 0;  // next staged row's slot, next accumulator
             bool ok = true;
-            auto wait_row = [&](uint32_t r) {
-                ok = ok && x_wait(&row_full[r % kRingX], (r / kRingX) & 1, abort_flag, p.err, p.wait_ns);
-                ok = ok && x_wait(&acc_free[r % kBufsX], ((r / kBufsX) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
-            };
-            auto commit_row = [&](uint32_t r) {
-                ptx::mma_commit_if(lead, &row_empty[r % kRingX]);
-                ptx::mma_commit_if(lead, &acc_full[r % kBufsX]);
+            auto wait_row = [&] {
+                ok = ok && x_wait(&row_full[rs], rph, abort_flag, p.err, p.wait_ns);
+                ok = ok && x_wait(&acc_free[as], aph ^ 1, abort_flag, p.err, p.wait_ns);
             };
             while (sx_next(p, pos, end, it)) {
-                const int nst = it.rows + 2;
-                wait_row(q);
-                for (int u = 0; u < nst; ++u, ++q) {
+                const int nst = __shfl_sync(0xffffffffu, it.rows, 0) + 2;
+                uint64_t* last_empty = nullptr;
+                uint64_t* last_full = nullptr;
+                wait_row();
+                for (int u = 0; u < nst; ++u) {
                     ptx::tc_fence_after();
-                    const uint32_t on = ok ? lead : 0u, d = tbase + (q % kBufsX) * kNx;
-                    const uint32_t a = (uint32_t)adesc + (((q % kRingX) * kSlotX) >> 4);
+                    const uint32_t on = ok ? lead : 0u, d = tbase + as * kNx;
+                    const uint32_t a = (uint32_t)adesc + rs * (uint32_t)(kSlotX >> 4);
+                    uint64_t* my_empty = &row_empty[rs];
+                    uint64_t* my_full = &acc_full[as];
+                    if (++rs == kRingX) {
+                        rs = 0;
+                        rph ^= 1;
+                    }
+                    if (++as == kBufsX) {
+                        as = 0;
+                        aph ^= 1;
+                    }
 #pragma unroll
                     for (int kx = 0; kx < 3; ++kx) {
                         const uint32_t b = (uint32_t)bdesc + ((kx * 2 * kNx * 16) >> 4);
@@ -196,11 +273,17 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
                                          ptx::idesc_f32acc(ptx::kFmtBF16, 128, 96));
                         ptx::mma_bf16_if(on, d + 96, a + (2 * kPart >> 4) + kx, a_hi, b, b_hi,
                                          ptx::idesc_f32acc(ptx::kFmtBF16, 128, 48));
-                        if (kx == 0 && u > 0) commit_row(q - 1);
-                        if (kx == 1 && u + 1 < nst) wait_row(q + 1);
+                        if (kx == 0 && u > 0) {
+                            ptx::mma_commit_if(lead, last_empty);
+                            ptx::mma_commit_if(lead, last_full);
+                        }
+                        if (kx == 1 && u + 1 < nst) wait_row();
                     }
+                    last_empty = my_empty;
+                    last_full = my_full;
                 }
-                commit_row(q - 1);
+                ptx::mma_commit_if(lead, last_empty);
+                ptx::mma_commit_if(lead, last_full);
             }
             if (lane == 0) x_drain(fin, p.err, p.wait_ns);
             __syncwarp();
@@ -231,7 +314,8 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
 #pragma unroll
                 for (int m = 0; m < 3; ++m) ptx::keep8(v[k][m]);
             ptx::tc_fence_before();
-            ptx::mbar_arrive(&acc_free[bf]);
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&acc_free[bf]);
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 done[c] = s1[c] + (v[2][0][c] + (v[2][1][c] + v[2][2][c]));
@@ -403,62 +487,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
     } else {
         ptx::setmaxnreg_dec<120>();
         // ================= producers ==================================================================
-        // Tasks e = pt + 128 i: 8 channels (e & 1) of pixel e >> 1. Each thread's loads of the row
-        // after next are issued before this row's are split (two rows in flight).
-        const int pt = tid - 384;
-        constexpr int kTasks = 3;  // ceil(2 * 130 / 128)
-        const int off = BWD ? -2 : 0, src_h = BWD ? p.H : p.H + 2, src_w = BWD ? p.W : p.W + 2;
-        uint32_t q = 0;
-        while (sx_next(p, pos, end, it)) {
-            const int nst = it.rows + 2;
-            const float* src = p.in + (int64_t)it.z * src_h * src_w * 16;
-            float4 v[2][kTasks][2];
-            auto load = [&](int u, float4 (&d)[kTasks][2]) {
-                const int y = it.y0 + u + off;
-#pragma unroll
-                for (int i = 0; i < kTasks; ++i) {
-                    const int e = pt + 128 * i, x = it.x0 + (e >> 1) + off;
-                    d[i][0] = d[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (e < 2 * 130 && u < nst && y >= 0 && y < src_h && x >= 0 && x < src_w) {
-                        const float4* a = reinterpret_cast<const float4*>(src + ((int64_t)y * src_w + x) * 16 + (e & 1) * 8);
-                        d[i][0] = __ldg(a);
-                        d[i][1] = __ldg(a + 1);
-                    }
-                }
-            };
-            auto put = [&](int u, float4 (&d)[kTasks][2]) {
-                if (u >= nst) return;
-                const uint32_t s = q % kRingX;
-                x_wait(&row_empty[s], ((q / kRingX) & 1) ^ 1, abort_flag, p.err, p.wait_ns);
-                uint8_t* dst = smem + oRingX + s * kSlotX;
-#pragma unroll
-                for (int i = 0; i < kTasks; ++i) {
-                    const int e = pt + 128 * i;
-                    if (e < 2 * 130) {
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            uint4 w;
-                            w.x = take_part(d[i][0].x, d[i][0].y);
-                            w.y = take_part(d[i][0].z, d[i][0].w);
-                            w.z = take_part(d[i][1].x, d[i][1].y);
-                            w.w = take_part(d[i][1].z, d[i][1].w);
-                            *reinterpret_cast<uint4*>(dst + k * kPart + ((e & 1) * kP + (e >> 1)) * 16) = w;
-                        }
-                    }
-                }
-                ptx::fence_proxy_async_smem();
-                if (!p.fault_stall) ptx::mbar_arrive(&row_full[s]);
-                ++q;
-            };
-            load(0, v[0]);
-            load(1, v[1]);
-            for (int u = 0; u < nst; u += 2) {
-                put(u, v[0]);
-                load(u + 2, v[0]);
-                put(u + 1, v[1]);
-                load(u + 3, v[1]);
-            }
-        }
+        produce(std::integral_constant<int, 2>{}, tid - 384);
     }
 
     ptx::tc_fence_before();
