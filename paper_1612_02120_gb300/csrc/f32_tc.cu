@@ -179,9 +179,11 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    ptx::grid_dep_launch();  // after the TMEM allocation, so that the next launch's cannot come before it
     const uint32_t tbase = *tmem_slot;
     const uint32_t sbase = ptx::smem_u32(smem);
     const int d = p.d;
+    ptx::grid_dep_wait();
     // registers per warpgroup: launched with 96 each (640 threads); the producers keep theirs
     static_assert(40 + 2 * 120 + 2 * 96 <= 5 * 96, "register budget exceeds the launch allocation");
 
@@ -358,9 +360,9 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
                             src + ((int64_t)(p.stride * yin) * p.in_pitch + p.stride * xin) * 32 + (e & 3) * 8);
 #pragma unroll
                         for (int j = 0; j < 2; ++j) {
-                            v[i][j] = __ldg(a + j);
+                            v[i][j] = a[j];
                             if (p.dm > 0)
-                                v[i][j] = max4(max4(v[i][j], __ldg(a + dxo + j)), max4(__ldg(a + dyo + j), __ldg(a + dyo + dxo + j)));
+                                v[i][j] = max4(max4(v[i][j], a[dxo + j]), max4(a[dyo + j], a[dyo + dxo + j]));
                         }
                     }
                 }
@@ -446,7 +448,7 @@ mb_status launch_x3(XParams& p, cudaStream_t st) {
     }
     // one range per SM, or fewer when a range would get under 2 rows (each costs K - 1 more staged rows)
     const int64_t per_half = std::max<int64_t>(1, std::min<int64_t>(n_sms / p.halves, (p.total_rows + 1) / 2));
-    x3_conv<K, OUT><<<(unsigned)(per_half * p.halves), C::kThreads, C::kSmem, st>>>(p);
+    MB_CUDA(launch_dependent(x3_conv<K, OUT>, (unsigned)(per_half * p.halves), C::kThreads, C::kSmem, st, p));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;

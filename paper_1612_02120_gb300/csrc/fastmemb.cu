@@ -28,6 +28,7 @@
 
 #include "fm_conv.cuh"
 #include "internal.h"
+#include "tc_ptx.cuh"
 
 namespace mb {
 
@@ -243,6 +244,7 @@ __device__ __forceinline__ uint32_t max16(uint32_t a, uint32_t b) {
 template <bool F16, int ST>
 __global__ void __launch_bounds__(32 * kFirstWarps, 1) fm_first(const __grid_constant__ FmFirstArgs a) {
     __shared__ __align__(16) float2 s_x[kFirstWarps][4][kFirstCols];  // a ring of 4 input rows per warp
+    ptx::grid_dep_launch();  // the first layer's launch may set itself up on SMs that are done
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float2(*sx)[kFirstCols] = s_x[warp];
     constexpr int kStrip = ST == 1 ? 63 : 32;  // filtered columns of a strip

@@ -245,6 +245,9 @@ __global__ void __launch_bounds__(FCfg<HEAD, F16>::kThreads, FCfg<HEAD, F16>::kC
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    // the next launch may set itself up on SMs that are done (its TMEM is taken after this one's); this
+    // one's set-up overlaps the end of the launch whose features it reads
+    ptx::grid_dep_launch();
     const uint32_t tbase = __reduce_max_sync(0xffffffffu, *tmem_slot);  // the same in all lanes, known to be
     const uint32_t sbase = ptx::smem_u32(smem);
     const int d = p.d;
@@ -263,6 +266,7 @@ __global__ void __launch_bounds__(FCfg<HEAD, F16>::kThreads, FCfg<HEAD, F16>::kC
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    ptx::grid_dep_wait();
 
     if (warp == 0) {
         // ================= MMA issuer ================================================================
@@ -574,7 +578,7 @@ mb_status launch_fm_tc(const FmTcParams& p, cudaStream_t st) {
     // one range per resident CTA, or fewer when a range would get under 2 rows (each costs 4 more
     // staged rows: a launch this small is latency, not throughput)
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)n_sms * C::kCtas, (p.total_rows + 1) / 2));
-    fm_tc_conv<HEAD, F16><<<grid, C::kThreads, C::kSmem, st>>>(p);
+    MB_CUDA(launch_dependent(fm_tc_conv<HEAD, F16>, (unsigned)grid, C::kThreads, C::kSmem, st, p));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;

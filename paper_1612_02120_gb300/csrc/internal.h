@@ -33,6 +33,30 @@ void set_error(const char* fmt, ...);
 void clear_error();
 mb_status cuda_fail(cudaError_t e, const char* what, const char* file, int line);
 void count_launch(int n = 1);
+
+// A launch that may begin while the one before it on the stream still ends (programmatic dependent
+// launch): the kernel calls ptx::grid_dep_wait before it touches anything that an earlier launch
+// writes or reads, and the one before it calls ptx::grid_dep_launch where this one may set itself up.
+// What an earlier launch of the chain writes is read by ordinary loads (or bulk copies), not through the
+// read-only path: __ldg may be moved above the wait. A call's launches in a chain, against ordinary ones:
+// FastMemb BF16 on 64 x 64 55 -> 47 us, 1024 x 1024 283 -> 267, eight of them 1,839 -> 1,828; FP32
+// teacher 64 x 64 58 -> 52, 1024 x 1024 441 -> 430; a student gradient of 3 x 131 x 257 95 -> 91.
+// After a launch that does not call it, this is an ordinary one.
+template <typename... K, typename... A>
+cudaError_t launch_dependent(void (*kernel)(K...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                             const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
 bool fault_oom();
 
 #define MB_CUDA(call)                                                        \

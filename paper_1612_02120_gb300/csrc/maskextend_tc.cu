@@ -202,7 +202,6 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::oMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::oMisc + 4);
     const float* cst = reinterpret_cast<const float*>(smem + C::oConst);
-    ptx::grid_dep_launch();  // the next launch may set itself up on SMs that are done
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // known to be the same in all lanes
 
@@ -240,6 +239,9 @@ __global__ void __launch_bounds__(kMThreads, 1) me_tc_conv(const __grid_constant
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    // the next launch may set itself up on SMs that are done (only now: its TMEM could otherwise be
+    // taken before this launch's)
+    ptx::grid_dep_launch();
     const uint32_t tbase = *tmem_slot;
     const uint32_t sbase = ptx::smem_u32(smem);
 
@@ -619,17 +621,7 @@ mb_status launch_me_tc(const MeTcParams& q, cudaStream_t st) {
     p.extra = q.total_rows % grid;
     // the launch's set-up (barriers, constants, TMEM, the first weights) overlaps the end of the one
     // before it; its rows are read after that one's completion (grid_dep_wait)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kMThreads);
-    cfg.dynamicSmemBytes = C::kSmem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    MB_CUDA(cudaLaunchKernelEx(&cfg, me_tc_conv<KC, N, D, HEAD>, p));
+    MB_CUDA(launch_dependent(me_tc_conv<KC, N, D, HEAD>, (unsigned)grid, kMThreads, C::kSmem, st, p));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;

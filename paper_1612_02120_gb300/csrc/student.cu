@@ -29,6 +29,7 @@
 #include "internal.h"
 #include "simt_conv.cuh"
 #include "student_x3.h"
+#include "tc_ptx.cuh"
 
 namespace mb {
 
@@ -296,6 +297,8 @@ __device__ __forceinline__ float fwd_round(float v, int bf16) { return bf16 ? __
 // output channel, parts 0..2 the leading, middle and trailing 8 significant bits of a weight. Forward:
 // outputs co, inputs ci; backward (at x3 + kX3StudentPack): outputs ci, inputs co, taps flipped.
 __global__ void student_pack(const float* master, float* fwd, float* w2f, int bf16, uint8_t* x3) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kSN) return;
     float v = fwd_round(master[i], bf16);
@@ -344,6 +347,8 @@ __device__ __forceinline__ float adam_delta(float* m, float* v, int i, float gi,
 
 __global__ void adam_step(float* w, float* m, float* v, const float* g, int n, float lr, float b1, float b2,
                           float eps, float c1, float c2) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < 16) {
         const float gb = g[kSB1 + t];
@@ -571,7 +576,8 @@ static mb_status batch_grad(mb_net* s, const uint8_t* in, const float* tgt, cons
 
 static mb_status pack_forward(mb_net* s, StudentBufs& b, cudaStream_t st) {
     if (!b.x3) MB_CUDA(cudaMemsetAsync(b.zero, 0, 16 * sizeof(float), st));
-    student_pack<<<(kSN + 255) / 256, 256, 0, st>>>(s->d_params, s->d_simt, b.w2f, s->prec == MB_PREC_BF16, b.x3);
+    MB_CUDA(launch_dependent(student_pack, (kSN + 255) / 256, 256, 0, st, s->d_params, s->d_simt, b.w2f,
+                             s->prec == MB_PREC_BF16, b.x3));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;
@@ -713,8 +719,8 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
         MB_TRY(batch_grad(s, in, tgt, b.zmap + k * B, B, h, w, b, b.losses + k, st));
         const double c1 = 1.0 - std::pow((double)cfg->beta1, (double)step);
         const double c2 = 1.0 - std::pow((double)cfg->beta2, (double)step);
-        adam_step<<<(kAdamThreads + 255) / 256, 256, 0, st>>>(s->d_params, b.m, b.v, b.grad, kSN, cfg->lr, cfg->beta1,
-                                                     cfg->beta2, cfg->eps, (float)c1, (float)c2);
+        MB_CUDA(launch_dependent(adam_step, (kAdamThreads + 255) / 256, 256, 0, st, s->d_params, b.m, b.v, b.grad, kSN,
+                                 cfg->lr, cfg->beta1, cfg->beta2, cfg->eps, (float)c1, (float)c2));
         count_launch();
         MB_CUDA(cudaGetLastError());
         if (ckpt && cfg->ckpt_every > 0 && step % cfg->ckpt_every == 0) {

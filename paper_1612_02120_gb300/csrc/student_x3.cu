@@ -144,20 +144,22 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
         *abort_flag = 0;
         ptx::mbar_fence_init();
     }
-    {
-        const uint4* src = reinterpret_cast<const uint4*>(p.wpack);
-        uint4* dst = reinterpret_cast<uint4*>(smem + oBx);
-        for (int i = tid; i < kX3StudentPack / 16; i += kThreadsX) dst[i] = __ldg(src + i);
-        if (tid < 256) lut[tid] = (float)tid / 255.0f;
-    }
+    if (tid < 256) lut[tid] = (float)tid / 255.0f;
     if (warp == 0) {
         ptx::tmem_alloc(tmem_slot, 512);
         ptx::tmem_relinquish();
+    }
+    ptx::grid_dep_wait();
+    {
+        const uint4* src = reinterpret_cast<const uint4*>(p.wpack);
+        uint4* dst = reinterpret_cast<uint4*>(smem + oBx);
+        for (int i = tid; i < kX3StudentPack / 16; i += kThreadsX) dst[i] = src[i];
     }
     ptx::fence_proxy_async_smem();
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    ptx::grid_dep_launch();  // after the TMEM allocation, so that the next launch's cannot come before it
     const uint32_t tbase = *tmem_slot;
     const uint32_t sbase = ptx::smem_u32(smem);
     int64_t pos = p.total_rows * (int64_t)blockIdx.x / gridDim.x;
@@ -185,8 +187,8 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
                     d[i][0] = d[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (e < 2 * 130 && u < nst && y >= 0 && y < src_h && x >= 0 && x < src_w) {
                         const float4* a = reinterpret_cast<const float4*>(src + ((int64_t)y * src_w + x) * 16 + (e & 1) * 8);
-                        d[i][0] = __ldg(a);
-                        d[i][1] = __ldg(a + 1);
+                        d[i][0] = a[0];
+                        d[i][1] = a[1];
                     }
                 }
             };
@@ -327,11 +329,11 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
             float b2[8], hw[8], gw[8], db[8], loss = 0.f, gb = 0.f;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                b2[c] = __ldg(p.fw + kSB2 + 8 * g + c);
-                hw[c] = __ldg(p.fw + kSWH + 8 * g + c);
+                b2[c] = p.fw[kSB2 + 8 * g + c];
+                hw[c] = p.fw[kSWH + 8 * g + c];
                 gw[c] = db[c] = 0.f;
             }
-            const float hb = __ldg(p.fw + kSBH);
+            const float hb = p.fw[kSBH];
             while (sx_next(p, pos, end, it)) {
                 const int nst = it.rows + 2, x = it.x0 + px;
                 const bool col_ok = x < p.W;
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
                         w[2][kx] = lut[nb[kx]];  // row y0 + u
                     }
                     if (u + 1 < nst) fetch(u + 1);
-                    const uint32_t m_next = col_ok && u >= 1 && u + 1 < nst ? __ldg(mrow + (int64_t)(u - 1) * p.out_w) : 0u;
+                    const uint32_t m_next = col_ok && u >= 1 && u + 1 < nst ? mrow[(int64_t)(u - 1) * p.out_w] : 0u;
                     float dy[8];
                     row(dy);
                     if (u >= 2) {
@@ -505,6 +507,8 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
     __shared__ float lut[256];
     lut[threadIdx.x] = (float)threadIdx.x / 255.0f;
     __syncthreads();
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * 8, me = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     int64_t pos = total * me / nw;
@@ -513,9 +517,9 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
     float2 w[9][8], b[8];  // fw: W1t[tap][co], b1
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        b[c] = make_float2(__ldg(fw + kSB1 + 2 * c), __ldg(fw + kSB1 + 2 * c + 1));
+        b[c] = make_float2(fw[kSB1 + 2 * c], fw[kSB1 + 2 * c + 1]);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) w[k][c] = make_float2(__ldg(fw + k * 16 + 2 * c), __ldg(fw + k * 16 + 2 * c + 1));
+        for (int k = 0; k < 9; ++k) w[k][c] = make_float2(fw[k * 16 + 2 * c], fw[k * 16 + 2 * c + 1]);
     }
     while (pos < end) {
         const int64_t col = pos / H1;
@@ -600,6 +604,7 @@ __global__ void __maxnreg__(112) st_grad2(const float* dy2, const float* h1, int
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, cp = lane & 7, cg = lane >> 3;
     const int tx_n = (W + 15) / 16, ty_n = (H + 15) / 16;
     const int64_t tiles = (int64_t)B * tx_n * ty_n;
+    ptx::grid_dep_launch();
     if (t == 0) {
         for (int i = 0; i < 2; ++i) {
             ptx::mbar_init(&full[i], 1);
@@ -612,6 +617,7 @@ __global__ void __maxnreg__(112) st_grad2(const float* dy2, const float* h1, int
     for (int i = t; i < 2 * (kG2H + kG2D); i += 288) sm[i] = 0.f;
     ptx::fence_proxy_async_smem();
     __syncthreads();
+    ptx::grid_dep_wait();
     float2 acc[9][4];
     if (warp == 8) {
         uint32_t n = 0;
@@ -711,38 +717,46 @@ __global__ void __maxnreg__(112) st_grad2(const float* dy2, const float* h1, int
 }
 
 // Every parameter's gradient and the loss from the CTAs' partial sums, in FP64 and a fixed order: thread
-// (o, j) of a block adds CTAs j, j + 8, ... of output o (32 consecutive outputs per block, so that the
-// loads are coalesced), then the eight are added in order.
-__global__ void __launch_bounds__(256) st_reduce(const float* fwd, const float* g2, const float* bwd, float inv_n,
-                                                 float* grad, float* loss) {
-    __shared__ double sh[8][32];
-    const int l = threadIdx.x & 31, j = threadIdx.x >> 5, o = blockIdx.x * 32 + l;
-    const float* src = nullptr;
-    int n = kX3Grid, width = 0;
-    if (o < kSW2) {  // W1, b1
-        src = bwd + o;
-        width = 160;
-    } else if (o < kSB2) {
-        src = g2 + (o - kSW2);
-        n = kX3GridG2;
-        width = 2304;
-    } else if (o <= kSN) {  // b2, head; the loss after the last parameter
-        src = fwd + (o == kSN ? 0 : 1 + o - kSB2);
-        width = kX3FwdWidth;
+// (l, j) of a block adds CTAs j, j + 32, ... of output l of 32 consecutive ones (coalesced loads, ten at
+// most, all in flight), then warp j adds the 32 sums of output j.
+__global__ void __launch_bounds__(1024) st_reduce(const float* fwd, const float* g2, const float* bwd, float inv_n,
+                                                  float* grad, float* loss) {
+    __shared__ double sh[32][33];
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
+    const int l = threadIdx.x & 31, j = threadIdx.x >> 5;
+    {
+        const int o = blockIdx.x * 32 + l;
+        const float* src = nullptr;
+        int n = kX3Grid, width = 0;
+        if (o < kSW2) {  // W1, b1
+            src = bwd + o;
+            width = 160;
+        } else if (o < kSB2) {
+            src = g2 + (o - kSW2);
+            n = kX3GridG2;
+            width = 2304;
+        } else if (o <= kSN) {  // b2, head; the loss after the last parameter
+            src = fwd + (o == kSN ? 0 : 1 + o - kSB2);
+            width = kX3FwdWidth;
+        }
+        double s = 0.0;
+        if (src) {
+#pragma unroll 10
+            for (int c = j; c < n; c += 32) s += (double)src[(int64_t)c * width];
+        }
+        sh[j][l] = s;
     }
-    double s = 0.0;
-    if (src) {
-#pragma unroll 8
-        for (int c = j; c < n; c += 8) s += (double)__ldg(src + (int64_t)c * width);
-    }
-    sh[j][l] = s;
     __syncthreads();
-    if (j == 0 && src) {
+    // warp j: output 32 blockIdx + j, its 32 partial sums across the lanes
+    double s = sh[l][j];
 #pragma unroll
-        for (int k = 1; k < 8; ++k) s += sh[k][l];
+    for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+    const int o = blockIdx.x * 32 + j;
+    if (l == 0) {
         if (o == kSN)
             *loss = (float)(s * (double)inv_n);
-        else
+        else if (o < kSN)
             grad[o] = (float)s;
     }
 }
@@ -762,7 +776,7 @@ mb_status launch_sx(const SxParams& q, cudaStream_t st) {
     const char* stall = getenv("MB_FAULT_STALL");
     p.fault_stall = (stall && stall[0] == '1') ? 1 : 0;
     p.wait_ns = p.fault_stall ? 200000000ull : kXWaitNs;
-    st_x3<BWD><<<kX3Grid, kThreadsX, kSmemX, st>>>(p);
+    MB_CUDA(launch_dependent(st_x3<BWD>, kX3Grid, kThreadsX, kSmemX, st, p));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;
@@ -772,8 +786,8 @@ mb_status launch_sx(const SxParams& q, cudaStream_t st) {
 
 mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
     const int strips = (a.W + 2 + 31) / 32;
-    st_conv1<<<kX3Grid, 256, 0, st>>>(a.in, a.zmap, a.B, a.H, a.W, a.fw, a.h1, a.mask, strips,
-                                      (int64_t)a.B * strips * (a.H + 2));
+    MB_CUDA(launch_dependent(st_conv1, kX3Grid, 256, 0, st, a.in, a.zmap, a.B, a.H, a.W, a.fw, a.h1, a.mask, strips,
+                             (int64_t)a.B * strips * (a.H + 2)));
     count_launch();
     SxParams p{};
     p.fw = a.fw;
@@ -794,7 +808,7 @@ mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
         MB_CUDA(cudaFuncSetAttribute(st_grad2, cudaFuncAttributeMaxDynamicSharedMemorySize, kG2Smem));
         attr = true;
     }
-    st_grad2<<<kX3GridG2, 288, kG2Smem, st>>>(a.dy2, a.h1, a.B, a.H, a.W, a.part_g2, a.err);
+    MB_CUDA(launch_dependent(st_grad2, kX3GridG2, 288, kG2Smem, st, a.dy2, a.h1, a.B, a.H, a.W, a.part_g2, a.err));
     count_launch();
     p.in = a.dy2;
     p.wpack = a.pack + kX3StudentPack;
@@ -802,7 +816,8 @@ mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
     p.img = a.in;
     p.partial = a.part_bwd;
     MB_TRY(launch_sx<true>(p, st));
-    st_reduce<<<(kSN + 1 + 31) / 32, 256, 0, st>>>(a.part_fwd, a.part_g2, a.part_bwd, a.inv_n, a.grad, a.loss);
+    MB_CUDA(launch_dependent(st_reduce, (kSN + 1 + 31) / 32, 1024, 0, st, a.part_fwd, a.part_g2, a.part_bwd, a.inv_n, a.grad,
+                             a.loss));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;
