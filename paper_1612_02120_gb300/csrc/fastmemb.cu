@@ -185,14 +185,16 @@ mb_status simt_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_
 // pairs, rounding to the net's 16-bit type, the 2x2 max-filter, and (ST = 2) its stride: features in
 // the layout that the next conv's bulk copies read, [slice][row][chunk of 8][column][16 B].
 //
-// FP32 FMA issue bounds it (2,048 FLOP per conv pixel). A warp walks down a 64-column strip on its
-// own; a lane holds all 64 conv channels of columns l and l + 32, packed by channel pairs, so a
-// max-out group is one accumulator pair and a pixel's 16-byte chunks are stored whole. The weights
-// are kernel parameters: constant-bank operands, no shared-memory broadcasts beside the FMAs (those
-// took 62 % of the shared-memory pipe and left the FMA pipe at 50 %: 528 us). The inputs sit in shared
-// memory duplicated, ready for packed FMAs. Tap order and rounding are those of fm_conv, so the
-// features are bitwise the same. 354 us on 1024 x 1024 x 8 (50 TFLOP/s, 0.63 of the FP32 FMA rate);
-// unpacked FMAs with the filter left to the next layer's loads took 534 us.
+// FP32 FMA issue bounds it (2,048 FLOP per conv pixel). A warp walks down a 32-column strip on its
+// own; a lane holds all 64 conv channels of its column, packed by channel pairs, so a max-out group
+// is one accumulator pair and a pixel's 16-byte chunks are stored whole. The weights are kernel
+// parameters, no shared-memory broadcasts beside the FMAs (those took 62 % of the shared-memory pipe
+// and left the FMA pipe at 50 %: 528 us). The inputs sit in shared memory duplicated, ready for packed
+// FMAs. Tap order and rounding are those of fm_conv, so the features are bitwise the same. 339 us on
+// 1024 x 1024 x 8 (FMA pipe 77 % busy, 16 warps of 118 registers); two columns a lane and 8 warps of 248
+// took 354 (the max-out, the filter and the stores of 2 warps a scheduler hide less behind FMAs), two
+// columns and half the channels a lane 869 (weights at a run-time offset); unpacked FMAs with the
+// filter left to the next layer's loads took 534.
 struct FmFirstArgs {
     const uint8_t* in;
     int64_t in_slice, in_pitch;
@@ -207,8 +209,9 @@ struct FmFirstArgs {
     float2 b[32];
 };
 
-constexpr int kFirstWarps = 8;
-constexpr int kFirstCols = 68;                // 64 + 3 inputs per row
+constexpr int kFirstPx = 1;                   // columns of a lane
+constexpr int kFirstWarps = 16 / kFirstPx;
+constexpr int kFirstCols = 32 * kFirstPx + 4; // 3 more inputs per row
 
 __device__ __forceinline__ int refl_clamp(int t, int n) {
     t = t < 0 ? -t : t;
@@ -247,7 +250,7 @@ __global__ void __launch_bounds__(32 * kFirstWarps, 1) fm_first(const __grid_con
     ptx::grid_dep_launch();  // the first layer's launch may set itself up on SMs that are done
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float2(*sx)[kFirstCols] = s_x[warp];
-    constexpr int kStrip = ST == 1 ? 63 : 32;  // filtered columns of a strip
+    constexpr int kStrip = ST == 1 ? 32 * kFirstPx - 1 : 16 * kFirstPx;  // filtered columns of a strip
     // one equal contiguous range of strip-rows per warp
     const int64_t n_warps = (int64_t)gridDim.x * kFirstWarps, me = (int64_t)blockIdx.x * kFirstWarps + warp;
     int64_t pos = a.total * me / n_warps;
@@ -260,25 +263,28 @@ __global__ void __launch_bounds__(32 * kFirstWarps, 1) fm_first(const __grid_con
         pos += rows;
         const int n_in = (ST == 1 ? rows + 1 : 2 * rows) + 3;  // conv rows + 3
         const uint8_t* src = a.in + (int64_t)zi * a.in_slice;
-        int sc[3];
+        constexpr int kIn = kFirstPx + 1;
+        int sc[kIn];
 #pragma unroll
-        for (int i = 0; i < 3; ++i) sc[i] = refl_clamp(ST * x0 + lane + 32 * i + a.off_x, a.src_w);
-        uint8_t u[3];
+        for (int i = 0; i < kIn; ++i) sc[i] = refl_clamp(ST * x0 + lane + 32 * i + a.off_x, a.src_w);
+        uint8_t u[kIn];
         auto fetch = [&](int r) {  // the bytes of input row r of the item
             const uint8_t* row = src + (int64_t)refl_clamp(ST * y0 + r + a.off_y, a.src_h) * a.in_pitch;
 #pragma unroll
-            for (int i = 0; i < 3; ++i) u[i] = __ldg(row + sc[i]);
+            for (int i = 0; i < kIn; ++i) u[i] = __ldg(row + sc[i]);
         };
         uint16_t* out = a.out + (int64_t)zi * a.out_slice;
-        uint32_t prev[2][16];
+        uint32_t prev[kFirstPx][16];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) prev[0][k] = prev[1][k] = 0u;
+        for (int i = 0; i < kFirstPx; ++i)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) prev[i][k] = 0u;
         fetch(0);
 #pragma unroll 1
         for (int r = 0; r < n_in; ++r) {
             __syncwarp();  // row r - 4, whose slot is written now, has been read
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+            for (int i = 0; i < kIn; ++i)
                 if (lane + 32 * i < kFirstCols) {
                     const float v = (float)u[i] / 255.0f;
                     sx[r & 3][lane + 32 * i] = make_float2(v, v);
@@ -287,27 +293,31 @@ __global__ void __launch_bounds__(32 * kFirstWarps, 1) fm_first(const __grid_con
             __syncwarp();
             const int yc = r - 3;  // conv row of the item that input row r completes
             if (yc < 0) continue;
-            float2 acc[2][32];
+            float2 acc[kFirstPx][32];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) acc[0][c] = acc[1][c] = a.b[c];
+            for (int c = 0; c < 32; ++c)
+#pragma unroll
+                for (int i = 0; i < kFirstPx; ++i) acc[i][c] = a.b[c];
 #pragma unroll
             for (int ky = 0; ky < 4; ++ky) {
                 const float2* row = sx[(r + 1 + ky) & 3] + lane;  // input row yc + ky
 #pragma unroll
                 for (int kx = 0; kx < 4; ++kx) {
-                    const float2 xa = row[kx], xb = row[kx + 32];
+                    float2 x[kFirstPx];
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        acc[0][c] = __ffma2_rn(a.w[4 * ky + kx][c], xa, acc[0][c]);
-                        acc[1][c] = __ffma2_rn(a.w[4 * ky + kx][c], xb, acc[1][c]);
-                    }
+                    for (int i = 0; i < kFirstPx; ++i) x[i] = row[kx + 32 * i];
+#pragma unroll
+                    for (int c = 0; c < 32; ++c)
+#pragma unroll
+                        for (int i = 0; i < kFirstPx; ++i)
+                            acc[i][c] = __ffma2_rn(a.w[4 * ky + kx][c], x[i], acc[i][c]);
                 }
             }
             const bool emit = ST == 1 ? yc > 0 : (yc & 1) != 0;
             const int y = ST == 1 ? y0 + yc - 1 : y0 + (yc >> 1);
-            uint32_t v[2][16];
+            uint32_t v[kFirstPx][16];
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < kFirstPx; ++i)
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {
                     const uint32_t f = pack16<F16>(fmaxf(acc[i][2 * k].x, acc[i][2 * k].y),
@@ -316,20 +326,20 @@ __global__ void __launch_bounds__(32 * kFirstWarps, 1) fm_first(const __grid_con
                     prev[i][k] = f;
                 }
             if (!emit) continue;
-            // horizontal partner: the next column, in the next lane; of column 31 it is lane 0's
-            // column 32, and column 63 has none (a strip yields 63)
+            // horizontal partner: the next column, in the next lane; of a column group's last it is the next
+            // group's first, and the strip's last column has none
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const uint32_t n0 = __shfl_sync(0xffffffffu, lane == 0 ? v[1][k] : v[0][k], (lane + 1) & 31);
-                const uint32_t n1 = __shfl_sync(0xffffffffu, v[1][k], (lane + 1) & 31);
-                v[0][k] = max16<F16>(v[0][k], n0);
-                v[1][k] = max16<F16>(v[1][k], n1);
-            }
+            for (int k = 0; k < 16; ++k)
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
+                for (int i = 0; i < kFirstPx; ++i) {
+                    const uint32_t mine = i + 1 < kFirstPx && lane == 0 ? v[(i + 1) % kFirstPx][k] : v[i][k];
+                    v[i][k] = max16<F16>(v[i][k], __shfl_sync(0xffffffffu, mine, (lane + 1) & 31));
+                }
+#pragma unroll
+            for (int i = 0; i < kFirstPx; ++i) {
                 const int c = lane + 32 * i;  // conv column of the strip
                 const int x = x0 + (ST == 1 ? c : c >> 1);
-                if ((ST == 1 ? c < 63 : (c & 1) == 0) && x < a.cols) {
+                if ((ST == 1 ? c < kStrip : (c & 1) == 0) && x < a.cols) {
                     uint16_t* o = out + ((int64_t)y * 4 * a.out_pitch + x) * 8;
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
@@ -349,7 +359,7 @@ static mb_status launch_first(FmFirstArgs a, int nz, cudaStream_t st) {
         MB_CUDA(cudaGetDevice(&dev));
         MB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    constexpr int kStrip = ST == 1 ? 63 : 32;
+    constexpr int kStrip = ST == 1 ? 32 * kFirstPx - 1 : 16 * kFirstPx;
     a.n_strips = (a.cols + kStrip - 1) / kStrip;
     a.total = (int64_t)nz * a.n_strips * a.rows;
     // one CTA per SM, or fewer where a warp would get no row (a row costs 2 conv rows at the start of
