@@ -80,13 +80,16 @@ typedef enum {
  * Supported networks: the teacher (conv5x5 1->32 ReLU, maxfilter 2, conv5x5 32->32 ReLU,
  * maxfilter 2, conv5x5 32->32 ReLU, head 32->1) in FP32, BF16 and FP8; the student (conv3x3
  * 1->16 ReLU, conv3x3 16->16 ReLU, head 16->1) in FP32 and BF16 (BF16 weights; its inference runs
- * on the tensor cores with BF16 layer-1 features and FP32 accumulation, its training forward in
- * FP32 arithmetic); and FastMemb in dense form
+ * on the tensor cores with BF16 layer-1 features and FP32 accumulation, its training with FP32
+ * accuracy: FMAs, and tensor cores on values split exactly into three BF16 parts); and FastMemb in
+ * dense form
  * (Sec. 2.2: conv4x4 1->32 G=2 d=1, maxfilter d=1, conv4x4 32->32 G=2 d=2, maxfilter d=2,
  * conv4x4 32->32 G=2 d=4, maxfilter d=4, softmax head conv4x4 32->2 d=8; no ReLU; radius 26,
  * so its slices need h, w >= 27) and FastMemb_3nm (Sec. 2.2, "A subsampling CNN for 3 nm data":
  * one more stage, conv4x4 32->32 G=2 d=8 and maxfilter d=8, then the head at d=16; radius 54,
- * slices h, w >= 55), both in FP32, BF16 and FP16 (the 16-bit nets: layer 1 on CUDA cores in
+ * slices h, w >= 55), both in FP32 (like the FP32 teacher: the 32-channel convolutions on the tensor
+ * cores in three exact BF16 parts per value, error below an FP32 FMA chain's, where weights and
+ * activations are bounded by 2^100, else on CUDA cores), BF16 and FP16 (the 16-bit nets: layer 1 on CUDA cores in
  * FP32 stored as 16-bit, the later convs and the head on the tensor cores with FP32 accumulation;
  * BF16 weights are split into two BF16 parts, FP16 weights are one FP16 value except the head's;
  * FP16 activations are finite below 65504); and MaskExtend (Sec. 3.2: conv4x4 12->32 G=2 d=1,

@@ -21,7 +21,7 @@
 // costs tens of cycles of MMA issue.
 //
 // Features in global memory are what the next conv reads, already max-filtered, chunk-planar:
-// [row][8-channel chunk][column][16 B], so a staged row is a few contiguous runs that one thread fetches
+// [row][8-channel chunk][column][16 B], so a staged row is a few contiguous runs that one warp fetches
 // with bulk copies. (Eight producer warps gathering 4 x 16 B per pixel took ~9,000 cycles for a row of
 // the last layer, a quarter of its launch before the first group was staged, and while they ran an MMA
 // took 85-100 cycles of the issuing thread against 65 alone.) The epilogue owns the values the filter
@@ -30,11 +30,16 @@
 // item one conv row more than filtered rows. The maxima are of values already rounded to FP16, so the
 // maps are bitwise those of filtering on the load.
 //
+// 16 sections of 512 x 512, us: 4,766 with gathering producers; 4,595 with whole-warp issue loops; 4,222 with
+// rows by bulk copies; 3,138 with two issuing warps, the loader's lanes, ranges without divisions and dependent
+// launches (23, 33, 45, 47, 46 a section for the five layers). The multiplies alone are 1,390 at the BF16 rate:
+// N = 96 .. 128 MMAs read shared memory at its full 128 B per cycle, beside the streamed weights.
+//
 // Warp roles (384 threads, 1 CTA per SM, persistent over work items):
 //   warps 0, 3   lane 0 issues the MMAs of the even / odd rows of a group (warp 0 also owns TMEM)
 //   warp 1       lane 0 streams the weight units into their ring with bulk copies (completion counted
 //                on the unit's mbarrier)
-//   warp 2       lane 0 fetches the staged rows (as many ahead as shared memory allows, up to 12)
+//   warp 2       lane c fetches chunk c of the staged rows (as many ahead as shared memory allows, up to 12)
 //   warps 4-11   epilogue, two groups of 4 warps, each half of the feature chunks: TMEM -> registers,
 //                + bias, max-out, FP16, max-filter, store. Last layer: the first group alone, the 1x1
 //                conv to 3 classes and the softmax, FP32 probabilities

@@ -4,7 +4,9 @@
 // Operation (Sec. 2.2): valid cross-correlation + bias + ReLU; the 2x2 stride-1 max-filter that
 // replaces max-pooling for dense computation is applied while the next layer stages its input;
 // the 1x1 head + sigmoid is fused into the last convolution. The first layer reads the uint8
-// slice directly, mirror-padding it (reflect-101) and scaling by 1/255.
+// slice directly, mirror-padding it (reflect-101) and scaling by 1/255. Where the weights are bounded,
+// the teacher's layers 2 and 3 run on the tensor cores instead (f32_tc.cu, no less accurate); the FP8
+// calibration always takes these kernels, so that its scales stay what they were.
 //
 // Domains for an output region of rows x cols (teacher, radius 7):
 //   layer-1 output (rows+10) x (cols+10) x 32, layer-2 output (rows+5) x (cols+5) x 32,

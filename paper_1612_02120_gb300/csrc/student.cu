@@ -14,7 +14,8 @@
 // uninterrupted one.
 // Adam (Kingma and Ba, 2014): FP32 master weights, first/second moments, bias correction, with
 // layer 1 optimised in centred-input coordinates (see adam_step); the forward copy is rounded to
-// BF16 for BF16 students.
+// BF16 for BF16 students. The convolution passes run in student_x3.cu where the weights allow its
+// split (train_bounded); the CUDA-core passes of this file are for the others.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <errno.h>
