@@ -268,8 +268,8 @@ mb_status student_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, i
     if (net->prec == MB_PREC_BF16)
         return st_tc_region(net, in, z, h, w, in_pitch, in_slice, y0, x0, rows, cols, out, out_pitch, out_slice, ot,
                             st);
-    return simt_student_region(net, in, z, h, w, in_pitch, in_slice, y0, x0, rows, cols, out, out_pitch, out_slice,
-                               ot, st);
+    return student_f32_region(net, in, z, h, w, in_pitch, in_slice, y0, x0, rows, cols, out, out_pitch, out_slice,
+                              ot, st);
 }
 
 static mb_status fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,

@@ -133,6 +133,13 @@ mb_status simt_teacher_region(mb_net* net, const uint8_t* in, int64_t z, int64_t
                               int64_t in_pitch, int64_t in_slice, int64_t y0, int64_t x0, int64_t rows,
                               int64_t cols, void* out, int64_t out_pitch, int64_t out_slice,
                               mb_out_type ot, cudaStream_t st);
+// Slices per pass of a workspace of per_slice bytes each (3 GB at most, at least one slice).
+int64_t chunk_slices(size_t per_slice, int64_t z);
+// FP32 student inference: on the tensor cores in exact three-part splits where the weights are bounded
+// (student.cu, student_x3.cu), else simt_student_region.
+mb_status student_f32_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,
+                             int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
+                             int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st);
 mb_status simt_student_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w,
                               int64_t in_pitch, int64_t in_slice, int64_t y0, int64_t x0, int64_t rows,
                               int64_t cols, void* out, int64_t out_pitch, int64_t out_slice,

@@ -70,7 +70,7 @@ static size_t teacher_ws_per_slice(int64_t rows, int64_t cols) {
     return (size_t)((rows + 10) * (cols + 10) + (rows + 5) * (cols + 5)) * 32 * sizeof(float);
 }
 
-static int64_t chunk_slices(size_t per_slice, int64_t z) {
+int64_t chunk_slices(size_t per_slice, int64_t z) {
     const size_t budget = (size_t)3 << 30;
     int64_t zc = (int64_t)std::max<size_t>(1, budget / std::max<size_t>(per_slice, 1));
     zc = std::min<int64_t>(zc, 65535);

@@ -435,6 +435,44 @@ static mb_status train_error(mb_net* s) {
     return MB_OK;
 }
 
+// The split passes where no activation can pass 2^70 (train_bounded), else the CUDA-core layers; the choice
+// does not depend on the sizes, so any region's map is the crop of the whole one's.
+mb_status student_f32_region(mb_net* s, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,
+                             int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
+                             int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st) {
+    if (!train_bounded(s->host_params.data(), 0.0))
+        return simt_student_region(s, in, z, h, w, in_pitch, in_slice, y0, x0, rows, cols, out, out_pitch, out_slice, ot, st);
+    if (z == 0 || rows == 0 || cols == 0) return MB_OK;
+    MB_TRY(train_words(s));
+    MB_TRY(train_error(s));
+    const size_t per = (size_t)(rows + 2) * (size_t)(cols + 2) * 16 * sizeof(float);
+    const int64_t zc = chunk_slices(per, z);
+    MB_TRY(s->ws.ensure(per * (size_t)zc));
+    StudentX3Region a{};
+    a.in_slice = in_slice;
+    a.in_pitch = in_pitch;
+    a.out_pitch = out_pitch;
+    a.out_slice = out_slice;
+    a.h = (int)h;
+    a.w = (int)w;
+    a.y0 = (int)y0;
+    a.x0 = (int)x0;
+    a.rows = (int)rows;
+    a.cols = (int)cols;
+    a.fw = s->d_simt;
+    a.h1 = static_cast<float*>(s->ws.ptr);
+    a.out_u8 = ot == MB_OUT_U8 ? 1 : 0;
+    a.err = s->train_dev;
+    for (int64_t z0 = 0; z0 < z; z0 += zc) {
+        a.in = in + z0 * in_slice;
+        a.z = (int)std::min<int64_t>(zc, z - z0);
+        a.out = static_cast<uint8_t*>(out) + z0 * out_slice * (ot == MB_OUT_F32 ? 4 : 1);
+        a.first = z0 == 0;
+        MB_TRY(student_x3_infer(a, st));
+    }
+    return train_error(s);
+}
+
 // Carves the training workspace; every sub-buffer starts on a 256-byte boundary (the convolution
 // kernels read weights and activations as float4).
 static mb_status ensure_bufs(mb_net* s, int64_t B, int64_t H, int64_t W, int64_t steps, bool x3, StudentBufs& b) {

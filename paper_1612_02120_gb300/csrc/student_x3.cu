@@ -1,13 +1,16 @@
-// student_x3.cu - the student's training convolutions on the tensor cores with FP32 accuracy, each fused
-// with what follows it: conv2 + ReLU + head + loss + dL/dy2 (st_x3<false>) and the data gradient +
-// ReLU mask + conv1's weight gradient (st_x3<true>); the first convolution (st_conv1) and conv2's weight
-// gradient (st_grad2) on packed FP32 FMAs.
+// student_x3.cu - the FP32 student's convolutions on the tensor cores with FP32 accuracy, each fused with
+// what follows it: conv2 + ReLU + head, with loss + dL/dy2 (st_x3<SX_FWD>) or the probability
+// (st_x3<SX_INFER>), and the data gradient + ReLU mask + conv1's weight gradient (st_x3<SX_BWD>); the first
+// convolution (st_conv1) and conv2's weight gradient (st_grad2) on packed FP32 FMAs.
 //
 // Numbers: the three-part BF16 split of f32_tc.cu (six of nine products, error below an FMA chain's).
 // With 16 channels the products of equal weight sit in columns of their own: part 1 of an input row
 // is multiplied by [w1 | w2 | w3] (N = 144: 3 parts x 3 row taps x 16), part 2 by [w1 | w2] into the
 // second and third column groups, part 3 by w1 into the third; the epilogue adds g1 + (g2 + g3) per row
 // tap and sums the row taps in FP32.
+//
+// Inference, FP32 student, against the CUDA-core convolutions: 64 x 64 20.6 -> 14.6 us, 1024 x 1024 133 -> 65,
+// 4096 x 4096 1,907 -> 794.
 //
 // st_x3 reads one 64-byte pixel of h1 or dy2 per output pixel, once, and the forward writes dy2 once
 // (h2 and dy1 exist in registers only): a row of 128 pixels costs ~500 cycles of MMAs and 360-710 of
@@ -56,6 +59,9 @@ constexpr int oMiscX = oBarX + kBarsX * 8;
 constexpr int kSmemX = oMiscX + 16;
 static_assert(kSmemX <= 227 * 1024 && kBufsX * kNx <= 512, "resources");
 
+// the passes of st_x3: training forward, training backward, inference
+enum { SX_FWD = 0, SX_BWD = 1, SX_INFER = 2 };
+
 struct SxParams {
     const float* in;       // h1 [B][H+2][W+2][16], or dy2 [B][H][W][16] read as zero-padded by 2
     const uint8_t* wpack;  // student_pack's B operand of this pass: per column tap kx [2 chunks][144 rows][16 B]
@@ -66,6 +72,10 @@ struct SxParams {
     const int* zmap;
     float* dy2;
     float inv_n;
+    // inference
+    void* out;             // probabilities [B][H][W], out_pitch and out_slice elements apart
+    int64_t out_pitch, out_slice;
+    int out_u8;
     // backward
     const uint16_t* mask;  // h1 > 0 per channel, [B][H+2][W+2]
     const uint8_t* img;    // [slices][H][W]
@@ -117,8 +127,9 @@ __device__ __forceinline__ void group_sum(const float (&v)[N], float* red, int g
     }
 }
 
-template <bool BWD>
+template <int MODE>
 __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ SxParams p) {
+    constexpr bool BWD = MODE == SX_BWD, INFER = MODE == SX_INFER;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t* row_full = reinterpret_cast<uint64_t*>(smem + oBarX);
     uint64_t* row_empty = row_full + kRingX;
@@ -149,8 +160,22 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
         ptx::tmem_alloc(tmem_slot, 512);
         ptx::tmem_relinquish();
     }
+    if constexpr (INFER) {
+        // no packing launch before it: W2t[ci][tap][co], which no launch of the chain writes, split here
+        for (int i = tid; i < 2304; i += kThreadsX) {
+            const int co = i % 16, tap = (i / 16) % 9, ci = i / 144, ky = tap / 3, kx = tap % 3;
+            float v = p.fw[kSW2 + i];
+#pragma unroll
+            for (int part = 0; part < 3; ++part) {
+                const uint32_t u = __float_as_uint(v) & 0xffff0000u;
+                v -= __uint_as_float(u);
+                *reinterpret_cast<uint16_t*>(smem + oBx + ((kx * 2 + (ci >> 3)) * kNx + 48 * part + 16 * ky + co) * 16 + 2 * (ci & 7)) =
+                    (uint16_t)(u >> 16);
+            }
+        }
+    }
     ptx::grid_dep_wait();
-    {
+    if constexpr (!INFER) {
         const uint4* src = reinterpret_cast<const uint4*>(p.wpack);
         uint4* dst = reinterpret_cast<uint4*>(smem + oBx);
         for (int i = tid; i < kX3StudentPack / 16; i += kThreadsX) dst[i] = src[i];
@@ -338,12 +363,12 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
                 const int nst = it.rows + 2, x = it.x0 + px;
                 const bool col_ok = x < p.W;
                 const int64_t pix0 = ((int64_t)it.z * p.H + it.y0) * p.W + x;  // conv row 0 of the item
-                const float* trow = p.target + ((int64_t)(p.zmap ? p.zmap[it.z] : it.z) * p.H + it.y0) * p.W + x;
+                const float* trow = INFER ? nullptr : p.target + ((int64_t)(p.zmap ? p.zmap[it.z] : it.z) * p.H + it.y0) * p.W + x;
 #pragma unroll
                 for (int c = 0; c < 8; ++c) s0[c] = s1[c] = 0.f;
                 float t = 0.f;
                 for (int u = 0; u < nst; ++u, ++q) {
-                    const float t_next = col_ok && u >= 1 && u + 1 < nst ? __ldg(trow + (int64_t)(u - 1) * p.W) : 0.f;
+                    const float t_next = !INFER && col_ok && u >= 1 && u + 1 < nst ? __ldg(trow + (int64_t)(u - 1) * p.W) : 0.f;
                     float h2[8];
                     row(h2);
                     if (u >= 2) {
@@ -360,50 +385,63 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
                         xc[g * 128 + px] = z;
                         asm volatile("bar.sync 2, 256;" ::: "memory");
                         z = (xc[px] + xc[128 + px]) + hb;
-                        const float pr = 1.0f / (1.0f + expf(-z));
-                        const float e = pr - t;
-                        const float dz = col_ok ? 2.0f * p.inv_n * e * pr * (1.0f - pr) : 0.f;
-                        if (g == 0 && col_ok) {
-                            loss = fmaf(e, e, loss);
-                            gb += dz;
-                        }
-                        float dy[8];
+                        if constexpr (INFER) {
+                            if (g == (u & 1) && col_ok && !*abort_flag) {  // the groups take rows in turn
+                                const float pr = 1.0f / (1.0f + expf(-z));
+                                const int64_t i = (int64_t)it.z * p.out_slice + (int64_t)(it.y0 + u - 2) * p.out_pitch + x;
+                                if (p.out_u8)
+                                    static_cast<uint8_t*>(p.out)[i] = (uint8_t)fminf(floorf(255.0f * pr + 0.5f), 255.0f);
+                                else
+                                    static_cast<float*>(p.out)[i] = pr;
+                            }
+                        } else {
+                            const float pr = 1.0f / (1.0f + expf(-z));
+                            const float e = pr - t;
+                            const float dz = col_ok ? 2.0f * p.inv_n * e * pr * (1.0f - pr) : 0.f;
+                            if (g == 0 && col_ok) {
+                                loss = fmaf(e, e, loss);
+                                gb += dz;
+                            }
+                            float dy[8];
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            gw[c] = fmaf(dz, h2[c], gw[c]);
-                            dy[c] = h2[c] > 0.f ? dz * hw[c] : 0.f;
-                            db[c] += dy[c];
-                        }
-                        if (col_ok && !*abort_flag) {
-                            float4* o = reinterpret_cast<float4*>(p.dy2 + (pix0 + (int64_t)(u - 2) * p.W) * 16 + 8 * g);
-                            o[0] = make_float4(dy[0], dy[1], dy[2], dy[3]);
-                            o[1] = make_float4(dy[4], dy[5], dy[6], dy[7]);
+                            for (int c = 0; c < 8; ++c) {
+                                gw[c] = fmaf(dz, h2[c], gw[c]);
+                                dy[c] = h2[c] > 0.f ? dz * hw[c] : 0.f;
+                                db[c] += dy[c];
+                            }
+                            if (col_ok && !*abort_flag) {
+                                float4* o = reinterpret_cast<float4*>(p.dy2 + (pix0 + (int64_t)(u - 2) * p.W) * 16 + 8 * g);
+                                o[0] = make_float4(dy[0], dy[1], dy[2], dy[3]);
+                                o[1] = make_float4(dy[4], dy[5], dy[6], dy[7]);
+                            }
                         }
                     }
                     t = t_next;
                 }
             }
-            // partials per CTA: [loss, db2[16], dWh[16], dbh]
-            float all[18];
+            if constexpr (!INFER) {
+                // partials per CTA: [loss, db2[16], dWh[16], dbh]
+                float all[18];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                all[c] = db[c];
-                all[8 + c] = gw[c];
-            }
-            all[16] = loss;
-            all[17] = gb;
-            float* out = reinterpret_cast<float*>(smem + oXch) + 128 * g;  // free: every row's exchange is over
-            asm volatile("bar.sync 2, 256;" ::: "memory");
-            group_sum(all, red, g, warp & 3, lane, out);
-            asm volatile("bar.sync %0, 128;" ::"r"(3 + g) : "memory");
-            float* part = p.partial + (int64_t)blockIdx.x * kX3FwdWidth;
-            if (px < 8) {
-                part[1 + 8 * g + px] = out[px];
-                part[17 + 8 * g + px] = out[8 + px];
-            }
-            if (g == 0 && px == 0) {
-                part[0] = out[16];
-                part[33] = out[17];
+                for (int c = 0; c < 8; ++c) {
+                    all[c] = db[c];
+                    all[8 + c] = gw[c];
+                }
+                all[16] = loss;
+                all[17] = gb;
+                float* out = reinterpret_cast<float*>(smem + oXch) + 128 * g;  // free: every row's exchange is over
+                asm volatile("bar.sync 2, 256;" ::: "memory");
+                group_sum(all, red, g, warp & 3, lane, out);
+                asm volatile("bar.sync %0, 128;" ::"r"(3 + g) : "memory");
+                float* part = p.partial + (int64_t)blockIdx.x * kX3FwdWidth;
+                if (px < 8) {
+                    part[1 + 8 * g + px] = out[px];
+                    part[17 + 8 * g + px] = out[8 + px];
+                }
+                if (g == 0 && px == 0) {
+                    part[0] = out[16];
+                    part[33] = out[17];
+                }
             }
         } else {
             // dy1 = (h1 > 0) conv row; dW1[co][ky][kx] += dy1[co] x(y + ky, x + kx), channel pairs packed
@@ -498,12 +536,25 @@ __global__ void __launch_bounds__(kThreadsX, 1) st_x3(const __grid_constant__ Sx
     if (warp == 0) ptx::tmem_dealloc(tbase, 512);
 }
 
+struct SxConv1 {
+    const uint8_t* in;   // slice zmap[z] (z without a map) at in_slice, rows in_pitch apart, H x W
+    const int* zmap;
+    int64_t in_slice, in_pitch;
+    int H, W;
+    int y0, x0;          // slice coordinates of the outputs' first row and column, plus 1
+    int H1, W1;          // rows and columns of h1
+    const float* fw;
+    float* h1;           // [z][H1][W1][16]
+    uint16_t* mask;      // bit c of [z][H1][W1]: h1[c] > 0 (NULL: not wanted)
+    int n_strips;        // of 32 columns
+    int64_t total;       // z x n_strips x H1
+};
+
 // conv1 + ReLU from the uint8 slice: h1 [B][H+2][W+2][16] FP32 and its mask (bit c: h1[c] > 0). HBM
 // writes bound it (66 B per pixel: 85 us on a batch of 32 x 512 x 512; 154 measured, 205 with weights
 // broadcast from shared memory). A warp walks down a 32-column strip; a lane keeps all 144 weights
 // (packed by channel pairs), its 3x3 input window and the bytes of the next four rows in registers.
-__global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int* zmap, int B, int H, int W, const float* fw,
-                                                   float* h1, uint16_t* mask, int n_strips, int64_t total) {
+__global__ void __launch_bounds__(256, 1) st_conv1(const __grid_constant__ SxConv1 a) {
     __shared__ float lut[256];
     lut[threadIdx.x] = (float)threadIdx.x / 255.0f;
     __syncthreads();
@@ -511,9 +562,10 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
     ptx::grid_dep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nw = (int64_t)gridDim.x * 8, me = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    int64_t pos = total * me / nw;
-    const int64_t end = total * (me + 1) / nw;
-    const int H1 = H + 2, W1 = W + 2;
+    int64_t pos = a.total * me / nw;
+    const int64_t end = a.total * (me + 1) / nw;
+    const int H1 = a.H1, W1 = a.W1;
+    const float* fw = a.fw;
     float2 w[9][8], b[8];  // fw: W1t[tap][co], b1
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
@@ -523,17 +575,17 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
     }
     while (pos < end) {
         const int64_t col = pos / H1;
-        const int y0 = (int)(pos - col * H1), z = (int)(col / n_strips), x = (int)(col % n_strips) * 32 + lane;
+        const int y0 = (int)(pos - col * H1), z = (int)(col / a.n_strips), x = (int)(col % a.n_strips) * 32 + lane;
         const int rows = (int)min((int64_t)(H1 - y0), end - pos);
         pos += rows;
-        const uint8_t* src = in + (int64_t)(zmap ? zmap[z] : z) * H * W;
+        const uint8_t* src = a.in + (int64_t)(a.zmap ? a.zmap[z] : z) * a.in_slice;
         int sc[3];
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx) sc[kx] = sx_refl(x + kx - 2, W);
+        for (int kx = 0; kx < 3; ++kx) sc[kx] = sx_refl(x + kx - 2 + a.x0, a.W);
         float win[3][3];
         uint8_t nb[4][3];  // four rows of bytes in flight
         auto fetch = [&](int r, uint8_t (&n)[3]) {
-            const uint8_t* row = src + (int64_t)sx_refl(y0 + r - 2, H) * W;
+            const uint8_t* row = src + (int64_t)sx_refl(y0 + r - 2 + a.y0, a.H) * a.in_pitch;
 #pragma unroll
             for (int kx = 0; kx < 3; ++kx) n[kx] = __ldg(row + sc[kx]);
         };
@@ -569,10 +621,10 @@ __global__ void __launch_bounds__(256, 1) st_conv1(const uint8_t* in, const int*
                     m |= (acc[c].x > 0.f ? 1u : 0u) << (2 * c) | (acc[c].y > 0.f ? 1u : 0u) << (2 * c + 1);
                     acc[c] = make_float2(fmaxf(acc[c].x, 0.f), fmaxf(acc[c].y, 0.f));
                 }
-                float4* o = reinterpret_cast<float4*>(h1 + pix * 16);
+                float4* o = reinterpret_cast<float4*>(a.h1 + pix * 16);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) o[c] = make_float4(acc[2 * c].x, acc[2 * c].y, acc[2 * c + 1].x, acc[2 * c + 1].y);
-                mask[pix] = (uint16_t)m;
+                if (a.mask) a.mask[pix] = (uint16_t)m;
             }
         };
 #pragma unroll 1
@@ -761,13 +813,14 @@ __global__ void __launch_bounds__(1024) st_reduce(const float* fwd, const float*
     }
 }
 
-template <bool BWD>
+template <int MODE>
 mb_status launch_sx(const SxParams& q, cudaStream_t st) {
     static bool attr = false;
     if (!attr) {
-        MB_CUDA(cudaFuncSetAttribute(st_x3<BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemX));
+        MB_CUDA(cudaFuncSetAttribute(st_x3<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemX));
         attr = true;
     }
+    constexpr bool BWD = MODE == SX_BWD;
     SxParams p = q;
     p.out_h = BWD ? p.H + 2 : p.H;
     p.out_w = BWD ? p.W + 2 : p.W;
@@ -776,7 +829,9 @@ mb_status launch_sx(const SxParams& q, cudaStream_t st) {
     const char* stall = getenv("MB_FAULT_STALL");
     p.fault_stall = (stall && stall[0] == '1') ? 1 : 0;
     p.wait_ns = p.fault_stall ? 200000000ull : kXWaitNs;
-    MB_CUDA(launch_dependent(st_x3<BWD>, kX3Grid, kThreadsX, kSmemX, st, p));
+    // inference: one range per SM, or fewer when a range would get under 2 rows; the training grids are fixed
+    const unsigned grid = MODE == SX_INFER ? (unsigned)std::max<int64_t>(1, std::min<int64_t>(kX3Grid, (p.total_rows + 1) / 2)) : kX3Grid;
+    MB_CUDA(launch_dependent(st_x3<MODE>, grid, kThreadsX, kSmemX, st, p));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;
@@ -786,8 +841,21 @@ mb_status launch_sx(const SxParams& q, cudaStream_t st) {
 
 mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
     const int strips = (a.W + 2 + 31) / 32;
-    MB_CUDA(launch_dependent(st_conv1, kX3Grid, 256, 0, st, a.in, a.zmap, a.B, a.H, a.W, a.fw, a.h1, a.mask, strips,
-                             (int64_t)a.B * strips * (a.H + 2)));
+    SxConv1 c{};
+    c.in = a.in;
+    c.zmap = a.zmap;
+    c.in_slice = (int64_t)a.H * a.W;
+    c.in_pitch = a.W;
+    c.H = a.H;
+    c.W = a.W;
+    c.H1 = a.H + 2;
+    c.W1 = a.W + 2;
+    c.fw = a.fw;
+    c.h1 = a.h1;
+    c.mask = a.mask;
+    c.n_strips = strips;
+    c.total = (int64_t)a.B * strips * c.H1;
+    MB_CUDA(launch_dependent(st_conv1, kX3Grid, 256, 0, st, c));
     count_launch();
     SxParams p{};
     p.fw = a.fw;
@@ -802,7 +870,7 @@ mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
     p.dy2 = a.dy2;
     p.inv_n = a.inv_n;
     p.partial = a.part_fwd;
-    MB_TRY(launch_sx<false>(p, st));
+    MB_TRY(launch_sx<SX_FWD>(p, st));
     static bool attr = false;
     if (!attr) {
         MB_CUDA(cudaFuncSetAttribute(st_grad2, cudaFuncAttributeMaxDynamicSharedMemorySize, kG2Smem));
@@ -815,12 +883,50 @@ mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
     p.mask = a.mask;
     p.img = a.in;
     p.partial = a.part_bwd;
-    MB_TRY(launch_sx<true>(p, st));
+    MB_TRY(launch_sx<SX_BWD>(p, st));
     MB_CUDA(launch_dependent(st_reduce, (kSN + 1 + 31) / 32, 1024, 0, st, a.part_fwd, a.part_g2, a.part_bwd, a.inv_n, a.grad,
                              a.loss));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;
+}
+
+// Probabilities of a region of z slices: h1 of the region and one pixel around it, then conv2, head and
+// sigmoid. h1: [z][rows + 2][cols + 2][16] floats.
+mb_status student_x3_infer(const StudentX3Region& a, cudaStream_t st) {
+    SxConv1 c{};
+    c.in = a.in;
+    c.in_slice = a.in_slice;
+    c.in_pitch = a.in_pitch;
+    c.H = a.h;
+    c.W = a.w;
+    c.y0 = a.y0;
+    c.x0 = a.x0;
+    c.H1 = a.rows + 2;
+    c.W1 = a.cols + 2;
+    c.fw = a.fw;
+    c.h1 = a.h1;
+    c.n_strips = (c.W1 + 31) / 32;
+    c.total = (int64_t)a.z * c.n_strips * c.H1;
+    // an ordinary launch for the first chunk of a call: later launches read the weights before their wait
+    if (a.first)
+        st_conv1<<<kX3Grid, 256, 0, st>>>(c);
+    else
+        MB_CUDA(launch_dependent(st_conv1, kX3Grid, 256, 0, st, c));
+    count_launch();
+    MB_CUDA(cudaGetLastError());
+    SxParams p{};
+    p.in = a.h1;
+    p.fw = a.fw;
+    p.B = a.z;
+    p.H = a.rows;
+    p.W = a.cols;
+    p.out = a.out;
+    p.out_pitch = a.out_pitch;
+    p.out_slice = a.out_slice;
+    p.out_u8 = a.out_u8;
+    p.err = a.err;
+    return launch_sx<SX_INFER>(p, st);
 }
 
 }  // namespace mb

@@ -36,4 +36,17 @@ struct StudentX3 {
 };
 mb_status student_x3_grad(const StudentX3& a, cudaStream_t st);
 
+// One chunk of slices of an inference call (out_pitch, out_slice in elements).
+struct StudentX3Region {
+    const uint8_t* in;
+    int64_t in_slice, in_pitch, out_pitch, out_slice;
+    int z, h, w, y0, x0, rows, cols;
+    const float* fw;
+    float* h1;               // [z][rows + 2][cols + 2][16]
+    void* out;
+    int out_u8, first;       // first: the call's first chunk
+    int* err;
+};
+mb_status student_x3_infer(const StudentX3Region& a, cudaStream_t st);
+
 }  // namespace mb
