@@ -110,26 +110,7 @@ constexpr uint32_t kFmtF16 = 0;
 constexpr uint32_t kFmtE4M3 = 0;
 
 // ---- MMA ---------------------------------------------------------------------------------------
-// D[tmem] (+)= A[smem] x B[smem]^T, issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// The same (accumulating), executed where `on` is non-zero: a whole warp walks the issue loop, its
+// D[tmem] += A[smem] x B[smem]^T, executed where `on` is non-zero: a whole warp walks the issue loop, its
 // values in uniform registers, with one lane issuing. Descriptors as their two 32-bit words (the
 // start address is in the low one, so a caller steps that alone).
 __device__ __forceinline__ void mma_bf16_if(uint32_t on, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
@@ -219,42 +200,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Two loads of 32 lanes x 16 consecutive 32-bit columns per warp (e.g. two row accumulators) and one
-// wait for both, so the second load's latency overlaps the first.
-__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float (&v)[16], float (&u)[16]) {
-    uint32_t r[16], q[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%32];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%33];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
-          "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
-        : "r"(ta), "r"(tb)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        v[i] = __uint_as_float(r[i]);
-        u[i] = __uint_as_float(q[i]);
-    }
-}
-
-// Zero two blocks of 32 lanes x 16 consecutive columns per warp, with one wait.
-__device__ __forceinline__ void tmem_st16x2_zero(uint32_t ta, uint32_t tb) {
-    const uint32_t z = 0u;
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2};\n\t"
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%1], "
-        "{%2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2, %2};\n\t"
-        "tcgen05.wait::st.sync.aligned;" ::"r"(ta),
-        "r"(tb), "r"(z)
-        : "memory");
-}
-
 // 32 lanes x 4 consecutive 32-bit columns per warp, with its wait.
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
     uint32_t r[4];
@@ -298,17 +243,6 @@ __device__ __forceinline__ void tmem_st32_zero(uint32_t taddr) {
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
         "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
         "%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};\n\t"
-        "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
-        "r"(z)
-        : "memory");
-}
-
-// Zero 32 lanes x 16 consecutive 32-bit columns per warp, with its wait.
-__device__ __forceinline__ void tmem_st16_zero(uint32_t taddr) {
-    const uint32_t z = 0u;
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
-        "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};\n\t"
         "tcgen05.wait::st.sync.aligned;" ::"r"(taddr),
         "r"(z)
         : "memory");
