@@ -1243,13 +1243,23 @@ mb_status tc_infer_blocks(mb_net* net, const mb_block* blocks, int n_blocks, con
 
 namespace mb {
 
-__global__ void fill_bytes(uint8_t* p, int64_t n, uint32_t seed) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t x = (uint32_t)i * 2654435761u ^ seed;
+// The tuner's slices, grey values as an EM slice has them: bilinear value noise on an 8-pixel lattice and a
+// little sensor noise. The kernel's time depends on the values (clocks under power): on white noise 1,024-row
+// items beat the even split by 1.5 % on 1024 x 1024 x 32, on EM slices they lose by 5 %.
+__global__ void fill_slices(uint8_t* p, int64_t n, int h, int w, uint32_t seed) {
+    auto hash = [&](uint32_t a, uint32_t b, uint32_t c) {
+        uint32_t x = (a * 2654435761u) ^ (b * 2246822519u) ^ (c * 3266489917u) ^ seed;
         x ^= x >> 15;
         x *= 2246822519u;
         x ^= x >> 13;
-        p[i] = (uint8_t)(x >> 24);
+        return x >> 24;
+    };
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t x = (uint32_t)(i % w), y = (uint32_t)(i / w % h), z = (uint32_t)(i / w / h);
+        const uint32_t lx = x >> 3, ly = y >> 3, fx = x & 7, fy = y & 7;
+        const uint32_t top = hash(lx, ly, z) * (8 - fx) + hash(lx + 1, ly, z) * fx;
+        const uint32_t low = hash(lx, ly + 1, z) * (8 - fx) + hash(lx + 1, ly + 1, z) * fx;
+        p[i] = (uint8_t)(((top * (8 - fy) + low * fy) * 15 / 16 + hash(x, y, z + 7919u) * 4) >> 6);
     }
 }
 
@@ -1394,7 +1404,7 @@ mb_status tc_autotune(mb_net* net, int64_t z, int64_t h, int64_t w, const char* 
     MB_TRY(dev_alloc((void**)&in, (size_t)(z * h * w)));
     mb_status rc = dev_alloc((void**)&out, (size_t)(z * h * w) * 4);
     if (rc == MB_OK) {
-        fill_bytes<<<1024, 256, 0, st>>>(in, z * h * w, 12345u);
+        fill_slices<<<1024, 256, 0, st>>>(in, z * h * w, (int)h, (int)w, 12345u);
         count_launch();
         mb_block b;
         b.in = in;
