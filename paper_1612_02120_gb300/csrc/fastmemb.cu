@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(32 * kFirstWarps, 1) fm_first(const __grid_con
 #pragma unroll
             for (int i = 0; i < kIn; ++i)
                 if (lane + 32 * i < kFirstCols) {
-                    const float v = (float)u[i] / 255.0f;
+                    const float v = unit_of_byte(u[i]);
                     sx[r & 3][lane + 32 * i] = make_float2(v, v);
                 }
             if (r + 1 < n_in) fetch(r + 1);

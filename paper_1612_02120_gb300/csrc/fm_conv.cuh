@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256) fm_conv(const FmArgs a) {
                 if (ok) {
                     const uint8_t* src = static_cast<const uint8_t*>(a.in) + (int64_t)zi * a.in_slice;
                     const int sy = refl101(gy + a.off_y, a.src_h), sx = refl101(gx + a.off_x, a.src_w);
-                    v = (float)src[(int64_t)sy * a.in_pitch + sx] / 255.0f;
+                    v = unit_of_byte(src[(int64_t)sy * a.in_pitch + sx]);
                 }
                 s_in[r * IWP + c] = v;
             } else {

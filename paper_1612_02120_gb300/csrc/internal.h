@@ -34,6 +34,13 @@ void clear_error();
 mb_status cuda_fail(cudaError_t e, const char* what, const char* file, int line);
 void count_launch(int n = 1);
 
+// u / 255, correctly rounded. A zero numerator takes the division's slow path, and a whole warp with it, so
+// zero is divided as one and set back: FP32's 0 / 255 is 0.
+__device__ __forceinline__ float unit_of_byte(uint32_t u) {
+    const float q = (float)(u > 1u ? u : 1u) / 255.0f;
+    return u ? q : 0.f;
+}
+
 // A launch that may begin while the one before it on the stream still ends (programmatic dependent
 // launch): the kernel calls ptx::grid_dep_wait before it touches anything that an earlier launch
 // writes or reads, and the one before it calls ptx::grid_dep_launch where this one may set itself up.

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128) me_assemble(const uint8_t* __restrict__ e
     const int64_t o = (int64_t)refl101(r - kMeR, h) * w + refl101(c - kMeR, w);
     float v[16];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) v[k] = (float)em[(z + dz * (k - 1)) * hw + o] / 255.0f;
+    for (int k = 0; k < 3; ++k) v[k] = unit_of_byte(em[(z + dz * (k - 1)) * hw + o]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[3 + k] = (float)mk.m[k][o];
 #pragma unroll

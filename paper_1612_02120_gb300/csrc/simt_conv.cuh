@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(256) conv_simt(const ConvArgs a) {
                     const int zs = a.zmap ? a.zmap[zi] : zi;
                     const uint8_t* src = static_cast<const uint8_t*>(a.in) + (int64_t)zs * a.in_slice;
                     int sy = refl101(gy + a.off_y, a.src_h), sx = refl101(gx + a.off_x, a.src_w);
-                    v = (float)src[(int64_t)sy * a.in_pitch + sx] / 255.0f;
+                    v = unit_of_byte(src[(int64_t)sy * a.in_pitch + sx]);
                 }
                 s_in[r * IWP + c] = v;
             } else if (IN == IN_F32_PAD) {

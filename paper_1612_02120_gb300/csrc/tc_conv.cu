@@ -104,7 +104,8 @@ struct Cfg {
     static constexpr int oIn = oR2 + kRing * kSlotBytes;
     static constexpr int oSt2 = oIn + kInRing * kPitch * 4;
     static constexpr int oConst = oSt2 + 2 * 4 * 32 * 4;
-    static constexpr int oBar = oConst + kConsts * 4;
+    static constexpr int oLut = oConst + kConsts * 4;  // u / 255
+    static constexpr int oBar = oLut + 256 * 4;
     static constexpr int kBars = 2 * kInRing + 4 * kRing + 4 * 8 + 2;
     static constexpr int oMisc = oBar + kBars * 8;
     static constexpr int kSmem = oMisc + 16;
@@ -356,6 +357,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
         uint4* dst = reinterpret_cast<uint4*>(smem + C::oB);
         for (int i = tid; i < 2 * C::kLayerB / 16; i += kThreads) dst[i] = __ldg(src + i);
         const uint4* csrc = reinterpret_cast<const uint4*>(p.wpack + kWpackConstOff);
+        // a table: a division takes its slow path, and a whole warp with it, where a byte is zero (1024 x 1024 x
+        // 32 of zeros 3,274 us, of EM slices 2,430)
+        if (tid < 256) reinterpret_cast<float*>(smem + C::oLut)[tid] = (float)tid / 255.0f;
         uint4* cdst = reinterpret_cast<uint4*>(smem + C::oConst);
         for (int i = tid; i < kConsts / 4; i += kThreads) cdst[i] = __ldg(csrc + i);
         // zero the whole A rings once (the dx overrun pixels 128..135 are read but never written)
@@ -487,6 +491,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
 #pragma unroll
                 for (int i = 0; i < 5; ++i) v[i] = (lane + 32 * i < kInCols) ? (uint32_t)__ldg(row + sx[i]) : 0u;
             };
+            const float* lut = reinterpret_cast<const float*>(smem + C::oLut);
             uint32_t v[5];
             load_row(0, v);
             for (int u = 0; u < nrows; ++u) {
@@ -497,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_fused_teacher(const __grid_con
                 float* dst = in_ring + s * kPitch;
 #pragma unroll
                 for (int i = 0; i < 5; ++i)
-                    if (lane + 32 * i < kInCols) dst[lane + 32 * i] = (float)v[i] / 255.0f;
+                    if (lane + 32 * i < kInCols) dst[lane + 32 * i] = lut[v[i]];
                 if (!p.fault_stall) ptx::mbar_arrive(&B.in_full[s]);
 #pragma unroll
                 for (int i = 0; i < 5; ++i) v[i] = nv[i];
