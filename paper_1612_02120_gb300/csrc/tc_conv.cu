@@ -863,7 +863,17 @@ struct GraphCacheEntry {
 
 static TcState* state_of(mb_net* net) { return reinterpret_cast<TcState*>(net->tc_state); }
 
+static void drop_graphs(mb_net* net) {
+    for (GraphCacheEntry* g : net->graphs) {
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+        if (g->graph) cudaGraphDestroy(g->graph);
+        delete g;
+    }
+    net->graphs.clear();
+}
+
 mb_status tc_prepare(mb_net* net) {
+    drop_graphs(net);  // they hold the old layer-1 weights and head bias as kernel parameters
     const bool fp8 = net->prec == MB_PREC_FP8;
     if (fp8 && !net->calibrated) {
         // calibration provides the activation scales; until then only the FP32 pieces exist
@@ -959,15 +969,6 @@ mb_status tc_prepare(mb_net* net) {
     q.wpack = S->d_wpack;
     q.err = S->d_err;
     return MB_OK;
-}
-
-static void drop_graphs(mb_net* net) {
-    for (GraphCacheEntry* g : net->graphs) {
-        if (g->exec) cudaGraphExecDestroy(g->exec);
-        if (g->graph) cudaGraphDestroy(g->graph);
-        delete g;
-    }
-    net->graphs.clear();
 }
 
 void tc_release(mb_net* net) {

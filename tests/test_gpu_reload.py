@@ -1,0 +1,82 @@
+"""New weights in a net that has run before: every later call uses them, bitwise as a fresh net does. A
+batch is captured into a graph that the library keeps for the same block list; loading weights or
+calibrating again may not leave parts of the old ones in it. Through the C ABI."""
+import numpy as np
+import pytest
+
+import synth
+from _common import make_net, teacher_params
+
+pytestmark = pytest.mark.gpu
+
+T = synth.TEACHER
+SHAPES = [(2, 37, 130), (1, 64, 40)]
+
+
+def other_params(params, seed):
+    """Other weights of the same scales (biases and the head's among them)."""
+    rng = np.random.default_rng(seed)
+    return (params * rng.uniform(0.5, 1.5, params.size)).astype(np.float32)
+
+
+def batch_of(seed):
+    import torch
+    xs = [torch.from_numpy(synth.em_volume(seed + i, *s)).cuda() for i, s in enumerate(SHAPES)]
+    outs = [torch.empty(s, device="cuda") for s in SHAPES]
+    blocks = [(x, *s, s[2], s[1] * s[2], o, s[2], s[1] * s[2]) for x, o, s in zip(xs, outs, SHAPES)]
+    return xs, outs, blocks
+
+
+def run_batch(net, outs, blocks, per_block=False):
+    import torch
+    from paper_1612_02120_gb300 import membrane as m
+    for o in outs:
+        o.fill_(-1.0)
+    (m.mb_infer_batch_per_block if per_block else m.mb_infer_batch)(net.handle, blocks)
+    torch.cuda.synchronize()
+    return [o.cpu().numpy() for o in outs]
+
+
+def calibrate(net, seed, gain=1):
+    import torch
+    from paper_1612_02120_gb300 import membrane as m
+    v = np.minimum(synth.em_volume(seed, 2, 64, 64).astype(np.int64) // gain, 255).astype(np.uint8)
+    m.mb_calibrate_fp8(net.handle, torch.from_numpy(v).cuda(), 2, 64, 64)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp8"])
+def test_batch_after_a_reload_uses_the_new_weights(prec):
+    from paper_1612_02120_gb300 import build, membrane as m
+    build.build()
+    code = {"bf16": m.MB_PREC_BF16, "fp8": m.MB_PREC_FP8}[prec]
+    a, b = teacher_params(), other_params(teacher_params(), 5)
+    net, fresh = make_net(T, code, a), make_net(T, code, b)
+    for n in (net, fresh):
+        if prec == "fp8":
+            calibrate(n, 9100)
+    _, outs, blocks = batch_of(9000)
+    old = run_batch(net, outs, blocks)
+    net.load(b)
+    if prec == "fp8":
+        calibrate(net, 9100)
+    got = run_batch(net, outs, blocks)
+    for g, w, p, o in zip(got, run_batch(fresh, outs, blocks), run_batch(net, outs, blocks, True), old):
+        assert np.abs(g - o).max() > 1e-3
+        np.testing.assert_array_equal(g, w)
+        np.testing.assert_array_equal(g, p)
+    net.close()
+    fresh.close()
+
+
+def test_batch_after_a_second_calibration_uses_its_scales():
+    from paper_1612_02120_gb300 import build, membrane as m
+    build.build()
+    net = make_net(T, m.MB_PREC_FP8, teacher_params())
+    calibrate(net, 9100)
+    _, outs, blocks = batch_of(9000)
+    run_batch(net, outs, blocks)
+    calibrate(net, 9200, gain=2)
+    got = run_batch(net, outs, blocks)
+    for g, p in zip(got, run_batch(net, outs, blocks, True)):
+        np.testing.assert_array_equal(g, p)
+    net.close()
