@@ -504,13 +504,13 @@ mb_status mb_net_create(const mb_layer_desc* layers, int32_t n_layers, mb_precis
     {
         DeviceGuard g(device);
         mb_status s = g.err == cudaSuccess ? MB_OK : cuda_fail(g.err, "cudaSetDevice", __FILE__, __LINE__);
-        if (s == MB_OK) s = dev_alloc((void**)&net->d_queue, 64 * sizeof(int));
+        if (s == MB_OK) s = dev_alloc((void**)&net->d_tag, sizeof(uint32_t));
         if (s == MB_OK) {
-            cudaError_t e = cudaMemset(net->d_queue, 0, 64 * sizeof(int));
+            cudaError_t e = cudaMemset(net->d_tag, 0, sizeof(uint32_t));
             if (e != cudaSuccess) s = cuda_fail(e, "cudaMemset", __FILE__, __LINE__);
         }
         if (s != MB_OK) {
-            dev_free(net->d_queue);
+            dev_free(net->d_tag);
             delete net;
             return s;
         }
@@ -533,7 +533,7 @@ mb_status mb_net_destroy(mb_net* net) {
         if (net->train_host) cudaFreeHost(net->train_host);
         dev_free(net->d_params);
         dev_free(net->d_simt);
-        dev_free(net->d_queue);
+        dev_free(net->d_tag);
         net->ws.release();
         net->ws2.release();
         net->slab_ws.release();
@@ -553,6 +553,13 @@ mb_status mb_net_param_count(const mb_net* net, int64_t* n_params) {
         return MB_ERR_INVALID_ARG;
     }
     *n_params = net->n_params;
+    return MB_OK;
+}
+
+// Launches captured from here on take the present weights along; those captured before see that they are old.
+static mb_status weights_changed(mb_net* net) {
+    ++net->tag;
+    MB_CUDA(cudaMemcpy(net->d_tag, &net->tag, sizeof(net->tag), cudaMemcpyHostToDevice));
     return MB_OK;
 }
 
@@ -587,6 +594,7 @@ mb_status mb_load_weights(mb_net* net, const float* params, int64_t n_params) {
     net->simt_floats = packed.size();
     MB_CUDA(cudaMemcpy(net->d_params, params, sizeof(float) * n_params, cudaMemcpyHostToDevice));
     MB_CUDA(cudaMemcpy(net->d_simt, packed.data(), sizeof(float) * packed.size(), cudaMemcpyHostToDevice));
+    MB_TRY(weights_changed(net));
     net->calibrated = false;
     net->loaded = true;
     if (net->family == FAMILY_TEACHER && net->prec == MB_PREC_BF16) MB_TRY(tc_prepare(net));
@@ -653,6 +661,7 @@ mb_status mb_calibrate_fp8(mb_net* net, const uint8_t* slices, int64_t n, int64_
         for (int c = 0; c < 32; ++c) net->fp8_amax[m][c] = host[m * 32 + c];
     if (amax_out) memcpy(amax_out, host, sizeof(host));
     MB_TRY(tc_prepare(net));
+    MB_TRY(weights_changed(net));
     net->calibrated = true;
     return MB_OK;
 }

@@ -91,6 +91,13 @@ struct Workspace {
 
 struct GraphCacheEntry;
 
+// Which weights a launch took along as kernel parameters. Parameters are fixed when a launch is captured in
+// a caller's CUDA graph, while device weights follow mb_load_weights: a kernel whose `taken` is no longer
+// the net's count (*word) reads its weights from device memory instead.
+struct WeightsTag {
+    const uint32_t* word;
+    uint32_t taken;
+};
 }  // namespace mb
 
 struct mb_net {
@@ -104,6 +111,8 @@ struct mb_net {
     bool calibrated = false;
     float* d_params = nullptr;   // FP32 parameters, API layout (student: the master copy)
     float* d_simt = nullptr;     // SIMT layout: per conv layer Wt[ci][ky][kx][co], b[co]; head w, b
+    uint32_t tag = 0;            // counts the changes of the weights (and FP8 scales)
+    uint32_t* d_tag = nullptr;   // the same on the device (WeightsTag)
     size_t simt_floats = 0;
     void* tc_state = nullptr;    // tensor-core path state (packed operands, constants), tc_conv.cu
     void* fm_state = nullptr;    // FastMemb tensor-core state (packed operands, error word), fastmemb_tc.cu
@@ -130,7 +139,6 @@ struct mb_net {
     bool tuned = false;
     // batch graph cache
     std::vector<mb::GraphCacheEntry*> graphs;
-    int* d_queue = nullptr;      // work-queue counter + error word (device)
 };
 
 namespace mb {

@@ -80,3 +80,76 @@ def test_batch_after_a_second_calibration_uses_its_scales():
     for g, p in zip(got, run_batch(net, outs, blocks, True)):
         np.testing.assert_array_equal(g, p)
     net.close()
+
+
+# --- calls captured in a caller's own graph -------------------------------------------------------
+
+VOL = (2, 70, 140)
+
+
+def net_and_other(layers, code, params, seed):
+    """A net with its weights, a second one with others, and those."""
+    from paper_1612_02120_gb300 import build
+    build.build()
+    b = other_params(params, seed)
+    return make_net(layers, code, params), make_net(layers, code, b), b
+
+
+def captured_volume(net, shape=VOL, sub=1):
+    """A captured mb_infer_volume of `shape` on new bytes, its output, and the same call made at once."""
+    import torch
+    from paper_1612_02120_gb300 import membrane as m
+    x = torch.from_numpy(synth.em_volume(9300, *shape)).cuda()
+    z, h, w = shape
+    out = torch.zeros((z, -(-h // sub), -(-w // sub)), device="cuda")
+
+    def call(n, o):
+        st = torch.cuda.current_stream()
+        if sub == 1:
+            m.mb_infer_volume(n.handle, x, z, h, w, o, stream=st)
+        else:
+            m.mb_infer_volume_subsampled(n.handle, x, z, h, w, sub, o, stream=st)
+
+    call(net, out)  # the workspace grows outside the capture
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(net, out)
+
+    def replayed():
+        out.fill_(-1.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        return out.cpu().numpy()
+
+    def at_once(n):
+        o = torch.full_like(out, -2.0)
+        call(n, o)
+        torch.cuda.synchronize()
+        return o.cpu().numpy()
+
+    return replayed, at_once
+
+
+def check_replay(net, fresh, new, prepare=lambda n: None, **kw):
+    for n in (net, fresh):
+        prepare(n)
+    replayed, at_once = captured_volume(net, **kw)
+    old = replayed()
+    np.testing.assert_array_equal(old, at_once(net))
+    net.load(new)
+    prepare(net)
+    got = replayed()
+    assert np.abs(got - old).max() > 1e-3
+    np.testing.assert_array_equal(got, at_once(fresh))
+    np.testing.assert_array_equal(at_once(net), got)
+    net.close()
+    fresh.close()
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp8"])
+def test_captured_teacher_follows_a_reload(prec):
+    from paper_1612_02120_gb300 import membrane as m
+    code = {"bf16": m.MB_PREC_BF16, "fp8": m.MB_PREC_FP8}[prec]
+    check_replay(*net_and_other(T, code, teacher_params(), 6),
+                 prepare=(lambda n: calibrate(n, 9100)) if prec == "fp8" else (lambda n: None))
