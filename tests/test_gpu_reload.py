@@ -153,3 +153,11 @@ def test_captured_teacher_follows_a_reload(prec):
     code = {"bf16": m.MB_PREC_BF16, "fp8": m.MB_PREC_FP8}[prec]
     check_replay(*net_and_other(T, code, teacher_params(), 6),
                  prepare=(lambda n: calibrate(n, 9100)) if prec == "fp8" else (lambda n: None))
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+@pytest.mark.parametrize("sub", [1, 2])
+def test_captured_fastmemb_follows_a_reload(prec, sub):
+    from paper_1612_02120_gb300 import membrane as m
+    code = {"bf16": m.MB_PREC_BF16, "fp16": m.MB_PREC_FP16}[prec]
+    check_replay(*net_and_other(synth.FASTMEMB, code, synth.init_params(synth.FASTMEMB, 99, bias_std=0.01), 7), sub=sub)
