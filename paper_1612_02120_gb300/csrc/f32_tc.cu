@@ -68,8 +68,10 @@ struct XCfg {
     static constexpr int kRing = K == 5 ? 2 : 4;      // staged rows
     static constexpr int oB = 0;
     static constexpr int oRing = oB + kBBytes;
-    static constexpr int oConst = oRing + kRing * kSlot;  // bias[32], head w[32]
-    static constexpr int oHead = oConst + 64 * 4;         // partial head sums, two rows in turn
+    static constexpr int kConsts = 68;                    // bias[32], head w[32], head b, 3 unused
+    static constexpr int kPack = kBBytes + kConsts * 4;   // bytes of one half's operands
+    static constexpr int oConst = oRing + kRing * kSlot;
+    static constexpr int oHead = oConst + kConsts * 4;    // partial head sums, two rows in turn
     static constexpr int oBar = oHead + (OUT == X_HEAD ? 2 * 128 * 4 : 0);
     static constexpr int kBars = 2 * kRing + 2 * kBufs + 1;
     static constexpr int oMisc = oBar + kBars * 8;
@@ -89,8 +91,7 @@ struct XParams {
     int64_t out_slice, out_pitch;
     int out_h, out_w, nz, n_strips;
     int64_t total_rows;          // strip-rows per half: nz x n_strips x out_h
-    const uint8_t* wpack;        // per half: B blocks, then bias[32], head w[32]
-    float hb;
+    const uint8_t* wpack;        // per half: B blocks, then the constants
     int halves, out_u8;
     int* err;
     int fault_stall;             // test injection: producers withhold their arrivals
@@ -165,11 +166,11 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
         ptx::mbar_fence_init();
     }
     {
-        const uint4* src = reinterpret_cast<const uint4*>(p.wpack + (size_t)half * (C::kBBytes + 256));
+        const uint4* src = reinterpret_cast<const uint4*>(p.wpack + (size_t)half * C::kPack);
         uint4* dst = reinterpret_cast<uint4*>(smem + C::oB);
         for (int i = tid; i < C::kBBytes / 16; i += C::kThreads) dst[i] = __ldg(src + i);
         uint4* cdst = reinterpret_cast<uint4*>(smem + C::oConst);
-        if (tid < 16) cdst[tid] = __ldg(src + C::kBBytes / 16 + tid);
+        if (tid < C::kConsts / 4) cdst[tid] = __ldg(src + C::kBBytes / 16 + tid);
     }
     if (warp == 0) {
         ptx::tmem_alloc(tmem_slot, 512);
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(640, 1) x3_conv(const __grid_constant__ XParam
                     if (g == 1) h[px] = z;
                     asm volatile("bar.sync 2, 256;" ::: "memory");
                     if (g == 0 && store) {
-                        const float prob = 1.0f / (1.0f + expf(-((z + h[px]) + p.hb)));
+                        const float prob = 1.0f / (1.0f + expf(-((z + h[px]) + cst[64])));
                         const int64_t idx = (int64_t)it.z * p.out_slice + (int64_t)y * p.out_pitch + x;
                         if (p.out_u8)
                             static_cast<uint8_t*>(p.out)[idx] = (uint8_t)fminf(floorf(255.0f * prob + 0.5f), 255.0f);
@@ -406,12 +407,12 @@ uint16_t part_bits(float& f) {
 }
 
 // One half's operands: conv channels c0 .. c0 + 31 of W[co][32][K][K], b[co]: B blocks [chunk kc][row
-// 32 ky + c][8 BF16], ci = 16 h + 8 kc + e, per (part, kx, K-half h); then bias[32], head w[32].
+// 32 ky + c][8 BF16], ci = 16 h + 8 kc + e, per (part, kx, K-half h); then bias[32], head w[32] and b.
 template <int K>
 void x3_pack(const float* W, const float* b, int c0, const float* head, std::vector<uint8_t>& out) {
     using C = XCfg<K, X_RELU>;
     const size_t base = out.size();
-    out.resize(base + C::kBBytes + 256, 0);
+    out.resize(base + C::kPack, 0);
     uint8_t* o = out.data() + base;
     for (int c = 0; c < 32; ++c)
         for (int g = 0; g < 4; ++g) {  // input channels 8 g .. 8 g + 7: one 16-byte chunk per (part, tap)
@@ -429,7 +430,7 @@ void x3_pack(const float* W, const float* b, int c0, const float* head, std::vec
                 }
         }
     memcpy(o + C::kBBytes, b + c0, 32 * 4);
-    if (head) memcpy(o + C::kBBytes + 128, head, 32 * 4);
+    if (head) memcpy(o + C::kBBytes + 128, head, 33 * 4);
 }
 
 template <int K, int OUT>
@@ -458,7 +459,6 @@ struct X3State {
     uint8_t* d_w[4] = {};  // the packed layers, parts of one allocation (d_w[0])
     int* h_err = nullptr;
     int* d_err = nullptr;
-    float hb = 0.f;
 };
 
 X3State* x3_of(const mb_net* net) { return reinterpret_cast<X3State*>(net->x3_state); }
@@ -498,8 +498,8 @@ mb_status x3_prepare(mb_net* net) {
         }
         net->x3_state = S;
     }
+    // (packed whatever the bound: a call captured with other weights in a caller's graph replays these layers)
     net->x3_ok = false;
-    if (!x3_bounded(net)) return MB_OK;
     const int n = teacher ? 2 : fastmemb_convs(net->family) - 2;
     const float* P = net->host_params.data() + (teacher ? 832 : 64 * 16 + 64);
     std::vector<uint8_t> pk;
@@ -518,7 +518,6 @@ mb_status x3_prepare(mb_net* net) {
     if (!S->d_w[0]) MB_TRY(dev_alloc((void**)&S->d_w[0], pk.size()));
     for (int l = 1; l < n; ++l) S->d_w[l] = S->d_w[0] + at[l];
     MB_CUDA(cudaMemcpy(S->d_w[0], pk.data(), pk.size(), cudaMemcpyHostToDevice));
-    if (teacher) S->hb = P[32];
     if (!S->h_err) {
         if (fault_oom()) {
             set_error("pinned allocation failed (MB_FAULT_OOM injected)");
@@ -528,7 +527,7 @@ mb_status x3_prepare(mb_net* net) {
         *S->h_err = 0;
         MB_CUDA(cudaHostGetDevicePointer((void**)&S->d_err, S->h_err, 0));
     }
-    net->x3_ok = true;
+    net->x3_ok = x3_bounded(net);
     return MB_OK;
 }
 
@@ -581,7 +580,6 @@ mb_status x3_layer(const mb_net* net, int layer, const X3Layer& a, cudaStream_t 
     p.n_strips = (a.out_w + 127) / 128;
     p.total_rows = (int64_t)a.nz * p.n_strips * a.out_h;
     p.wpack = S->d_w[layer];
-    p.hb = S->hb;
     p.halves = teacher ? 1 : 2;
     p.out_u8 = a.out_u8;
     p.err = S->d_err;

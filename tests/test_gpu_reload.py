@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import synth
-from _common import make_net, teacher_params
+from _common import make_net, student_params, teacher_params
 
 pytestmark = pytest.mark.gpu
 
@@ -161,3 +161,35 @@ def test_captured_fastmemb_follows_a_reload(prec, sub):
     from paper_1612_02120_gb300 import membrane as m
     code = {"bf16": m.MB_PREC_BF16, "fp16": m.MB_PREC_FP16}[prec]
     check_replay(*net_and_other(synth.FASTMEMB, code, synth.init_params(synth.FASTMEMB, 99, bias_std=0.01), 7), sub=sub)
+
+
+@pytest.mark.parametrize("kind", ["teacher", "fastmemb", "student", "student_bf16"])
+def test_captured_fp32_and_student_calls_follow_a_reload(kind):
+    from paper_1612_02120_gb300 import membrane as m
+    layers, code, params = {
+        "teacher": (T, m.MB_PREC_FP32, teacher_params()),
+        "fastmemb": (synth.FASTMEMB, m.MB_PREC_FP32, synth.init_params(synth.FASTMEMB, 99, bias_std=0.01)),
+        "student": (synth.STUDENT, m.MB_PREC_FP32, student_params()),
+        "student_bf16": (synth.STUDENT, m.MB_PREC_BF16, student_params())}[kind]
+    check_replay(*net_and_other(layers, code, params, 8))
+
+
+def test_captured_fp32_call_follows_weights_that_the_split_layers_refuse():
+    """The new weights are the other net's with the first layer times 2^104 and the second over 2^104: the
+    same network exactly, but beyond the bound of the split layers, so later calls take the CUDA cores. The
+    captured call keeps its layers and gets the new weights; 2e-6 is the two paths' distance (see
+    test_gpu_f32_tc)."""
+    from paper_1612_02120_gb300 import membrane as m
+    net, fresh, b = net_and_other(T, m.MB_PREC_FP32, teacher_params(), 8)
+    replayed, at_once = captured_volume(net)
+    old = replayed()
+    big = b.copy()
+    big[:832] *= np.float32(2.0 ** 104)
+    big[832:832 + 25600] /= np.float32(2.0 ** 104)
+    net.load(big)
+    got = replayed()
+    assert np.abs(got - old).max() > 1e-3
+    assert np.abs(got - at_once(fresh)).max() <= 2e-6
+    assert np.abs(at_once(net) - at_once(fresh)).max() <= 2e-6
+    net.close()
+    fresh.close()
