@@ -467,21 +467,30 @@ X3State* x3_of(const mb_net* net) { return reinterpret_cast<X3State*>(net->x3_st
 
 // Whether no input can drive an activation of the net beyond 2^100 (finite with room for the sums):
 // max |feature| of a layer <= max |b| + (max over filters of the sum of |w|) x max |feature| before it.
+// And whether no layer before the head lives, with its features or its weights, wholly below 2^-60: the
+// trailing part of a value is 2^-24 of it, and BF16 ends at 2^-133 (a first layer times 2^-118 with the second
+// over 2^-118, the same network exactly, would lose its third parts: 2^-16 instead of 2^-24).
 static bool x3_bounded(const mb_net* net) {
     const float* P = net->host_params.data();
+    const double least = 8.7e-19;
     double bound = 1.0;
     for (const mb_layer_desc& L : net->layers) {
         if (L.kind == MB_MAXFILTER) continue;
+        const bool head = L.kind != MB_CONV;
         const int co = L.cout * std::max(1, L.maxout_groups), k = L.cin * L.ksize * L.ksize;
-        double worst = 0.0;
+        double worst = 0.0, wmax = 0.0;
         for (int c = 0; c < co; ++c) {
             double s = std::fabs((double)P[(size_t)co * k + c]);
-            for (int i = 0; i < k; ++i) s += bound * std::fabs((double)P[(size_t)c * k + i]);
+            for (int i = 0; i < k; ++i) {
+                const double w = std::fabs((double)P[(size_t)c * k + i]);
+                wmax = std::max(wmax, w);
+                s += bound * w;
+            }
             worst = std::max(worst, s);
         }
         bound = worst;
         P += (size_t)co * k + co;
-        if (!(bound < 1.2e30)) return false;
+        if (!(bound < 1.2e30) || (!head && (bound < least || wmax < least))) return false;
     }
     return true;
 }
