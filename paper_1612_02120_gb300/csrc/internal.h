@@ -119,7 +119,9 @@ struct mb_net {
     void* me_state = nullptr;    // MaskExtend tensor-core state (packed operands, error word), maskextend_tc.cu
     void* x3_state = nullptr;    // FP32 tensor-core layers (packed split operands, error word), f32_tc.cu
     bool x3_ok = false;          // its activations are bounded: those layers run on the tensor cores
-    int* train_host = nullptr;   // mapped host words of the student's training: error word, loss of the last gradient
+    // mapped host words of the FP32-accurate student passes: error word of the training, loss of the last
+    // gradient, error word of the inference
+    int* train_host = nullptr;
     int* train_dev = nullptr;    // their device address
     void* st_state = nullptr;    // student tensor-core state (packed operands, error word), student_tc.cu
     float fp8_amax[2][32] = {};

@@ -419,20 +419,28 @@ static mb_status train_words(mb_net* s) {
         set_error("pinned allocation failed (MB_FAULT_OOM injected)");
         return MB_ERR_OOM;
     }
-    MB_CUDA(cudaHostAlloc((void**)&s->train_host, 2 * sizeof(int), cudaHostAllocMapped));
-    s->train_host[0] = s->train_host[1] = 0;
+    MB_CUDA(cudaHostAlloc((void**)&s->train_host, 3 * sizeof(int), cudaHostAllocMapped));
+    s->train_host[0] = s->train_host[1] = s->train_host[2] = 0;
     MB_CUDA(cudaHostGetDevicePointer((void**)&s->train_dev, s->train_host, 0));
     return MB_OK;
 }
 
-// The error word after a synchronisation.
+static bool train_gave_up(const mb_net* s) { return s->train_host && *(volatile int*)s->train_host; }
+
+// The training's error word, after a synchronisation.
 static mb_status train_error(mb_net* s) {
-    if (s->train_host && *(volatile int*)s->train_host) {
-        *(volatile int*)s->train_host = 0;
-        set_error("a training launch gave up waiting (device-side wait limit)");
-        return MB_ERR_TIMEOUT;
-    }
-    return MB_OK;
+    if (!train_gave_up(s)) return MB_OK;
+    *(volatile int*)s->train_host = 0;
+    set_error("a training launch gave up waiting (device-side wait limit)");
+    return MB_ERR_TIMEOUT;
+}
+
+// The inference's (asynchronous calls: reported by the next call that looks).
+static mb_status infer_error(mb_net* s) {
+    if (!s->train_host || !*(volatile int*)(s->train_host + 2)) return MB_OK;
+    *(volatile int*)(s->train_host + 2) = 0;
+    set_error("an FP32 student launch gave up waiting (device-side wait limit)");
+    return MB_ERR_TIMEOUT;
 }
 
 // The split passes where no activation can pass 2^70 (train_bounded), else the CUDA-core layers; the choice
@@ -444,7 +452,7 @@ mb_status student_f32_region(mb_net* s, const uint8_t* in, int64_t z, int64_t h,
         return simt_student_region(s, in, z, h, w, in_pitch, in_slice, y0, x0, rows, cols, out, out_pitch, out_slice, ot, st);
     if (z == 0 || rows == 0 || cols == 0) return MB_OK;
     MB_TRY(train_words(s));
-    MB_TRY(train_error(s));
+    MB_TRY(infer_error(s));
     const size_t per = (size_t)(rows + 2) * (size_t)(cols + 2) * 16 * sizeof(float);
     const int64_t zc = chunk_slices(per, z);
     MB_TRY(s->ws.ensure(per * (size_t)zc));
@@ -462,7 +470,7 @@ mb_status student_f32_region(mb_net* s, const uint8_t* in, int64_t z, int64_t h,
     a.fw = s->d_simt;
     a.h1 = static_cast<float*>(s->ws.ptr);
     a.out_u8 = ot == MB_OUT_U8 ? 1 : 0;
-    a.err = s->train_dev;
+    a.err = s->train_dev + 2;
     for (int64_t z0 = 0; z0 < z; z0 += zc) {
         a.in = in + z0 * in_slice;
         a.z = (int)std::min<int64_t>(zc, z - z0);
@@ -470,7 +478,7 @@ mb_status student_f32_region(mb_net* s, const uint8_t* in, int64_t z, int64_t h,
         a.first = z0 == 0;
         MB_TRY(student_x3_infer(a, st));
     }
-    return train_error(s);
+    return infer_error(s);
 }
 
 // Carves the training workspace; every sub-buffer starts on a 256-byte boundary (the convolution
@@ -627,6 +635,7 @@ mb_status student_loss_grad(mb_net* s, const uint8_t* in, const float* tgt, int6
     StudentBufs b;
     const bool x3 = train_bounded(s->host_params.data(), 0.0);
     MB_TRY(ensure_bufs(s, n, h, w, 1, x3, b));
+    MB_TRY(train_error(s));
     MB_TRY(pack_forward(s, b, st));
     if (x3) {  // straight into the caller's gradient; the loss through the mapped word
         b.grad = grad;
@@ -730,6 +739,18 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
     const bool x3 = train_bounded(found == CkptRead::kOk ? buf.data() : s->host_params.data(), adam_drift(cfg));
     StudentBufs b;
     MB_TRY(ensure_bufs(s, B, h, w, cfg->steps, x3, b));
+    MB_TRY(train_error(s));
+    // After a wait that ran out the gradients are not to be trusted: nothing of the run is kept, neither in the
+    // net (its weights are those of before the call again) nor in the checkpoint or the curve.
+    auto trained = [&]() -> mb_status {
+        MB_CUDA(cudaStreamSynchronize(st));
+        const mb_status err = train_error(s);
+        if (err == MB_OK) return MB_OK;
+        MB_CUDA(cudaMemcpyAsync(s->d_params, s->host_params.data(), kSN * 4, cudaMemcpyHostToDevice, st));
+        MB_TRY(pack_forward(s, b, st));
+        MB_CUDA(cudaStreamSynchronize(st));
+        return err;
+    };
     if (found == CkptRead::kOk) {
         start = hd.step;
         MB_CUDA(cudaMemcpyAsync(s->d_params, buf.data(), kSN * 4, cudaMemcpyHostToDevice, st));
@@ -762,19 +783,20 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
                                  cfg->lr, cfg->beta1, cfg->beta2, cfg->eps, (float)c1, (float)c2));
         count_launch();
         MB_CUDA(cudaGetLastError());
+        if (train_gave_up(s)) break;
         if (ckpt && cfg->ckpt_every > 0 && step % cfg->ckpt_every == 0) {
+            MB_TRY(trained());
             hd.step = step;
             hd.sampler = sampler_after[(size_t)k];
             MB_TRY(write_ckpt(ckpt, hd, s->d_params, b.m, b.v, st));
         }
     }
     MB_TRY(pack_forward(s, b, st));
-    if (curve && nsteps > 0)
-        MB_CUDA(cudaMemcpyAsync(curve, b.losses, nsteps * sizeof(float), cudaMemcpyDeviceToHost, st));
-    MB_CUDA(cudaStreamSynchronize(st));
+    MB_TRY(trained());
+    if (curve && nsteps > 0) MB_CUDA(cudaMemcpy(curve, b.losses, nsteps * sizeof(float), cudaMemcpyDeviceToHost));
     // the host master copy follows the device
     MB_CUDA(cudaMemcpy(s->host_params.data(), s->d_params, kSN * 4, cudaMemcpyDeviceToHost));
-    return train_error(s);
+    return MB_OK;
 }
 
 // ---- cascade -------------------------------------------------------------------------------------
