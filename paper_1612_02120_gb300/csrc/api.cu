@@ -292,6 +292,15 @@ static mb_status net_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h
     return student_region(net, in, z, h, w, w, h * w, y0, x0, rows, cols, out, cols, rows * cols, ot, st);
 }
 
+mb_status net_poll_error(mb_net* net) {
+    mb_status rc = MB_OK;
+    for (auto poll : {tc_poll_error, fm_tc_poll_error, me_tc_poll_error, st_tc_poll_error, x3_poll_error, student_f32_poll_error}) {
+        const mb_status s = poll(net);
+        if (rc == MB_OK) rc = s;
+    }
+    return rc;
+}
+
 // Host-memory volumes. Mapped page-locked buffers on a coherent link: the kernels access them
 // directly. Otherwise z-slabs through double-buffered device slabs, H2D / compute / D2H on their
 // own streams so copies overlap compute (the tensor-core teacher computes on two alternating
@@ -311,9 +320,11 @@ static mb_status infer_host_volume(mb_net* net, const uint8_t* in, int64_t z, in
         void* mo = mi ? mapped_host_ptr(out) : nullptr;
         if (mi && mo) {
             if (!s[1]) MB_CUDA(cudaStreamCreateWithFlags(&s[1], cudaStreamNonBlocking));
-            MB_TRY(net_region(net, static_cast<const uint8_t*>(mi), z, h, w, 0, 0, h, w, mo, ot, s[1]));
-            MB_CUDA(cudaStreamSynchronize(s[1]));
-            return MB_OK;
+            const mb_status rc = net_region(net, static_cast<const uint8_t*>(mi), z, h, w, 0, 0, h, w, mo, ot, s[1]);
+            const cudaError_t e = cudaStreamSynchronize(s[1]);
+            const mb_status late = net_poll_error(net);
+            if (rc == MB_OK) MB_CUDA(e);
+            return rc != MB_OK ? rc : late;
         }
     }
     // Slabs of about 8 Mvox: large enough that one launch fills every SM, small enough that the
@@ -388,7 +399,8 @@ static mb_status infer_host_volume(mb_net* net, const uint8_t* in, int64_t z, in
         cudaError_t e = cudaStreamSynchronize(s[i]);
         if (e != cudaSuccess && rc == MB_OK) fail(e, "cudaStreamSynchronize");
     }
-    return rc;
+    const mb_status late = net_poll_error(net);
+    return rc != MB_OK ? rc : late;
 }
 
 static uint16_t f32_to_bf16_bits(float f) {

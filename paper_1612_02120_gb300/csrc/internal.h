@@ -208,6 +208,11 @@ mb_status st_tc_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int
                        int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
                        int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st);
 void st_tc_release(mb_net* net);
+mb_status st_tc_poll_error(mb_net* net);
+mb_status student_f32_poll_error(mb_net* net);  // the FP32 student's inference
+// MB_ERR_TIMEOUT (and every error word of the net cleared) if a launch of an inference on this net gave up
+// waiting: what a call that has synchronised returns, so that MB_OK means complete maps.
+mb_status net_poll_error(mb_net* net);
 mb_status student_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,
                          int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
                          int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st);

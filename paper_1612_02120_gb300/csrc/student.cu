@@ -436,7 +436,7 @@ static mb_status train_error(mb_net* s) {
 }
 
 // The inference's (asynchronous calls: reported by the next call that looks).
-static mb_status infer_error(mb_net* s) {
+mb_status student_f32_poll_error(mb_net* s) {
     if (!s->train_host || !*(volatile int*)(s->train_host + 2)) return MB_OK;
     *(volatile int*)(s->train_host + 2) = 0;
     set_error("an FP32 student launch gave up waiting (device-side wait limit)");
@@ -452,7 +452,7 @@ mb_status student_f32_region(mb_net* s, const uint8_t* in, int64_t z, int64_t h,
         return simt_student_region(s, in, z, h, w, in_pitch, in_slice, y0, x0, rows, cols, out, out_pitch, out_slice, ot, st);
     if (z == 0 || rows == 0 || cols == 0) return MB_OK;
     MB_TRY(train_words(s));
-    MB_TRY(infer_error(s));
+    MB_TRY(student_f32_poll_error(s));
     const size_t per = (size_t)(rows + 2) * (size_t)(cols + 2) * 16 * sizeof(float);
     const int64_t zc = chunk_slices(per, z);
     MB_TRY(s->ws.ensure(per * (size_t)zc));
@@ -478,7 +478,7 @@ mb_status student_f32_region(mb_net* s, const uint8_t* in, int64_t z, int64_t h,
         a.first = z0 == 0;
         MB_TRY(student_x3_infer(a, st));
     }
-    return infer_error(s);
+    return student_f32_poll_error(s);
 }
 
 // Carves the training workspace; every sub-buffer starts on a 256-byte boundary (the convolution
@@ -928,8 +928,8 @@ mb_status cascade(mb_net* s, mb_net* t, const uint8_t* in, int64_t z, int64_t h,
         *rate = (double)nflag / (double)ntiles;
     } while (0);
     dev_free(d_flags);
-    if (rc == MB_OK) rc = tc_poll_error(t);
-    return rc;
+    const mb_status es = net_poll_error(s), et = net_poll_error(t);
+    return rc != MB_OK ? rc : es != MB_OK ? es : et;
 }
 
 }  // namespace mb

@@ -625,6 +625,16 @@ void st_tc_release(mb_net* net) {
     net->st_state = nullptr;
 }
 
+mb_status st_tc_poll_error(mb_net* net) {
+    StTcState* S = reinterpret_cast<StTcState*>(net->st_state);
+    if (S && S->h_err && *(volatile int*)S->h_err) {
+        *(volatile int*)S->h_err = 0;
+        set_error("a student tensor-core launch gave up waiting (device-side wait limit)");
+        return MB_ERR_TIMEOUT;
+    }
+    return MB_OK;
+}
+
 mb_status st_tc_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int64_t w, int64_t in_pitch,
                        int64_t in_slice, int64_t y0, int64_t x0, int64_t rows, int64_t cols, void* out,
                        int64_t out_pitch, int64_t out_slice, mb_out_type ot, cudaStream_t st) {
@@ -648,11 +658,7 @@ mb_status st_tc_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int
         *S->h_err = 0;
         MB_CUDA(cudaHostGetDevicePointer((void**)&S->d_err, S->h_err, 0));
     }
-    if (*(volatile int*)S->h_err) {
-        *(volatile int*)S->h_err = 0;
-        set_error("a student tensor-core launch gave up waiting (device-side wait limit)");
-        return MB_ERR_TIMEOUT;
-    }
+    MB_TRY(st_tc_poll_error(net));
     if (!S->n_sms) {
         int dev = 0;
         MB_CUDA(cudaGetDevice(&dev));
