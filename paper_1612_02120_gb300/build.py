@@ -16,6 +16,7 @@ SOURCES = ["api.cu", "simt_conv.cu", "tc_conv.cu", "student.cu", "noalloc.cu", "
            "maskextend_tc.cu", "student_tc.cu", "f32_tc.cu", "student_x3.cu"]
 HEADERS = [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "tc_ptx.cuh"), os.path.join(CSRC, "simt_conv.cuh"),
            os.path.join(CSRC, "fm_conv.cuh"), os.path.join(CSRC, "f32_split.cuh"), os.path.join(CSRC, "student_x3.h"),
+           os.path.join(CSRC, "per_device.h"),
            os.path.join(ROOT, "include", "membrane.h")]
 
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

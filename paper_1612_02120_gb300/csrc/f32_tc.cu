@@ -442,11 +442,8 @@ mb_status launch_x3(XParams& p, cudaStream_t st) {
         MB_CUDA(cudaGetDevice(&dev));
         MB_CUDA(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    static bool attr = false;
-    if (!attr) {
-        MB_CUDA(cudaFuncSetAttribute(x3_conv<K, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem));
-        attr = true;
-    }
+    static std::atomic<uint64_t> smem_set{0};
+    MB_TRY(set_smem_once(smem_set, x3_conv<K, OUT>, C::kSmem));
     // one range per SM, or fewer when a range would get under 2 rows (each costs K - 1 more staged rows)
     const int64_t per_half = std::max<int64_t>(1, std::min<int64_t>(n_sms / p.halves, (p.total_rows + 1) / 2));
     MB_CUDA(launch_dependent(x3_conv<K, OUT>, (unsigned)(per_half * p.halves), C::kThreads, C::kSmem, st, p));

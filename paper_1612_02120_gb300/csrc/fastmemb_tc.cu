@@ -570,11 +570,8 @@ mb_status launch_fm_tc(const FmTcParams& p, cudaStream_t st) {
         MB_CUDA(cudaGetDevice(&dev));
         MB_CUDA(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    static bool attr = false;
-    if (!attr) {
-        MB_CUDA(cudaFuncSetAttribute(fm_tc_conv<HEAD, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem));
-        attr = true;
-    }
+    static std::atomic<uint64_t> smem_set{0};
+    MB_TRY(set_smem_once(smem_set, fm_tc_conv<HEAD, F16>, C::kSmem));
     // one range per resident CTA, or fewer when a range would get under 2 rows (each costs 4 more
     // staged rows: a launch this small is latency, not throughput)
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)n_sms * C::kCtas, (p.total_rows + 1) / 2));

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/membrane.h"
+#include "per_device.h"
 
 namespace mb {
 
@@ -80,6 +81,17 @@ bool fault_oom();
 
 mb_status dev_alloc(void** p, size_t bytes);
 void dev_free(void* p);
+
+// Lets `kernel` use `bytes` of dynamic shared memory on the current device.
+template <typename... K>
+mb_status set_smem_once(std::atomic<uint64_t>& done, void (*kernel)(K...), int bytes) {
+    int device = 0;
+    MB_CUDA(cudaGetDevice(&device));
+    return once_per_device(done, device, [&]() -> mb_status {
+        MB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        return MB_OK;
+    });
+}
 
 // A growable device scratch buffer owned by a net.
 struct Workspace {

@@ -613,12 +613,8 @@ mb_status launch_me_tc(const MeTcParams& q, cudaStream_t st) {
         MB_CUDA(cudaGetDevice(&dev));
         MB_CUDA(cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    static bool attr = false;
-    if (!attr) {
-        MB_CUDA(cudaFuncSetAttribute(me_tc_conv<KC, N, D, HEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     C::kSmem));
-        attr = true;
-    }
+    static std::atomic<uint64_t> smem_set{0};
+    MB_TRY(set_smem_once(smem_set, me_tc_conv<KC, N, D, HEAD>, C::kSmem));
     // one range per SM, or fewer when a range would get under 2 rows
     const int grid = std::max(1, std::min(n_sms, (q.total_rows + 1) / 2));
     MeTcParams p = q;

@@ -663,8 +663,9 @@ mb_status st_tc_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, int
         int dev = 0;
         MB_CUDA(cudaGetDevice(&dev));
         MB_CUDA(cudaDeviceGetAttribute(&S->n_sms, cudaDevAttrMultiProcessorCount, dev));
-        MB_CUDA(cudaFuncSetAttribute(st_tc_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, kSSmem));
     }
+    static std::atomic<uint64_t> smem_set{0};
+    MB_TRY(set_smem_once(smem_set, st_tc_infer, kSSmem));
     // the forward copy changes while the student trains: pack it on every call
     // (the inference launch sets itself up meanwhile: 64 x 64 17.2 -> 12.9 us, 1024 x 1024 27.4 -> 23.7)
     st_tc_pack<<<1, 1024, 0, st>>>(net->d_simt, S->d_wpack);

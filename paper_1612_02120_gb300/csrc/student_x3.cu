@@ -815,11 +815,8 @@ __global__ void __launch_bounds__(1024) st_reduce(const float* fwd, const float*
 
 template <int MODE>
 mb_status launch_sx(const SxParams& q, cudaStream_t st) {
-    static bool attr = false;
-    if (!attr) {
-        MB_CUDA(cudaFuncSetAttribute(st_x3<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemX));
-        attr = true;
-    }
+    static std::atomic<uint64_t> smem_set{0};
+    MB_TRY(set_smem_once(smem_set, st_x3<MODE>, kSmemX));
     constexpr bool BWD = MODE == SX_BWD;
     SxParams p = q;
     p.out_h = BWD ? p.H + 2 : p.H;
@@ -871,11 +868,8 @@ mb_status student_x3_grad(const StudentX3& a, cudaStream_t st) {
     p.inv_n = a.inv_n;
     p.partial = a.part_fwd;
     MB_TRY(launch_sx<SX_FWD>(p, st));
-    static bool attr = false;
-    if (!attr) {
-        MB_CUDA(cudaFuncSetAttribute(st_grad2, cudaFuncAttributeMaxDynamicSharedMemorySize, kG2Smem));
-        attr = true;
-    }
+    static std::atomic<uint64_t> smem_set{0};
+    MB_TRY(set_smem_once(smem_set, st_grad2, kG2Smem));
     MB_CUDA(launch_dependent(st_grad2, kX3GridG2, 288, kG2Smem, st, a.dy2, a.h1, a.B, a.H, a.W, a.part_g2, a.err));
     count_launch();
     p.in = a.dy2;

@@ -1005,12 +1005,8 @@ static bool ring_supported(bool fp8, int ring) {
 template <bool FP8, int RING, bool RNG>
 static mb_status launch_ring(TcParams& prm, int grid, cudaStream_t st) {
     using C = Cfg<FP8, RING>;
-    static bool attr = false;  // per instantiation
-    if (!attr) {
-        MB_CUDA(cudaFuncSetAttribute(tc_fused_teacher<FP8, RING, RNG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     C::kSmem));
-        attr = true;
-    }
+    static std::atomic<uint64_t> smem_set{0};
+    MB_TRY(set_smem_once(smem_set, tc_fused_teacher<FP8, RING, RNG>, C::kSmem));
     tc_fused_teacher<FP8, RING, RNG><<<grid, kThreads, C::kSmem, st>>>(prm);
     return MB_OK;
 }
