@@ -621,10 +621,17 @@ static mb_status batch_grad(mb_net* s, const uint8_t* in, const float* tgt, cons
     return MB_OK;
 }
 
-static mb_status pack_forward(mb_net* s, StudentBufs& b, cudaStream_t st) {
+// `first`: the launch that begins a call's chain, an ordinary one. The launches after it may begin early (one
+// begins when those before it have begun, however far they are), but none while an earlier call's still runs:
+// that one's output may be this call's slices or targets, which are read through the read-only path.
+static mb_status pack_forward(mb_net* s, StudentBufs& b, cudaStream_t st, bool first) {
     if (!b.x3) MB_CUDA(cudaMemsetAsync(b.zero, 0, 16 * sizeof(float), st));
-    MB_CUDA(launch_dependent(student_pack, (kSN + 255) / 256, 256, 0, st, s->d_params, s->d_simt, b.w2f,
-                             s->prec == MB_PREC_BF16, b.x3));
+    const unsigned grid = (kSN + 255) / 256;
+    const int bf16 = s->prec == MB_PREC_BF16;
+    if (first)
+        student_pack<<<grid, 256, 0, st>>>(s->d_params, s->d_simt, b.w2f, bf16, b.x3);
+    else
+        MB_CUDA(launch_dependent(student_pack, grid, 256, 0, st, s->d_params, s->d_simt, b.w2f, bf16, b.x3));
     count_launch();
     MB_CUDA(cudaGetLastError());
     return MB_OK;
@@ -636,7 +643,7 @@ mb_status student_loss_grad(mb_net* s, const uint8_t* in, const float* tgt, int6
     const bool x3 = train_bounded(s->host_params.data(), 0.0);
     MB_TRY(ensure_bufs(s, n, h, w, 1, x3, b));
     MB_TRY(train_error(s));
-    MB_TRY(pack_forward(s, b, st));
+    MB_TRY(pack_forward(s, b, st, true));
     if (x3) {  // straight into the caller's gradient; the loss through the mapped word
         b.grad = grad;
         MB_TRY(batch_grad(s, in, tgt, nullptr, n, h, w, b, reinterpret_cast<float*>(s->train_dev + 1), st));
@@ -747,7 +754,7 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
         const mb_status err = train_error(s);
         if (err == MB_OK) return MB_OK;
         MB_CUDA(cudaMemcpyAsync(s->d_params, s->host_params.data(), kSN * 4, cudaMemcpyHostToDevice, st));
-        MB_TRY(pack_forward(s, b, st));
+        MB_TRY(pack_forward(s, b, st, true));
         MB_CUDA(cudaStreamSynchronize(st));
         return err;
     };
@@ -775,7 +782,7 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
         MB_CUDA(cudaMemcpyAsync(b.zmap, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     for (int64_t k = 0; k < nsteps; ++k) {
         const int64_t step = start + k + 1;
-        MB_TRY(pack_forward(s, b, st));
+        MB_TRY(pack_forward(s, b, st, k == 0));
         MB_TRY(batch_grad(s, in, tgt, b.zmap + k * B, B, h, w, b, b.losses + k, st));
         const double c1 = 1.0 - std::pow((double)cfg->beta1, (double)step);
         const double c2 = 1.0 - std::pow((double)cfg->beta2, (double)step);
@@ -791,7 +798,7 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
             MB_TRY(write_ckpt(ckpt, hd, s->d_params, b.m, b.v, st));
         }
     }
-    MB_TRY(pack_forward(s, b, st));
+    MB_TRY(pack_forward(s, b, st, nsteps == 0));
     MB_TRY(trained());
     if (curve && nsteps > 0) MB_CUDA(cudaMemcpy(curve, b.losses, nsteps * sizeof(float), cudaMemcpyDeviceToHost));
     // the host master copy follows the device

@@ -25,6 +25,8 @@
 //   warps 4-11    epilogue, two groups of 8 channels, one pixel column per thread; sums over pixels
 //                 (loss, head, bias and conv1 weight gradients) stay in registers until the end
 //   warps 12-15   producers: load 8 channels of a pixel, split, store 3 x 16 B
+// Slices and targets are read through the read-only path: no launch of the chain writes them, and its first
+// launch (student_pack; st_conv1 for inference) is an ordinary one, so that what wrote them has ended.
 // The grids are fixed, so the partial sums, and with them a training run, are reproducible.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
