@@ -1273,11 +1273,13 @@ __global__ void fill_slices(uint8_t* p, int64_t n, int h, int w, uint32_t seed) 
     }
 }
 
+// The key names what the candidates were timed on: a choice made on other slices (white noise: keys without a
+// name) is not taken over.
 static std::string tune_key(int dev, mb_precision prec, int64_t z, int64_t h, int64_t w) {
     cudaDeviceProp pr;
     char buf[512];
     const char* name = cudaGetDeviceProperties(&pr, dev) == cudaSuccess ? pr.name : "unknown";
-    snprintf(buf, sizeof(buf), "%s|%s|%lldx%lldx%lld", name, prec == MB_PREC_FP8 ? "fp8" : "bf16", (long long)z,
+    snprintf(buf, sizeof(buf), "%s|%s|%lldx%lldx%lld|value noise", name, prec == MB_PREC_FP8 ? "fp8" : "bf16", (long long)z,
              (long long)h, (long long)w);
     for (char* c = buf; *c; ++c)
         if (*c == '"' || *c == '\\') *c = '_';
