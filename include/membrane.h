@@ -88,8 +88,8 @@ typedef enum {
  * so its slices need h, w >= 27) and FastMemb_3nm (Sec. 2.2, "A subsampling CNN for 3 nm data":
  * one more stage, conv4x4 32->32 G=2 d=8 and maxfilter d=8, then the head at d=16; radius 54,
  * slices h, w >= 55), both in FP32 (like the FP32 teacher: the 32-channel convolutions on the tensor
- * cores in three exact BF16 parts per value, error below an FP32 FMA chain's, where weights and
- * activations are bounded by 2^100, else on CUDA cores), BF16 and FP16 (the 16-bit nets: layer 1 on CUDA cores in
+ * cores in three exact BF16 parts per value, error below an FP32 FMA chain's, where no
+ * activation can pass 2^100 and no layer lies wholly below 2^-60, else on CUDA cores), BF16 and FP16 (the 16-bit nets: layer 1 on CUDA cores in
  * FP32 stored as 16-bit, the later convs and the head on the tensor cores with FP32 accumulation;
  * BF16 weights are split into two BF16 parts, FP16 weights are one FP16 value except the head's;
  * FP16 activations are finite below 65504); and MaskExtend (Sec. 3.2: conv4x4 12->32 G=2 d=1,
@@ -137,6 +137,9 @@ mb_status mb_net_param_count(const mb_net* net, int64_t* n_params);
 /* Copy FP32 parameters from HOST memory (caller keeps ownership). Layout: for each
  * parameterised layer in order, W[cout][cin][k][k] then b[cout]. BF16/FP8 nets round their
  * own copies from these. An FP8 net needs mb_calibrate_fp8 afterwards. Synchronous.
+ * Later calls use the new weights, the batch graphs that the library keeps included. So does a call
+ * that the caller captured in a CUDA graph before: a replay computes with the weights (and FP8
+ * scales) that are loaded then, by the kernels that were chosen when it was captured.
  * Errors: MB_ERR_INVALID_ARG when n_params differs from mb_net_param_count. */
 mb_status mb_load_weights(mb_net* net, const float* params, int64_t n_params);
 
@@ -198,9 +201,10 @@ mb_status mb_infer_region(mb_net* net, const uint8_t* in, int64_t z, int64_t h, 
 
 /*
  * A batch of independent blocks of uneven size (Sec. 2: blocks are segmented independently).
- * BF16/FP8 teacher nets: one persistent launch drains a device work queue of (block, slice,
- * strip) items; the first call for a new batch geometry captures the launch in a CUDA graph
- * that later calls with the same geometry replay. Other nets: one launch per block.
+ * BF16/FP8 teacher nets: one persistent launch for up to 64 blocks, its CTAs taking equal ranges of
+ * the batch's rows (or, tuned so, round-robin items); the first call for a list of blocks captures
+ * the launches in a CUDA graph that later calls with the same list (shapes, addresses, output type)
+ * replay, until weights, FP8 scales or the tuning change. Other nets: one launch per block.
  * Device pointers; asynchronous. Output of each block equals mb_infer_volume of that block.
  */
 mb_status mb_infer_batch(mb_net* net, const mb_block* blocks, int32_t n_blocks, mb_out_type out_type,
@@ -223,7 +227,8 @@ mb_status mb_infer_batch_per_block(mb_net* net, const mb_block* blocks, int32_t 
  * same MMAs for fewer columns. Every candidate gives bitwise the same maps.
  * Times every candidate on a synthetic h x w x z workload on `stream` (median of 4 launches after
  * one), keeps the fastest in the net and records it in the JSON cache at cache_path (HOST string,
- * may be NULL) keyed on GPU name, precision and shape; a cached entry is reused without timing.
+ * may be NULL) keyed on GPU name, precision, shape and the kind of slices timed; a cached entry with
+ * that key is reused without timing.
  * choice_out (HOST, may be NULL) receives {rows_per_item, stages, from_cache}. Synchronous.
  */
 mb_status mb_autotune(mb_net* net, int64_t z, int64_t h, int64_t w, const char* cache_path,
@@ -278,7 +283,9 @@ mb_status mb_student_loss_grad(mb_net* student, const uint8_t* in, const float* 
  * cfg->ckpt_every steps; with cfg->resume the run continues from it, bitwise as if never
  * interrupted. With cfg->resume and no file at ckpt_path the run starts fresh; a file there that
  * is not a complete format-2 checkpoint of this student returns MB_ERR_INVALID_ARG before any
- * step and leaves the file unchanged. Synchronous.
+ * step and leaves the file unchanged. MB_ERR_TIMEOUT (a device-side wait ran out): nothing of
+ * the failing steps is kept; the checkpoint file is the last one written before them, loss_curve is
+ * untouched and the net has its weights of before the call. Synchronous.
  */
 mb_status mb_student_train(mb_net* student, const uint8_t* in, const float* target, int64_t n, int64_t h,
                            int64_t w, const mb_train_cfg* cfg, const char* ckpt_path, float* loss_curve,

@@ -46,7 +46,9 @@ __device__ __forceinline__ float unit_of_byte(uint32_t u) {
 // launch): the kernel calls ptx::grid_dep_wait before it touches anything that an earlier launch
 // writes or reads, and the one before it calls ptx::grid_dep_launch where this one may set itself up.
 // What an earlier launch of the chain writes is read by ordinary loads (or bulk copies), not through the
-// read-only path: __ldg may be moved above the wait. A call's launches in a chain, against ordinary ones:
+// read-only path: __ldg may be moved above the wait. A call's first launch is an ordinary one, so that a
+// chain does not begin while what an earlier call writes (this one's inputs) is still being written.
+// A call's launches in a chain, against ordinary ones:
 // FastMemb BF16 on 64 x 64 55 -> 47 us, 1024 x 1024 283 -> 267, eight of them 1,839 -> 1,828; FP32
 // teacher 64 x 64 58 -> 52, 1024 x 1024 441 -> 430; a student gradient of 3 x 131 x 257 95 -> 91.
 // After a launch that does not call it, this is an ordinary one.
@@ -262,7 +264,6 @@ void simt_pack(const mb_net* net, const float* params, std::vector<float>& out);
 mb_status tc_prepare(mb_net* net);   // pack BF16 / FP8 weights from host_params (+ calibration)
 void tc_release(mb_net* net);
 mb_status tc_poll_error(mb_net* net);  // MB_ERR_TIMEOUT if a launch recorded a timed-out wait
-struct TcItem;                       // work item (device layout in tc_conv.cu)
 mb_status tc_infer_blocks(mb_net* net, const mb_block* blocks, int n_blocks, const int64_t* y0,
                           const int64_t* x0, const int64_t* rows, const int64_t* cols, mb_out_type ot,
                           cudaStream_t st, bool use_graph);

@@ -637,7 +637,6 @@ struct MeTcState {
     uint8_t* d_wpack[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     int* h_err = nullptr;
     int* d_err = nullptr;
-    int n_sms = 0;
 };
 
 }  // namespace
@@ -672,11 +671,6 @@ mb_status me_tc_prepare(mb_net* net) {
         MB_CUDA(cudaHostAlloc((void**)&S->h_err, sizeof(int), cudaHostAllocMapped));
         *S->h_err = 0;
         MB_CUDA(cudaHostGetDevicePointer((void**)&S->d_err, S->h_err, 0));
-    }
-    if (!S->n_sms) {
-        int dev = 0;
-        MB_CUDA(cudaGetDevice(&dev));
-        MB_CUDA(cudaDeviceGetAttribute(&S->n_sms, cudaDevAttrMultiProcessorCount, dev));
     }
     return MB_OK;
 }

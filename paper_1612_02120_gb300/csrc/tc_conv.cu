@@ -59,7 +59,7 @@ struct TcBlockDesc {
     int h, w;               // source slice size (mirror padding range)
     int ry0, rx0, rh, rw;   // output region
     int z, n_strips, n_chunks, item_start;
-    int64_t row_start;      // FP8 split: first strip-row of the block in (block, slice, strip, row) order
+    int64_t row_start;      // even split: first strip-row of the block in (block, slice, strip, row) order
 };
 
 // Constants, staged into shared memory at kernel start (floats):
@@ -72,7 +72,7 @@ struct TcParams {
     const uint8_t* wpack;   // global: packed B operands of layers 2 and 3, then the constants
     int* err;               // error word (MB_ERR_TIMEOUT on a timed-out wait)
     int n_blocks, n_items, rows_per_item, out_u8;
-    int64_t total_rows;     // FP8 split: strip-rows of the launch
+    int64_t total_rows;     // even split: strip-rows of the launch
     int fault_stall;        // test injection: the input loader withholds its arrivals
     uint64_t wait_ns;       // limit of every device-side wait
     float4 w1[25][8];       // layer 1: [tap][channel quad]
@@ -1015,8 +1015,8 @@ static mb_status launch_ring(TcParams& prm, int grid, cudaStream_t st) {
 // (strip of a slice) that it touches (1.65 us per row, 22 rows of 8 + 14 in 39 us). One CTA per SM
 // cuts columns anywhere, so that a range may touch two; where the launch has fewer columns than SMs,
 // the same number of CTAs for every column touches one each. The cheaper of the two. 256 x 256, one
-// slice, BF16: 12 CTAs of 64 rows 125 us, 152 cut anywhere 48 us, 3 x 50 36 us; 1024 x 1024: 136 us cut
-// anywhere, 127 us as 9 x 16.
+// slice, BF16: 12 CTAs of 64 rows 125 us, 152 cut anywhere 48 us, 3 x 50 36 us (30.7 since); 1024 x 1024:
+// 136 us cut anywhere, 127 us as 9 x 16.
 static int range_grid(const TcParams& prm) {
     const int64_t sms = g_num_sms;
     const int64_t any = std::max<int64_t>(1, std::min<int64_t>(sms, (prm.total_rows + 7) / 8));
