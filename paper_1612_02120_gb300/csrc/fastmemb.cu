@@ -191,8 +191,8 @@ mb_status simt_fastmemb_region(mb_net* net, const uint8_t* in, int64_t z, int64_
 // is one accumulator pair and a pixel's 16-byte chunks are stored whole. The weights are kernel
 // parameters, no shared-memory broadcasts beside the FMAs (those took 62 % of the shared-memory pipe
 // and left the FMA pipe at 50 %: 528 us). The inputs sit in shared memory duplicated, ready for packed
-// FMAs. Tap order and rounding are those of fm_conv, so the features are bitwise the same. 339 us on
-// 1024 x 1024 x 8 (FMA pipe 77 % busy, 16 warps of 118 registers); two columns a lane and 8 warps of 248
+// FMAs. Tap order and rounding are those of fm_conv, so the features are bitwise the same. 343 us on
+// 1024 x 1024 x 8 (FMA pipe 77 % busy, 16 warps of 128 registers); two columns a lane and 8 warps of 248
 // took 354 (the max-out, the filter and the stores of 2 warps a scheduler hide less behind FMAs), two
 // columns and half the channels a lane 869 (weights at a run-time offset); unpacked FMAs with the
 // filter left to the next layer's loads took 534.

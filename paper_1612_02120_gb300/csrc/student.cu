@@ -799,10 +799,14 @@ mb_status student_train(mb_net* s, const uint8_t* in, const float* tgt, int64_t 
         }
     }
     MB_TRY(pack_forward(s, b, st, nsteps == 0));
-    MB_TRY(trained());
-    if (curve && nsteps > 0) MB_CUDA(cudaMemcpy(curve, b.losses, nsteps * sizeof(float), cudaMemcpyDeviceToHost));
     // the host master copy follows the device
-    MB_CUDA(cudaMemcpy(s->host_params.data(), s->d_params, kSN * 4, cudaMemcpyDeviceToHost));
+    std::vector<float> losses(curve ? (size_t)nsteps : 0), master(kSN);
+    if (!losses.empty())
+        MB_CUDA(cudaMemcpyAsync(losses.data(), b.losses, losses.size() * 4, cudaMemcpyDeviceToHost, st));
+    MB_CUDA(cudaMemcpyAsync(master.data(), s->d_params, kSN * 4, cudaMemcpyDeviceToHost, st));
+    MB_TRY(trained());
+    std::copy(losses.begin(), losses.end(), curve);
+    s->host_params.swap(master);
     return MB_OK;
 }
 
