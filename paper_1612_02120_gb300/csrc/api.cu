@@ -335,8 +335,10 @@ static mb_status infer_host_volume(mb_net* net, const uint8_t* in, int64_t z, in
     slab = std::min<int64_t>(slab, z);
     if (z == 0) return MB_OK;
     constexpr int NB = 2;
-    // device slabs, streams and events live with the net and are reused by later calls
-    const size_t slab_bytes = (in_slice + out_slice) * (size_t)slab;
+    // device slabs, streams and events live with the net and are reused by later calls. Each part starts on
+    // a 256-byte boundary: the input's bytes (h x w x slices, any number) precede an output of floats.
+    auto part = [](size_t n) { return (n + 255) & ~(size_t)255; };
+    const size_t in_bytes = part(in_slice * (size_t)slab), slab_bytes = in_bytes + part(out_slice * (size_t)slab);
     MB_TRY(net->slab_ws.ensure(NB * slab_bytes));
     for (int i = 0; i < 4; ++i)
         if (!s[i]) MB_CUDA(cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking));
@@ -373,7 +375,7 @@ static mb_status infer_host_volume(mb_net* net, const uint8_t* in, int64_t z, in
         const int b = (int)(k % NB);
         const int64_t z0 = zb[(size_t)k], nz = zb[(size_t)k + 1] - z0;
         uint8_t* din = static_cast<uint8_t*>(net->slab_ws.ptr) + b * slab_bytes;
-        uint8_t* dout = din + in_slice * slab;
+        uint8_t* dout = din + in_bytes;
         cudaError_t e = cudaSuccess;
         if (k >= NB) e = cudaStreamWaitEvent(s[0], ev_comp[b], 0);  // input buffer free
         if (e == cudaSuccess) e = cudaMemcpyAsync(din, in + z0 * in_slice, in_slice * nz, cudaMemcpyHostToDevice, s[0]);
